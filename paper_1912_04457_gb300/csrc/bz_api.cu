@@ -807,8 +807,6 @@ static void fill_collide(bz_handle h, CollideArgs<R>& a, long long* A, int nsamp
     a.L64 = h->g.L;
     for (int d = 0; d < 3; ++d) a.dp64[d] = twoL / h->g.np[d];
     {
-        const int64_t nchunk = (nsamples + 31) / 32;
-        a.dv_group = div_magic((uint32_t)((nchunk + F32_GROUP - 1) / F32_GROUP));
         a.dv_slot = div_magic((uint32_t)std::min<int64_t>(h->nxc * h->npc, 0x7fffffff));
         a.dv_npc = div_magic((uint32_t)h->npc);
         a.dv_yz = div_magic((uint32_t)(h->g.np[1] * h->g.np[2]));
@@ -849,6 +847,17 @@ static void fill_collide(bz_handle h, CollideArgs<R>& a, long long* A, int nsamp
     std::memcpy(a.nterms, nterms, sizeof nterms);
 }
 
+// The work units of an FP32 argument block.
+static void set_split(CollideArgs<float>& a, const F32Split& f)
+{
+    a.a_stride = std::min<int64_t>(a.a_stride, 0x7fffffff);  // anchor indices are 32-bit there; a longer stride selects one
+    a.units = f.units;
+    a.upa = f.upa;
+    a.cpg = f.cpg;
+    a.gpa = f.gpa;
+    a.dv_group = div_magic((uint32_t)f.gpa);
+}
+
 static int run_collide(bz_handle h, long long* A, int nsamples, int step, double dt, int prec, int sampler,
                        cudaStream_t s, const int* step_dev = nullptr)
 {
@@ -865,24 +874,28 @@ static int run_collide(bz_handle h, long long* A, int nsamples, int step, double
         CK(h, launch_collide_f64(a, (int)blocks, s));
         return BZ_OK;
     }
-    // FP32 integrand, one warp per unit (an anchor and up to 256 of its samples);
+    // FP32 integrand, one warp per unit (f32_split);
     // ill-conditioned terms queued per warp for the float-float re-evaluation.
     // Cell indices are 32-bit there.
     if (h->ncell >= (int64_t)1 << 31)
         return fail(h, BZ_EINVAL, "the FP32 path needs fewer than 2^31 cells (has %lld)", (long long)h->ncell);
-    const int64_t units = f32_units(n_sel, nsamples);
-    if (units >= ((int64_t)1 << 31))
+    const int64_t old_units = f32_split(n_sel, nsamples, F32_RECORD_CHUNKS).units;
+    if (old_units >= ((int64_t)1 << 31))
         return fail(h, BZ_EINVAL, "anchors x samples too large for one FP32 call (%lld work units); use an anchor subset",
-                    (long long)units);
+                    (long long)old_units);
     CollideArgs<float> a{};
     fill_collide(h, a, A, nsamples, step, dt, sampler);
     a.step_dev = step_dev;
+    const int64_t resident = (int64_t)h->nsm * collide_f32_resident_blocks(a);
+    const int64_t items = n_sel * ((nsamples + 31) / 32);
+    const int chunks = f32_unit_chunks(items, resident * F32_WARPS);
+    set_split(a, f32_split(n_sel, nsamples, chunks));
+    const int64_t units = a.units;
     // a resident grid whose warps take one unit at a time from a counter; a
     // problem of at most two units per resident warp keeps one warp per unit
     // (no counter to reset, no atomics).  BZ_F32_SCHEDULE=counter|static
     // forces either form, so tests can check that they give the same bits.
     blocks = (units + F32_WARPS - 1) / F32_WARPS;
-    const int64_t resident = (int64_t)h->nsm * collide_f32_resident_blocks(a);
     bool dyn = blocks > 2 * resident;
     if (const char* sched = std::getenv("BZ_F32_SCHEDULE")) {
         if (!std::strcmp(sched, "counter")) dyn = true;
@@ -893,7 +906,7 @@ static int run_collide(bz_handle h, long long* A, int nsamples, int step, double
     if (dyn && !h->d_counter && cudaMalloc(&h->d_counter, sizeof(unsigned long long)) != cudaSuccess)
         return fail(h, BZ_ENOMEM, "cannot allocate the unit counter");
     const int64_t warps = blocks * F32_WARPS;
-    const int64_t samples_per_warp = ((units + warps - 1) / warps) * 32 * F32_GROUP;
+    const int64_t samples_per_warp = ((units + warps - 1) / warps) * 32 * ((int64_t)a.upa * a.cpg);
     const int64_t qcap = samples_per_warp * MAX_TERMS / DEFER_CAP_DIV + 64;
     if (warps > h->q_warps || warps * qcap > h->q_items) {
         cudaFree(h->d_qcount);
@@ -1347,6 +1360,7 @@ struct bz_batch_s {
     std::vector<bz_handle_s> hb;  // per-box descriptors; their device pointers alias the batch buffers
     std::vector<int64_t> cell_prefix, unit_prefix, mchunk_prefix, cchunk_prefix;
     std::vector<int> slot_prefix;
+    std::vector<F32Split> split;  // each box's work units
     int64_t ncell = 0, nunits = 0, nmchunks = 0, ncchunks = 0;
     int total_slots = 0;
     float* d_f = nullptr;
@@ -1433,6 +1447,7 @@ extern "C" int bz_batch_create(bz_batch* out, int32_t nboxes, const bz_box* boxe
     b->mchunk_prefix.assign(nboxes + 1, 0);
     b->cchunk_prefix.assign(nboxes + 1, 0);
     b->slot_prefix.assign(nboxes + 1, 0);
+    int64_t items = 0;  // chunks of 32 samples of all boxes
     for (int i = 0; i < nboxes; ++i) {
         const bz_box& d = boxes[i];
         for (int k = 0; k < 3; ++k)
@@ -1466,24 +1481,32 @@ extern "C" int bz_batch_create(bz_batch* out, int32_t nboxes, const bz_box* boxe
         h.ncell = h.nslots * h.npc;
         h.nsm = b->nsm;
         b->cell_prefix[i + 1] = b->cell_prefix[i] + h.ncell;
-        b->unit_prefix[i + 1] = b->unit_prefix[i] + f32_units(h.ncell, d.nsamples);
+        items += h.ncell * ((d.nsamples + 31) / 32);
         b->mchunk_prefix[i + 1] = b->mchunk_prefix[i] + (h.npc + 2047) / 2048;
         b->cchunk_prefix[i + 1] = b->cchunk_prefix[i] + (h.ncell + 2047) / 2048;
         b->slot_prefix[i + 1] = b->slot_prefix[i] + h.nslots;
+    }
+    const int chunks = f32_unit_chunks(items, (int64_t)b->nsm * 24);
+    int64_t old_units = 0;
+    b->split.resize(nboxes);
+    for (int i = 0; i < nboxes; ++i) {
+        old_units += f32_split(b->hb[i].ncell, boxes[i].nsamples, F32_RECORD_CHUNKS).units;
+        b->split[i] = f32_split(b->hb[i].ncell, boxes[i].nsamples, chunks);
+        b->unit_prefix[i + 1] = b->unit_prefix[i] + b->split[i].units;
     }
     b->ncell = b->cell_prefix[nboxes];
     b->nunits = b->unit_prefix[nboxes];
     b->nmchunks = b->mchunk_prefix[nboxes];
     b->ncchunks = b->cchunk_prefix[nboxes];
     b->total_slots = b->slot_prefix[nboxes];
-    if (b->ncell >= ((int64_t)1 << 31) || b->nunits >= ((int64_t)1 << 31)) {
+    if (b->ncell >= ((int64_t)1 << 31) || old_units >= ((int64_t)1 << 31)) {
         delete b;
         return bfail(nullptr, BZ_EINVAL, "the batch needs fewer than 2^31 cells and work units");
     }
     // persistent grid of up to 32 warps per SM; per-warp queue room for 4% of an
     // even share at 24 warps per SM (2.7% at 16, 5.3% at 32)
     b->qwarps = (int64_t)b->nsm * 32;
-    b->qcap = (b->nunits * 32 * F32_GROUP * MAX_TERMS) / ((int64_t)b->nsm * 24) / 25 + 64;
+    b->qcap = (items * 32 * MAX_TERMS) / ((int64_t)b->nsm * 24) / 25 + 64;
     bool ok = dalloc(&b->d_f, b->ncell) && dalloc(&b->d_m2_cur, 4 * nboxes) && dalloc(&b->d_m2_prev, 4 * nboxes) &&
               dalloc(&b->d_acc, 4 * nboxes) && dalloc(&b->d_flags, 4) && dalloc(&b->d_have_prev, 1) &&
               dalloc(&b->d_step, 1) && dalloc(&b->d_kidx, 1) && dalloc(&b->d_counter, 1) &&
@@ -1591,6 +1614,7 @@ static int batch_fill_args(bz_batch b, long long* state, double dt, cudaStream_t
         bz_handle_s* h = &b->hb[i];
         long long* st = state + b->cell_prefix[i];
         fill_collide(h, b->a32[i], st, b->desc[i].nsamples, 0, dt, BZ_SAMPLER_SYMMETRIC);
+        set_split(b->a32[i], b->split[i]);
         b->a32[i].tau = (float)DEFER_TAU;
         fill_masses(h, b->mass[i], st, b->d_acc + 4 * i, b->d_m2_cur + 4 * i,
                     h->mass_mode == BZ_MASS_MASSLESS ? nullptr : b->d_m2_prev + 4 * i);
@@ -1945,13 +1969,15 @@ extern "C" int bz_record(bz_handle h, const int64_t* state, int32_t nsamples, in
     unsigned long long* cnt = h->d_rec_count;
     CK(h, cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
     const int64_t n_sel = h->a_offset < h->ncell ? (h->ncell - h->a_offset + h->a_stride - 1) / h->a_stride : 0;
-    const int64_t units = f32_units(n_sel, nsamples);
+    const F32Split split = f32_split(n_sel, nsamples, F32_RECORD_CHUNKS);
+    const int64_t units = split.units;
     if (units >= ((int64_t)1 << 31)) return fail(h, BZ_EINVAL, "anchors x samples too large for one record call");
     int64_t blocks = (units + F32_WARPS - 1) / F32_WARPS;
     if (blocks > (int64_t)h->nsm * 48) blocks = (int64_t)h->nsm * 48;
     if (blocks < 1) blocks = 1;
     CollideArgs<float> a{};
     fill_collide(h, a, nullptr, nsamples, step, dt, BZ_SAMPLER_SYMMETRIC);
+    set_split(a, split);
     a.tau = 0.0f;
     a.rec = static_cast<ProposalRecord*>(records);
     a.rec_count = cnt;

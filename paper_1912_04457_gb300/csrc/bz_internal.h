@@ -139,7 +139,7 @@ struct CollideArgs {
     R L, twoL, dp[3];
     double L64, dp64[3];    // L and 2L/n in FP64 (the FP32 path's fixup works in FP64 geometry)
     // FP32 path index decode without hardware division (all indices < 2^31):
-    // units per anchor, cells per slot, p cells, np[1] np[2], np[2]
+    // units per anchor (gpa), cells per slot, p cells, np[1] np[2], np[2]
     DivMagic dv_group, dv_slot, dv_npc, dv_yz, dv_z;
     uint32_t key0, key1;
     uint32_t ks[20];        // Philox key schedule: (k0, k1) of rounds 0..9, so a kernel whose
@@ -147,6 +147,10 @@ struct CollideArgs {
     int nsamples, step;
     const int* step_dev;    // FP32 path: the step index in device memory (a replayed step graph), or null: step
     int64_t n_sel, a_stride, a_offset;
+    // FP32 path: the work units (f32_split): upa whole anchors each, or (upa = 1) cpg
+    // chunks of 32 samples of one anchor, gpa units per anchor
+    int64_t units;
+    int upa, cpg, gpa;
     int sampler, mass_mode, analytic, p_center;
     int param;              // FP64 path: 0 k2 eliminated (the paper's choice), 1 k3 eliminated
     const UserRow* urows;   // [MSQ_ROWS] device table of user-defined |M|^2 rows, or null
@@ -295,14 +299,36 @@ constexpr double DEFER_TAU = BZ_DEFER_TAU;  // FP32 terms with |H| < tau kappa^2
 #endif
 constexpr int DEFER_CAP_DIV = BZ_DEFER_CAP_DIV;  // queue room: 1/DIV of a warp's term evaluations
 constexpr int MAX_SAMPLES = 1 << 20;
-// FP32 collision kernel: warps per block, and 32-sample chunks per work unit
-// (an anchor and up to 256 of its samples; the live ones are compacted).
+// FP32 collision kernel: warps per block.
 constexpr int F32_WARPS = 4;
-constexpr int F32_GROUP = 8;
-__host__ __device__ inline int64_t f32_units(int64_t n_sel, int nsamples)
+// Work units of the FP32 collision kernel: `chunks` chunks of 32 samples each,
+// as whole anchors where an anchor has fewer, else as parts of one anchor.
+struct F32Split {
+    int64_t units;
+    int upa, cpg, gpa;
+};
+inline F32Split f32_split(int64_t n_sel, int nsamples, int chunks)
 {
-    const int64_t nchunk = (nsamples + 31) / 32;
-    return n_sel * ((nchunk + F32_GROUP - 1) / F32_GROUP);
+    const int nchunk = (nsamples + 31) / 32;
+    F32Split f;
+    f.upa = chunks / nchunk > 1 ? chunks / nchunk : 1;
+    f.cpg = f.upa > 1 ? nchunk : (chunks < nchunk ? chunks : nchunk);
+    f.gpa = f.upa > 1 ? 1 : (nchunk + f.cpg - 1) / f.cpg;
+    f.units = f.upa > 1 ? (n_sel + f.upa - 1) / f.upa : n_sel * f.gpa;
+    return f;
+}
+constexpr int F32_RECORD_CHUNKS = 8;  // record mode: a unit is an anchor and up to 256 of its samples
+// Chunks of a unit for a problem of `items` chunks on `warps` resident warps.  A
+// warp's last passes over a unit's samples and roots are short (on average
+// half empty), so units are long -- 32 chunks -- where there are many per
+// warp; up to 8 chunks a warp the whole share is one unit, so that a small
+// problem is one even wave.
+inline int f32_unit_chunks(int64_t items, int64_t warps)
+{
+    const int64_t share = (items + warps - 1) / (warps > 0 ? warps : 1);
+    if (share <= 8) return share < 1 ? 1 : (int)share;
+    const int64_t c = share / 8;
+    return (int)(c < 8 ? 8 : (c > 32 ? 32 : c));
 }
 int mlp_nparam();
 // ntot > 0: minibatch position r reads record splitmix64(key + r) mod ntot of rec

@@ -28,12 +28,21 @@
 
 namespace bz {
 
+// hi and lo words of the 32 x 32-bit product a b, as one wide multiplication
+__device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t& hi, uint32_t& lo)
+{
+    const unsigned long long p = (unsigned long long)a * b;
+    hi = (uint32_t)(p >> 32);
+    lo = (uint32_t)p;
+}
+
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1)
 {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
-        uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
+        uint32_t hi0, lo0, hi1, lo1;
+        mul_wide(0xD2511F53u, c.x, hi0, lo0);
+        mul_wide(0xCD9E8D57u, c.z, hi1, lo1);
         c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
         k0 += 0x9E3779B9u;
         k1 += 0xBB67AE85u;
@@ -46,8 +55,9 @@ __device__ __forceinline__ uint4 philox4x32_10_ks(uint4 c, const uint32_t* ks)
 {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
-        uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
+        uint32_t hi0, lo0, hi1, lo1;
+        mul_wide(0xD2511F53u, c.x, hi0, lo0);
+        mul_wide(0xCD9E8D57u, c.z, hi1, lo1);
         c = make_uint4(hi1 ^ c.y ^ ks[2 * r], lo1, hi0 ^ c.w ^ ks[2 * r + 1], lo0);
     }
     return c;
@@ -72,9 +82,10 @@ __device__ __forceinline__ uint4 philox_head(uint32_t cy, uint32_t cz, uint32_t 
 // Rounds 1 and 2 of counter c0 from the head, rounds 3..10 in full.
 __device__ __forceinline__ uint4 philox_tail_first2(uint32_t c0, uint4 h)
 {
-    const uint32_t hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
-    const uint32_t z1 = hi0 ^ h.x;
-    return make_uint4(__umulhi(0xCD9E8D57u, z1) ^ h.y, 0xCD9E8D57u * z1, h.z ^ lo0, h.w);
+    uint32_t hi0, lo0, hi1, lo1;
+    mul_wide(0xD2511F53u, c0, hi0, lo0);
+    mul_wide(0xCD9E8D57u, hi0 ^ h.x, hi1, lo1);
+    return make_uint4(hi1 ^ h.y, lo1, h.z ^ lo0, h.w);
 }
 
 // The key words of every round from a schedule (philox_key_schedule).
@@ -83,8 +94,9 @@ __device__ __forceinline__ uint4 philox_tail_ks(uint32_t c0, uint4 h, const uint
     uint4 c = philox_tail_first2(c0, h);
 #pragma unroll
     for (int r = 2; r < 10; ++r) {
-        uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
-        uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
+        uint32_t hi0, lo0, hi1, lo1;
+        mul_wide(0xD2511F53u, c.x, hi0, lo0);
+        mul_wide(0xCD9E8D57u, c.z, hi1, lo1);
         c = make_uint4(hi1 ^ c.y ^ ks[2 * r], lo1, hi0 ^ c.w ^ ks[2 * r + 1], lo0);
     }
     return c;
@@ -98,8 +110,9 @@ __device__ __forceinline__ uint4 philox_tail(uint32_t c0, uint4 h, uint32_t k0, 
     k1 += 2u * 0xBB67AE85u;
 #pragma unroll
     for (int r = 2; r < 10; ++r) {
-        uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
-        uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
+        uint32_t hi0, lo0, hi1, lo1;
+        mul_wide(0xD2511F53u, c.x, hi0, lo0);
+        mul_wide(0xCD9E8D57u, c.z, hi1, lo1);
         c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
         k0 += 0x9E3779B9u;
         k1 += 0xBB67AE85u;
@@ -153,6 +166,16 @@ __device__ __forceinline__ R upow(R x, int n)
     return r;
 }
 
+// a / b: FP64 as written; FP32 by the hardware reciprocal (the arguments are
+// far from its range limits), without the scaling of the approximate division.
+__device__ __forceinline__ double div_approx(double a, double b) { return a / b; }
+__device__ __forceinline__ float div_approx(float a, float b)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+    return a * r;
+}
+
 template <typename R>
 __device__ __forceinline__ R msq_user(const UserRow* row, R s, R t, R u, R mg2)
 {
@@ -176,21 +199,21 @@ __device__ __forceinline__ R msq(int cls, const CollideArgs<R>& P, R s, R t, R u
     R tm = t - mg2, um = u - mg2;
     switch (cls) {
     case M_QQP:
-        return P.A1 * ((s * s + u * u) / (tm * tm));
+        return P.A1 * div_approx(s * s + u * u, tm * tm);
     case M_QQ:
-        return P.A1 * ((s * s + u * u) / (tm * tm) + (s * s + t * t) / (um * um))
-               + P.A2 * ((s * s) / (tm * um));
+        return P.A1 * (div_approx(s * s + u * u, tm * tm) + div_approx(s * s + t * t, um * um))
+               + P.A2 * div_approx(s * s, tm * um);
     case M_QQB:
-        return P.A1 * ((s * s + u * u) / (tm * tm) + (u * u + t * t) / (s * s))
-               + P.A2 * ((u * u) / (tm * s));
+        return P.A1 * (div_approx(s * s + u * u, tm * tm) + div_approx(u * u + t * t, s * s))
+               + P.A2 * div_approx(u * u, tm * s);
     case M_QQB2:
-        return P.A1 * ((t * t + u * u) / (s * s));
+        return P.A1 * div_approx(t * t + u * u, s * s);
     case M_QQBGG:
-        return P.A3 * (u / tm + t / um) - P.A4 * ((t * t + u * u) / (s * s));
+        return P.A3 * (div_approx(u, tm) + div_approx(t, um)) - P.A4 * div_approx(t * t + u * u, s * s);
     case M_QG:
-        return P.A4 * ((s * s + u * u) / (tm * tm)) - P.A3 * (u / s + s / um);
+        return P.A4 * div_approx(s * s + u * u, tm * tm) - P.A3 * (div_approx(u, s) + div_approx(s, um));
     default:  // M_GG
-        return P.A5 * (R(3) - (s * u) / (tm * tm) - (s * t) / (um * um) - (t * u) / (s * s));
+        return P.A5 * (R(3) - div_approx(s * u, tm * tm) - div_approx(s * t, um * um) - div_approx(t * u, s * s));
     }
 }
 
@@ -316,9 +339,8 @@ __device__ __forceinline__ void make_geom(const CollideArgs<R>& P, int64_t a, in
 
 // Per-warp queue of deferred (anchor, sample, term) items (FP32 path).
 struct DeferCtx {
-    int* s_count;          // this warp's counter in shared memory
     unsigned long long* seg;
-    int cap;
+    int count, cap;        // items queued (at most cap); the same in every lane
 };
 
 // Evaluates term ti of sample (a, smp); deposits the k1, k2, k3 legs and

@@ -1,0 +1,52 @@
+"""FP32 collision: work units that run over several anchors and rows, parts of
+one anchor, anchor subsets, and momentum axes on both sides of 128 cells (the
+32-bit position of k2), against the oracle on the same 23-bit uniforms (the
+FP32 bar, 2e-5 relative L2), sum A = 0, the same bits from both schedules."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1912_04457_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # nx, np, mask, N, stride, offset
+    ((1, 1, 1), (256, 2, 4), 0x01, 64, 1, 0),      # the longest axis
+    ((1, 1, 1), (130, 129, 2), 0x03, 8, 1, 0),     # just above 128
+    ((1, 1, 1), (128, 127, 2), 0x01, 8, 1, 0),     # and at it
+    ((3, 2, 4), (4, 3, 2), 0x01, 33, 1, 0),        # rows shorter than a unit's anchors
+    ((2, 1, 2), (6, 5, 4), 0x13, 1, 1, 0),         # one sample per anchor
+    ((2, 2, 1), (6, 4, 8), 0x17, 100, 7, 3),       # a subset that skips over row ends
+    ((1, 1, 1), (4, 4, 4), 0x02, 1100, 1, 0),      # an anchor in several units (N > 1024)
+    ((1, 1, 1), (4, 4, 4), 0x01, 64, 1 << 33, 5),  # one anchor of a stride beyond 32 bits
+]
+
+
+@pytest.mark.parametrize("nx,np_,mask,N,stride,offset", CASES)
+def test_units(nx, np_, mask, N, stride, offset):
+    import torch
+    from paper_1912_04457_gb300 import bz
+    nxc = int(np.prod(nx))
+    h = bz.Handle(nx=nx, dx=0.2, np_=np_, L=2.0, seed=6, species_mask=mask)
+    cfg = O.make_config(nx=nx, dx=0.2, np_=np_, L=2.0, seed=6, species_mask=mask)
+    h.set_anchor_subset(stride, offset)
+    st = I.encode(I.random_f(np_, bin(mask).count("1"), nxc, 14, 0.05, 0.5), mask)
+    dev = torch.from_numpy(st.reshape(-1)).cuda()
+    A, B = torch.empty_like(dev), torch.empty_like(dev)
+    h.collision_term(dev, A, N, 2, 0.01, bz.PREC_F32)
+    ref = O.collision(cfg, st, O.masses(cfg, st), N, step=2, dt=0.01, ubits=23, anchor_stride=stride,
+                      anchor_offset=offset)["A"].reshape(-1).astype(float)
+    got = A.cpu().numpy()
+    assert int(got.sum()) == 0 and np.count_nonzero(got) > 0
+    assert np.linalg.norm(got - ref) <= 2e-5 * np.linalg.norm(ref)
+    try:
+        for sched in ("counter", "static"):
+            os.environ["BZ_F32_SCHEDULE"] = sched
+            h.reset_masses()
+            h.collision_term(dev, B, N, 2, 0.01, bz.PREC_F32)
+            assert torch.equal(A, B), sched
+    finally:
+        del os.environ["BZ_F32_SCHEDULE"]
