@@ -862,16 +862,11 @@ static int run_collide(bz_handle h, long long* A, int nsamples, int step, double
                        cudaStream_t s, const int* step_dev = nullptr)
 {
     const int64_t n_sel = h->a_offset < h->ncell ? (h->ncell - h->a_offset + h->a_stride - 1) / h->a_stride : 0;
-    const int64_t total = n_sel * (int64_t)nsamples;
-    int64_t blocks = (total + 255) / 256;
-    int64_t cap = (int64_t)h->nsm * 8;
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
     if (prec == BZ_PREC_F64) {
         CollideArgs<double> a{};
         fill_collide(h, a, A, nsamples, step, dt, sampler);
         ProfScope ps(h, BZ_K_COLLIDE, s);
-        CK(h, launch_collide_f64(a, (int)blocks, s));
+        CK(h, launch_collide_f64(a, h->nsm, s));
         return BZ_OK;
     }
     // FP32 integrand, one warp per unit (f32_split);
@@ -895,7 +890,7 @@ static int run_collide(bz_handle h, long long* A, int nsamples, int step, double
     // problem of at most two units per resident warp keeps one warp per unit
     // (no counter to reset, no atomics).  BZ_F32_SCHEDULE=counter|static
     // forces either form, so tests can check that they give the same bits.
-    blocks = (units + F32_WARPS - 1) / F32_WARPS;
+    int64_t blocks = (units + F32_WARPS - 1) / F32_WARPS;
     bool dyn = blocks > 2 * resident;
     if (const char* sched = std::getenv("BZ_F32_SCHEDULE")) {
         if (!std::strcmp(sched, "counter")) dyn = true;

@@ -261,7 +261,7 @@ struct ConvScale {
 };
 
 // launchers (return cudaGetLastError())
-cudaError_t launch_collide_f64(const CollideArgs<double>& a, int grid, cudaStream_t s);
+cudaError_t launch_collide_f64(const CollideArgs<double>& a, int nsm, cudaStream_t s);
 cudaError_t launch_fill_jtab(int* jtab, const int* np, cudaStream_t s);
 // exact int64 sum of a[0, n) added into *out
 cudaError_t launch_sum_ll(const long long* a, int64_t n, long long* out, cudaStream_t s);

@@ -259,10 +259,6 @@ extern "C" int bz_collision_term_static(const bz_grid* g, uint32_t species_mask,
     a.A5 = 16.0 * g4 * dA * CA * CA;
     for (int q = 0; q < NSPEC; ++q) a.slot_species[q] = slot_species[q];
     terms_of(species_mask, slot_of, a.terms, a.nterms);
-    const int64_t total = ncell * (int64_t)nsamples;
-    int64_t blocks = (total + 255) / 256;
-    if (blocks > (int64_t)sc->nsm * 8) blocks = (int64_t)sc->nsm * 8;
-    if (blocks < 1) blocks = 1;
-    CKS(launch_collide_f64(a, (int)blocks, s));
+    CKS(launch_collide_f64(a, sc->nsm, s));
     return BZ_OK;
 }

@@ -1,0 +1,42 @@
+"""FP64 collision: the warp-cooperative kernel (FP32 classification of the k1z
+roots, integer bins) against the oracle, bit for bit: axes at and around 128 and 256
+cells, rows shorter than a unit's anchors, subsets, one sample per anchor, an
+anchor in several units, both uniform resolutions, scales of L far from 1."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1912_04457_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # nx, np, L, mask, mass mode, N, sampler, uniform bits, stride, offset
+    ((1, 1, 1), (256, 2, 4), 2.0, 0x01, 0, 64, 0, 32, 1, 0),
+    ((1, 1, 1), (130, 129, 2), 2.0, 0x03, 0, 8, 0, 23, 1, 0),
+    ((3, 2, 4), (4, 3, 2), 2.0, 0x01, 0, 33, 0, 32, 1, 0),
+    ((2, 1, 2), (6, 5, 4), 2.0, 0x13, 0, 1, 0, 32, 1, 0),
+    ((2, 2, 1), (6, 4, 8), 2.0, 0x17, 0, 100, 1, 32, 7, 3),
+    ((1, 1, 1), (4, 4, 4), 2.0, 0x02, 0, 1100, 0, 23, 1, 0),
+    ((1, 1, 1), (6, 6, 6), 1e-3, 0x7F, 1, 48, 0, 32, 1, 0),
+    ((1, 1, 1), (6, 6, 6), 5e3, 0x7F, 0, 48, 0, 32, 1, 0),
+    ((1, 1, 1), (4, 4, 4), 2.0, 0x01, 0, 64, 0, 32, 1 << 33, 5),
+]
+
+
+@pytest.mark.parametrize("nx,np_,L,mask,mode,N,sampler,bits,stride,offset", CASES)
+def test_bits(nx, np_, L, mask, mode, N, sampler, bits, stride, offset):
+    import torch
+    from paper_1912_04457_gb300 import bz
+    h = bz.Handle(nx=nx, dx=0.2, np_=np_, L=L, seed=8, species_mask=mask, mass_mode=mode)
+    cfg = O.make_config(nx=nx, dx=0.2, np_=np_, L=L, seed=8, species_mask=mask, mass_mode=mode)
+    h.set_uniform_bits(bits)
+    h.set_anchor_subset(stride, offset)
+    st = I.encode(I.random_f(np_, bin(mask).count("1"), int(np.prod(nx)), 15, 0.0, 0.6), mask)
+    A = torch.empty(st.size, dtype=torch.int64, device="cuda")
+    h.collision_term(torch.from_numpy(st.reshape(-1)).cuda(), A, N, 2, 0.01, bz.PREC_F64, sampler)
+    ref = O.collision(cfg, st, O.masses(cfg, st), N, step=2, dt=0.01, sampler=sampler, ubits=bits, anchor_stride=stride,
+                      anchor_offset=offset)
+    got = A.cpu().numpy()
+    assert np.array_equal(got, ref["A"].reshape(-1)) and np.count_nonzero(got) > 0
+    assert np.array_equal(h.flags()[:2], ref["flags"])
