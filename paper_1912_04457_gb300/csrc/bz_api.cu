@@ -989,10 +989,10 @@ static int fill_moments(bz_handle h, MomentArgs& a, const long long* state, doub
         a.half_dp[d] = 0.5 * dp[d];
         for (int j = 0; j < h->g.np[d]; ++j) a.pf[d][j] = (float)(-h->g.L + ((double)j + 0.5) * dp[d]);
     }
+    momentum_octets(a);
     for (int sl = 0; sl < NSPEC; ++sl) a.slot_mslot[sl] = mass_slot(sl < h->nslots ? h->slot_species[sl] : 0);
     double twopi = 2.0 * PI;
     a.pref = dp[0] * dp[1] * dp[2] / (twopi * twopi * twopi) * TWO_POW_M40;
-    a.jtab = h->d_jtab;  // null for the boxes of a batch
     a.sflags = h->d_sflags;
     for (int sl = 0; sl < NSPEC; ++sl) {
         const int sp = sl < h->nslots ? h->slot_species[sl] : 0;

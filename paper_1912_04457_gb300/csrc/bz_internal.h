@@ -179,6 +179,24 @@ struct CollideArgs {
     long long qcap;
 };
 
+// Octets of momentum cells (j or n-1-j along each axis): half[d] = ceil(n_d / 2)
+// per axis, octet o = (h0 half[1] + h1) half[2] + h2.  False (no octets) unless
+// every axis' FP32 centres are exact mirror images.
+template <typename Args>
+inline bool momentum_octets(Args& a)
+{
+    a.noct = 0;
+    for (int d = 0; d < 3; ++d) {
+        for (int j = 0; j < a.np[d]; ++j)
+            if (a.pf[d][j] != -a.pf[d][a.np[d] - 1 - j]) return false;
+        a.half[d] = (a.np[d] + 1) / 2;
+    }
+    a.dv_h12 = div_magic((uint32_t)(a.half[1] * a.half[2]));
+    a.dv_h2 = div_magic((uint32_t)a.half[2]);
+    a.noct = a.half[0] * a.half[1] * a.half[2];
+    return true;
+}
+
 struct MassArgs {
     const long long* state;
     long long* acc;         // [x][4] fixed-point sums (zeroed by the caller)
@@ -238,7 +256,6 @@ struct MomentArgs {
     int slot_mslot[NSPEC];
     double pref, half_dp[3];
     float pf[3][MAX_NP];
-    const int* jtab;        // [npc] jx | jy << 8 | jz << 16, or null (decoded by division)
     long long* sflags;      // [2] cells with n < 0, fermion cells with f > 1 (added), or null
     long long pauli[NSPEC]; // per slot: N_s 2^40 (f = 1) for (anti)quarks, LLONG_MAX for gluons
     // energy source (k_energy_source): out is [x][slot][3], masses of the previous evaluation, dt
@@ -248,6 +265,10 @@ struct MomentArgs {
     // ([x][slot][chunk][5] 128-bit as (lo, hi) int64 pairs) when nchunk > 1
     int nchunk;
     long long* part;
+    // grids whose FP32 cell centres are mirror images, pf[n-1-j] = -pf[j]: octets of mirrored cells
+    // (momentum_octets), noct = 0 otherwise
+    int noct, half[3];
+    DivMagic dv_h12, dv_h2;
     // a replayed step graph writes the moments of step *kidx at out + *kidx kstride (kidx null: out)
     const int* kidx;
     int64_t kstride;

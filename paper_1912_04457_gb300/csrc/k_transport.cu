@@ -936,12 +936,63 @@ __device__ __forceinline__ double i128_to_double(__int128 v)
     return (double)(long long)(v >> 64) * 18446744073709551616.0 + (double)(unsigned long long)v;
 }
 
-#ifndef BZ_MOM_UNROLL
-#define BZ_MOM_UNROLL 2  // cells in flight per thread
-#endif
-#ifndef BZ_MOM_MINB
-#define BZ_MOM_MINB 4    // resident blocks per SM (register budget)
-#endif
+constexpr int MOM_THREADS = 128;  // per (x cell, slot) or chunk of one
+
+// Octets of mirrored cells.  The 8 cells (+-p_x, +-p_y, +-p_z) share E and, up to
+// its sign, every momentum component, so that a sum over the octet and three
+// differences (18 64-bit additions) leave one multiplication per moment instead
+// of one per cell: 12 instructions a cell instead of 150, which leaves the loads
+// the bound (16^3 x 20^3 box: moments 187 -> 68 us, energy source 134 -> 52 us, 262 MB
+// read; 7 blocks per SM, 72 registers: more bytes in flight than with 94).
+// The eight n as loaded, lower cells first: bit d of the index is set for the
+// upper cell of axis d; a cell on the mirror plane of an odd axis counts as its
+// lower cell only (its momentum component there is 0).
+struct Octet {
+    long long n[8];
+    int h[3];
+    unsigned hi;  // the high words, or-ed
+};
+template <typename Args>
+__device__ __forceinline__ void octet_index(const Args& P, int o, int h[3])
+{
+    h[0] = (int)udiv((uint32_t)o, P.dv_h12);
+    const int r = o - h[0] * (P.half[1] * P.half[2]);
+    h[1] = (int)udiv((uint32_t)r, P.dv_h2);
+    h[2] = r - h[1] * P.half[2];
+}
+__device__ __forceinline__ void load_octet(const MomentArgs& P, const long long* st, int o, Octet& q)
+{
+    octet_index(P, o, q.h);
+    const int u0 = P.np[0] - 1 - q.h[0], u1 = P.np[1] - 1 - q.h[1], u2 = P.np[2] - 1 - q.h[2];
+    const int j[4] = {(q.h[0] * P.np[1] + q.h[1]) * P.np[2], (u0 * P.np[1] + q.h[1]) * P.np[2],
+                      (q.h[0] * P.np[1] + u1) * P.np[2], (u0 * P.np[1] + u1) * P.np[2]};
+    const bool d0 = u0 != q.h[0], d1 = u1 != q.h[1], d2 = u2 != q.h[2];
+    const bool live[4] = {true, d0, d1, d0 && d1};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        q.n[i] = live[i] ? __ldg(st + j[i] + q.h[2]) : 0;
+        q.n[4 + i] = live[i] & d2 ? __ldg(st + j[i] + u2) : 0;
+    }
+    unsigned o4[2] = {0u, 0u};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        o4[0] |= (unsigned)(q.n[i] >> 32);
+        o4[1] |= (unsigned)(q.n[4 + i] >> 32);
+    }
+    q.hi = o4[0] | o4[1];
+}
+// every |n| < 2^58, so that the sums of eight stay far inside 64 bits
+__device__ __forceinline__ bool octet_narrow(const Octet& q)
+{
+    unsigned t = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) t |= (unsigned)(q.n[i] >> 32) ^ (unsigned)(q.n[i] >> 63);
+    return t < (1u << 26);
+}
+__device__ __forceinline__ long long octet_sum(const Octet& q)
+{
+    return ((q.n[0] + q.n[1]) + (q.n[2] + q.n[3])) + ((q.n[4] + q.n[5]) + (q.n[6] + q.n[7]));
+}
 
 // The 5 doubles of one (x cell, slot) from its exact sums.
 __device__ __forceinline__ void moments_out(const MomentArgs& P, const __int128* t, double* o)
@@ -951,10 +1002,60 @@ __device__ __forceinline__ void moments_out(const MomentArgs& P, const __int128*
     for (int d = 0; d < 3; ++d) o[2 + d] = i128_to_double(t[2 + d]) * P.pref * P.half_dp[d];
 }
 
-// Exact sums of the cells [jlo, jhi) of one (x cell, slot): 5 doubles at o,
-// or, with part set, the 5 exact 128-bit sums (lo, hi words) at part.
-__device__ __forceinline__ void moments_block(const MomentArgs& P, int64_t x, int sl, int jlo, int jhi, double* o,
-                                              long long* part)
+// Per-thread exact sums of the moments.  n = nh 2^32 + nl (nl unsigned): every
+// product below is 32 x 32 bits and every partial sum is exact, for at most 2^17
+// cells or octets per thread (npc <= 2^24, 128 threads): sum nl < 2^49, sum k nl
+// < 2^57 and sum k nh < 2^56 in size with 0 <= |k| < 2^8.  E_fx n is accumulated
+// in 128 bits (lo word and carries).
+struct MomSums {
+    unsigned long long s_nl = 0;
+    long long s_nh = 0;
+    unsigned long long el_lo = 0, el_hi = 0;  // sum E_fx nl (unsigned, 128 bits)
+    unsigned long long eh_lo = 0;             // sum E_fx nh (signed, 128 bits: lo word ...
+    long long eh_hi = 0;                      // ... and high word)
+    long long kl[3] = {0, 0, 0};              // sum k_d nl
+    long long kh[3] = {0, 0, 0};              // sum k_d nh
+    __int128 e_wide = 0;                      // sum E_fx n where E_fx >= 2^31 (exact, rare)
+    __device__ __forceinline__ void add_n(long long n)
+    {
+        s_nl += (unsigned)n;
+        s_nh += n >> 32;
+    }
+    __device__ __forceinline__ void add_e(float ew, long long n)  // ew = E 2^24, rounded half even
+    {
+        if (ew < 2147483648.0f) {  // E_fx < 2^31 (ew is >= 0 or NaN)
+            const unsigned Efx = (unsigned)__float2int_rn(ew);
+            const unsigned long long tl = (unsigned long long)Efx * (unsigned)n;
+            el_lo += tl;
+            el_hi += el_lo < tl;
+            const long long th = (long long)(int)Efx * (int)(n >> 32);
+            const unsigned long long o = eh_lo;
+            eh_lo += (unsigned long long)th;
+            eh_hi += (th >> 63) + (eh_lo < o);
+        } else {
+            e_wide += (__int128)rint_ll(ew) * n;
+        }
+    }
+    __device__ __forceinline__ void add_k(int d, int k, long long n)
+    {
+        kl[d] += (long long)((unsigned long long)(unsigned)(k < 0 ? -k : k) * (unsigned)n) * (k < 0 ? -1 : 1);
+        kh[d] += (long long)k * (int)(n >> 32);
+    }
+    __device__ __forceinline__ void add_k_pos(int d, unsigned k, long long n)  // k >= 0
+    {
+        kl[d] += (long long)((unsigned long long)k * (unsigned)n);
+        kh[d] += (long long)(int)k * (int)(n >> 32);
+    }
+    __device__ __forceinline__ __int128 energy() const
+    {
+        const __int128 eh = (__int128)(((unsigned __int128)(unsigned long long)eh_hi << 64) | eh_lo);
+        return (__int128)(((unsigned __int128)el_hi << 64) | el_lo) + eh * ((__int128)1 << 32) + e_wide;
+    }
+};
+
+// Exact sums of chunk c of nch of one (x cell, slot): 5 doubles at o, or, with
+// part set, the 5 exact 128-bit sums (lo, hi words) at part.
+__device__ __forceinline__ void moments_block(const MomentArgs& P, int64_t x, int sl, int c, int nch, double* o, long long* part)
 {
     __shared__ float s_pf[3][MAX_NP];  // cell-centre momenta (lanes index them at different cells)
     for (int d = 0; d < 3; ++d)
@@ -962,83 +1063,72 @@ __device__ __forceinline__ void moments_block(const MomentArgs& P, int64_t x, in
     __syncthreads();
     const float m = P.mass_mode == 1 ? 0.0f : (float)P.m2[x * 4 + P.slot_mslot[sl]];
     const long long* st = P.state + ((int64_t)sl * P.nxc + x) * P.npc;
-    const int np1 = P.np[1], np2 = P.np[2];
     const long long pauli = P.pauli[sl];
     int neg = 0, over = 0;  // state warnings: f < 0 anywhere, f > 1 for fermions (Pauli)
-    // n = nh 2^32 + nl (nl unsigned): every product below is 32 x 32 bits and
-    // every partial sum is exact, for at most 2^16 cells per thread
-    // (npc <= 2^24, 256 threads): sum nl < 2^48, sum (k_d + 256) nl < 2^57,
-    // sum k_d nh < 2^55 with |k_d| = |2 j_d + 1 - n_d| < 2^8.  E_fx n is
-    // accumulated in 128 bits (lo word and carries).
-    unsigned long long s_nl = 0;
-    long long s_nh = 0;
-    unsigned long long el_lo = 0, el_hi = 0;  // sum E_fx nl (unsigned, 128 bits)
-    unsigned long long eh_lo = 0;             // sum E_fx nh (signed, 128 bits: lo word ...
-    long long eh_hi = 0;                      // ... and high word)
-    unsigned long long kl[3] = {0, 0, 0};     // sum (k_d + 256) nl
-    long long kh[3] = {0, 0, 0};              // sum k_d nh
-    __int128 e_wide = 0;                      // sum E_fx n of cells with E_fx >= 2^31 (exact, rare)
-    constexpr int U = BZ_MOM_UNROLL;          // cells in flight per thread
-    for (int j0 = jlo + (int)threadIdx.x; j0 < jhi; j0 += U * (int)blockDim.x) {
-        long long nv[U];
-        int jpv[U];
+    MomSums M;
+    auto cell = [&](int j0, int j1, int j2, long long n) {
+        const float pf0 = s_pf[0][j0], pf1 = s_pf[1][j1], pf2 = s_pf[2][j2];
+        M.add_n(n);
+        M.add_e(sqrtf((pf0 * pf0 + pf1 * pf1) + pf2 * pf2 + m) * 16777216.0f, n);
+        M.add_k(0, 2 * j0 + 1 - P.np[0], n);
+        M.add_k(1, 2 * j1 + 1 - P.np[1], n);
+        M.add_k(2, 2 * j2 + 1 - P.np[2], n);
+    };
+    const int items = P.noct ? P.noct : (int)P.npc;
+    const int lo = (int)((int64_t)c * items / nch), hi = (int)((int64_t)(c + 1) * items / nch);
+    if (P.noct) {
+        // high words or-ed below this: no n is negative, none of a fermion above its limit
+        // (4 2^40 < N_s 2^40 = f of 1), and every n is below 2^58
+        const unsigned plain = pauli == 0x7fffffffffffffffLL ? 1u << 26 : 1024u;
+        for (int i = lo + (int)threadIdx.x; i < hi; i += MOM_THREADS) {
+            Octet q;
+            load_octet(P, st, i, q);
+            if (q.hi >= plain) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int j = j0 + u * (int)blockDim.x;
-            nv[u] = j < jhi ? __ldg(&st[j]) : 0;
-            if (P.jtab) {
-                jpv[u] = j < jhi ? __ldg(P.jtab + j) : 0;
-            } else {
-                const int jj = j < jhi ? j : 0, jxy = jj / np2;
-                jpv[u] = (jxy / np1) | ((jxy % np1) << 8) | ((jj % np2) << 16);
+                for (int k = 0; k < 8; ++k) {
+                    neg += q.n[k] < 0;
+                    over += q.n[k] > pauli;
+                }
+                if (!octet_narrow(q)) {
+                    for (int k = 0; k < 8; ++k) {  // absent cells have n = 0
+                        if (q.n[k] == 0) continue;
+                        const int j0 = k & 1 ? P.np[0] - 1 - q.h[0] : q.h[0], j1 = k & 2 ? P.np[1] - 1 - q.h[1] : q.h[1];
+                        cell(j0, j1, k & 4 ? P.np[2] - 1 - q.h[2] : q.h[2], q.n[k]);
+                    }
+                    continue;
+                }
             }
+            const float pf0 = s_pf[0][q.h[0]], pf1 = s_pf[1][q.h[1]], pf2 = s_pf[2][q.h[2]];
+            const float ew = sqrtf((pf0 * pf0 + pf1 * pf1) + pf2 * pf2 + m) * 16777216.0f;
+            const long long z0 = q.n[0] + q.n[4], z1 = q.n[1] + q.n[5], z2 = q.n[2] + q.n[6], z3 = q.n[3] + q.n[7];
+            const long long y0 = z0 + z2, y1 = z1 + z3;
+            const long long sum = y0 + y1, dx = y1 - y0, dy = (z2 - z0) + (z3 - z1);
+            const long long dz = sum - 2 * ((q.n[0] + q.n[1]) + (q.n[2] + q.n[3]));
+            M.add_n(sum);
+            M.add_e(ew, sum);
+            M.add_k_pos(0, P.np[0] - 1 - 2 * q.h[0], dx);  // 2 (n-1-h) + 1 - n of the upper cell
+            M.add_k_pos(1, P.np[1] - 1 - 2 * q.h[1], dy);
+            M.add_k_pos(2, P.np[2] - 1 - 2 * q.h[2], dz);
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int j = j0 + u * (int)blockDim.x;
-            if (j >= jhi) break;
-            const long long n = nv[u];
-            const int jv[3] = {jpv[u] & 0xff, (jpv[u] >> 8) & 0xff, jpv[u] >> 16};
-            const float pf0 = s_pf[0][jv[0]], pf1 = s_pf[1][jv[1]], pf2 = s_pf[2][jv[2]];
-            const float ppf = (pf0 * pf0 + pf1 * pf1) + pf2 * pf2;
-            const float ew = sqrtf(ppf + m) * 16777216.0f;
+    } else {
+        const int np1 = P.np[1], np2 = P.np[2];
+        for (int j = lo + (int)threadIdx.x; j < hi; j += MOM_THREADS) {
+            const long long n = __ldg(st + j);
+            const int jxy = j / np2;
             neg += n < 0;
             over += n > pauli;
-            const unsigned nl = (unsigned)n;
-            const int nh = (int)(n >> 32);
-            s_nl += nl;
-            s_nh += nh;
-            if (ew < 2147483648.0f) {  // E_fx < 2^31 (ew is >= 0 or NaN)
-                const unsigned Efx = (unsigned)__float2int_rn(ew);  // round half even
-                const unsigned long long tl = (unsigned long long)Efx * nl;
-                el_lo += tl;
-                el_hi += el_lo < tl;
-                const long long th = (long long)(int)Efx * nh;
-                const unsigned long long o = eh_lo;
-                eh_lo += (unsigned long long)th;
-                eh_hi += (th >> 63) + (eh_lo < o);
-            } else {
-                e_wide += (__int128)rint_ll(ew) * n;
-            }
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const int k = 2 * jv[d] + 1 - P.np[d];
-                kl[d] += (unsigned long long)(unsigned)(k + 256) * nl;
-                kh[d] += (long long)k * nh;
-            }
+            cell(jxy / np1, jxy % np1, j % np2, n);
         }
     }
-    __int128 v[5];
-    const __int128 snl = (__int128)s_nl;
     const __int128 two32 = (__int128)1 << 32;
-    v[0] = (__int128)s_nh * two32 + snl;
-    const __int128 eh = (__int128)(((unsigned __int128)(unsigned long long)eh_hi << 64) | eh_lo);
-    v[1] = (__int128)(((unsigned __int128)el_hi << 64) | el_lo) + eh * two32 + e_wide;
+    __int128 v[5];
+    v[0] = (__int128)M.s_nh * two32 + (__int128)M.s_nl;
+    v[1] = M.energy();
 #pragma unroll
-    for (int d = 0; d < 3; ++d) v[2 + d] = (__int128)kh[d] * two32 + ((__int128)kl[d] - 256 * snl);
-    __shared__ __int128 red[5][8];
+    for (int d = 0; d < 3; ++d) v[2 + d] = (__int128)M.kh[d] * two32 + (__int128)M.kl[d];
+    __shared__ __int128 red[5][MOM_THREADS / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (P.sflags) {
+    if (P.sflags && __any_sync(0xffffffffu, neg | over)) {
         neg = warp_sum(neg);
         over = warp_sum(over);
         if (lane == 0 && neg) red_add_ll(&P.sflags[0], neg);
@@ -1052,7 +1142,7 @@ __device__ __forceinline__ void moments_block(const MomentArgs& P, int64_t x, in
     __syncthreads();
     if (threadIdx.x == 0) {
         __int128 t[5] = {0, 0, 0, 0, 0};
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+        for (int w = 0; w < MOM_THREADS / 32; ++w)
             for (int i = 0; i < 5; ++i) t[i] += red[i][w];
         if (part) {  // exact partial sums of this chunk, combined by k_moments_finish
             for (int i = 0; i < 5; ++i) {
@@ -1067,16 +1157,15 @@ __device__ __forceinline__ void moments_block(const MomentArgs& P, int64_t x, in
 
 // Block = (x cell, slot, chunk of the p cells); with one chunk the block
 // writes the moments, else its exact partial sums for k_moments_finish.
-__global__ void __launch_bounds__(256, BZ_MOM_MINB) k_moments(const __grid_constant__ MomentArgs P)
+__global__ void __launch_bounds__(MOM_THREADS, 7) k_moments(const __grid_constant__ MomentArgs P)
 {
     const int nch = P.nchunk > 1 ? P.nchunk : 1;
     const int64_t row = blockIdx.x / nch;
     const int c = (int)(blockIdx.x % nch);
     const int64_t x = row / P.nslots;
     const int sl = (int)(row % P.nslots);
-    const int jlo = (int)((int64_t)c * P.npc / nch), jhi = (int)((int64_t)(c + 1) * P.npc / nch);
     double* out = P.out + (P.kidx ? (int64_t)*P.kidx * P.kstride : 0);
-    moments_block(P, x, sl, jlo, jhi, out + (x * P.nslots + sl) * 5, nch > 1 ? P.part + (int64_t)blockIdx.x * 10 : nullptr);
+    moments_block(P, x, sl, c, nch, out + (x * P.nslots + sl) * 5, nch > 1 ? P.part + (int64_t)blockIdx.x * 10 : nullptr);
 }
 
 // Adds the chunks' partial sums of each (x cell, slot) in chunk order.
@@ -1098,7 +1187,7 @@ cudaError_t launch_moments(const MomentArgs& a, cudaStream_t s)
     const int nch = a.nchunk > 1 && a.part ? a.nchunk : 1;
     MomentArgs b = a;
     b.nchunk = nch;
-    k_moments<<<(unsigned)(a.nxc * a.nslots * nch), 256, 0, s>>>(b);
+    k_moments<<<(unsigned)(a.nxc * a.nslots * nch), MOM_THREADS, 0, s>>>(b);
     if (nch > 1) k_moments_finish<<<(unsigned)((a.nxc * a.nslots + 127) / 128), 128, 0, s>>>(b);
     return cudaGetLastError();
 }
@@ -1110,7 +1199,7 @@ cudaError_t launch_moments(const MomentArgs& a, cudaStream_t s)
 // S_ex^0 part (1/2)((m^2 - m^2_prev)/dt) I and the T_total term -(1/4) m^2 I
 // in FP64.  With the massless dispersion both m^2 terms are zero.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_energy_source(const __grid_constant__ MomentArgs P)
+__global__ void __launch_bounds__(MOM_THREADS) k_energy_source(const __grid_constant__ MomentArgs P)
 {
     __shared__ float s_pf[3][MAX_NP];
     for (int d = 0; d < 3; ++d)
@@ -1121,40 +1210,36 @@ __global__ void __launch_bounds__(256) k_energy_source(const __grid_constant__ M
     const int ms = P.slot_mslot[sl];
     const float m = P.mass_mode == 1 ? 0.0f : (float)P.m2[x * 4 + ms];
     const long long* st = P.state + ((int64_t)sl * P.nxc + x) * P.npc;
-    const int npc = (int)P.npc;
-    // n = nh 2^32 + nl: sum R nl (unsigned) and sum R nh (signed), each in 128 bits by carries
-    unsigned long long l_lo = 0, l_hi = 0, h_lo = 0;
-    long long h_hi = 0;
-    __int128 wide = 0;  // cells with 2^24 / E >= 2^31 (E < 2^-7 GeV)
-    for (int j = threadIdx.x; j < npc; j += blockDim.x) {
-        const int jp = __ldg(P.jtab + j);
-        const float pf0 = s_pf[0][jp & 0xff], pf1 = s_pf[1][(jp >> 8) & 0xff], pf2 = s_pf[2][jp >> 16];
-        const float ppf = (pf0 * pf0 + pf1 * pf1) + pf2 * pf2;
-        const float w = (1.0f / sqrtf(ppf + m)) * 16777216.0f;
-        const long long n = __ldg(st + j);
-        if (w < 2147483648.0f) {
-            const unsigned R = (unsigned)rint_split(w);
-            const unsigned long long tl = (unsigned long long)R * (unsigned)n;
-            l_lo += tl;
-            l_hi += l_lo < tl;
-            const long long th = (long long)(int)R * (int)(n >> 32);
-            const unsigned long long o = h_lo;
-            h_lo += (unsigned long long)th;
-            h_hi += (th >> 63) + (h_lo < o);
-        } else {
-            wide += (__int128)rint_ll(w) * n;
+    MomSums M;  // its energy sums, with 2^24 / E in the place of E 2^24
+    auto weight = [&](int j0, int j1, int j2) {
+        const float pf0 = s_pf[0][j0], pf1 = s_pf[1][j1], pf2 = s_pf[2][j2];
+        return (1.0f / sqrtf((pf0 * pf0 + pf1 * pf1) + pf2 * pf2 + m)) * 16777216.0f;
+    };
+    if (P.noct) {
+        for (int i = (int)threadIdx.x; i < P.noct; i += MOM_THREADS) {
+            Octet q;
+            load_octet(P, st, i, q);
+            const float w = weight(q.h[0], q.h[1], q.h[2]);
+            if (q.hi < (1u << 26) || octet_narrow(q))
+                M.add_e(w, octet_sum(q));
+            else
+                for (int k = 0; k < 8; ++k) M.add_e(w, q.n[k]);
+        }
+    } else {
+        const int np1 = P.np[1], np2 = P.np[2];
+        for (int j = (int)threadIdx.x; j < (int)P.npc; j += MOM_THREADS) {
+            const int jxy = j / np2;
+            M.add_e(weight(jxy / np1, jxy % np1, j % np2), __ldg(st + j));
         }
     }
-    const __int128 hpart = (__int128)(((unsigned __int128)(unsigned long long)h_hi << 64) | h_lo);
-    __int128 v = (__int128)(((unsigned __int128)l_hi << 64) | l_lo) + hpart * ((__int128)1 << 32) + wide;
-    __shared__ __int128 red[8];
+    __shared__ __int128 red[MOM_THREADS / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    v = warp_sum_i128(v);
+    const __int128 v = warp_sum_i128(M.energy());
     if (lane == 0) red[warp] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
         __int128 t = 0;
-        for (int w8 = 0; w8 < (int)(blockDim.x >> 5); ++w8) t += red[w8];
+        for (int w = 0; w < MOM_THREADS / 32; ++w) t += red[w];
         const double I = i128_to_double(t) * P.pref * (1.0 / 16777216.0);
         const double mc = P.mass_mode == 1 ? 0.0 : P.m2[x * 4 + ms];
         const double mp = P.mass_mode == 1 ? 0.0 : P.m2_prev[x * 4 + ms];
@@ -1167,8 +1252,8 @@ __global__ void __launch_bounds__(256) k_energy_source(const __grid_constant__ M
 
 cudaError_t launch_energy_source(const MomentArgs& a, cudaStream_t s)
 {
-    if (!a.jtab || !a.m2_prev) return cudaErrorInvalidValue;
-    k_energy_source<<<(unsigned)(a.nxc * a.nslots), 256, 0, s>>>(a);
+    if (!a.m2_prev) return cudaErrorInvalidValue;
+    k_energy_source<<<(unsigned)(a.nxc * a.nslots), MOM_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1214,7 +1299,7 @@ cudaError_t launch_convert_batch(const long long* state, float* f, const int64_t
 
 // Moments of every (box, slot): one block each, through slot_prefix; out
 // advances by one step's worth per call index (*kidx).
-__global__ void __launch_bounds__(256, BZ_MOM_MINB) k_moments_batch(const MomentArgs* __restrict__ boxes,
+__global__ void __launch_bounds__(MOM_THREADS) k_moments_batch(const MomentArgs* __restrict__ boxes,
                                                        const int* __restrict__ slot_prefix, int nboxes,
                                                        double* out, const int* kidx, int per_step)
 {
@@ -1223,14 +1308,14 @@ __global__ void __launch_bounds__(256, BZ_MOM_MINB) k_moments_batch(const Moment
         const int mid = (lo + hi + 1) >> 1;
         if (slot_prefix[mid] <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
     }
-    moments_block(boxes[lo], 0, (int)blockIdx.x - slot_prefix[lo], 0, (int)boxes[lo].npc,
+    moments_block(boxes[lo], 0, (int)blockIdx.x - slot_prefix[lo], 0, 1,
                   out + (int64_t)(*kidx) * per_step + 5 * (int64_t)blockIdx.x, nullptr);
 }
 
 cudaError_t launch_moments_batch(const MomentArgs* boxes, const int* slot_prefix, int nboxes, int nblocks,
                                  double* out, const int* kidx, int per_step, cudaStream_t s)
 {
-    k_moments_batch<<<nblocks, 256, 0, s>>>(boxes, slot_prefix, nboxes, out, kidx, per_step);
+    k_moments_batch<<<nblocks, MOM_THREADS, 0, s>>>(boxes, slot_prefix, nboxes, out, kidx, per_step);
     return cudaGetLastError();
 }
 
