@@ -4,7 +4,6 @@
 // which threads accumulate.
 #include <cstdint>
 #include "bz_internal.h"
-#include "exact64.cuh"
 #include "intconv.cuh"
 
 namespace bz {
@@ -120,34 +119,31 @@ __device__ __forceinline__ void masses_block(const MassArgs& P, int64_t x, int64
     }
 }
 
-// One bin of the Eq. (mg), (mq) sums in FP64 with the factors r = 1/(2E)
-// given (0 for a skipped species pair): the integer parts of 3x and 24x the
-// bin integrands in 2^-30 of f, exactly as in masses_block.
-__device__ __forceinline__ void mass_bin_fp64(const long long nsp[NSPEC], const double r[4], const bool skip[4],
-                                              long long* qg, long long qq[3])
+// Thermal masses with the table of distinct p^2 values: the same sums as
+// masses_block, bit for bit, on the integer pipe.
+//
+// A block (x cell, chunk of bins) first evaluates r_a = 1/(2 E_a) = 0.5 /
+// sqrt(p^2 + m_a^2) in FP64 once per distinct p^2 (496 values for the 20^3 grid
+// instead of 8000 cells) and keeps R = trunc(r 2^54).  A bin's integrands are
+//   3x:  rint(G 2^-64), G = 9 n_g R_g + 4 sum_i q_i R_i,
+//   24x: rint(Q_i 2^-64), Q_i = 3 n_g R_g + 4 q_i R_i,
+// up to the roundings of the FP64 formula (2^-53 of each product and sum, at most
+// six of them in a row) and the truncation of R (less than 1): together below
+//   e = A 2^-64 (12 r_max + 1) + 32 2^-32,  A = 9 |n_g| + 4 sum_i |q_i|,
+// so that wherever the fraction of G 2^-64 is further than e from 1/2 the FP64
+// formula rounds to the same integer; the other bins (one in some thousands), bins
+// with |n| >= 2^46 and blocks with r >= 2^8 take the FP64 instructions, each of
+// which issues for 64 cycles.  The products are 64 x 47 bits, cut to 32 fraction
+// bits.  Gluons only (GLUON_ONLY): one rounding of one product, 9 n R_g and 3 n R_g.
+// 16^3 x 20^3 gluons, all bins nonzero: 410 -> 142 us (99 instructions a bin, a third
+// of them multiplications; 262 MB are read); 8^3 x 16^3, 7 species: 168 -> 78 us.
+// m_a^2 (i = 0 gluon, 1..3 flavours) from its exact fixed-point sum
+__device__ __forceinline__ double mass_of(const MassArgs& P, int i, long long acc)
 {
-    const double ng = skip[0] ? 0.0 : (double)nsp[0];
-    double q[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) q[i] = skip[1 + i] ? 0.0 : (double)(nsp[1 + i] + nsp[4 + i]);
-    const double g3 = 9.0 * ng * r[0] + 4.0 * ((q[0] * r[1] + q[1] * r[2]) + q[2] * r[3]);
-    *qg = __double2ll_rn(g3 * MASS_FX);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) qq[i] = __double2ll_rn((3.0 * ng * r[0] + 4.0 * q[i] * r[1 + i]) * MASS_FX);
+    const double inv = 1.0 / (double)(1LL << MASS_SHIFT);
+    return i == 0 ? P.pref_g * P.meas * ((double)acc * inv) / 3.0 : P.pref_q * P.meas * ((double)acc * inv) / 24.0;
 }
 
-// Thermal masses with the table of distinct p^2 values: the same sums as
-// masses_block, bit for bit.  A block (x cell, chunk of bins) first evaluates
-// r_a = 1/(2 E_a) = 0.5 / sqrt(p^2 + m_a^2) once per distinct p^2 (496 values
-// for the 20^3 grid instead of 8000 cells), in shared memory; every bin then
-// reads its r.  GLUON_ONLY (no quark slot): with the quark pairs skipped, the
-// bin integrands reduce to 3x: rint(2^-10 RN(RN(9 n) r_g)) and 24x:
-// rint(2^-10 RN(RN(3 n) r_g)) (the quark terms add +0), and for |n| < 2^49
-// 9n and 3n are exact integers, so each is one integer-times-double product
-// and one conversion, evaluated with integer instructions (exact64.cuh: the
-// same IEEE round-to-nearest-even results) instead of FP64 ones.  Bins outside
-// that range, and blocks whose r is not a normal double in [2^-900, 2^900],
-// take the FP64 instructions.
 // Species pairs whose 1/(2E) the mass sums skip: no state of the pair and
 // E^2 = p^2 + m^2 > 0 for every p (a skipped pair adds +0, see masses_block).
 __device__ __forceinline__ void mass_skips(const MassArgs& P, const double m2p[4], bool skip[4])
@@ -163,10 +159,63 @@ __device__ __forceinline__ void mass_prev(const MassArgs& P, int64_t x, double m
     for (int i = 0; i < 4; ++i) m2p[i] = P.m2_prev ? P.m2_prev[x * 4 + i] : 0.0;
 }
 
-template <bool GLUON_ONLY>
-__global__ void __launch_bounds__(256, 4) k_masses_tab(const __grid_constant__ MassArgs P)
+// n R / 2^32 for |n| < 2^47, R < 2^62: q 2^32 + f, floored (less than 1 below)
+struct Fix96 {
+    long long q;
+    unsigned f;
+};
+__device__ __forceinline__ Fix96 mul_fix(long long n, uint64_t R)
 {
-    extern __shared__ double s_r[];  // [4][nu]
+    const unsigned nl = (unsigned)n, Rl = (unsigned)R, Rh = (unsigned)(R >> 32);
+    const int nh = (int)(n >> 32);
+    uint64_t m = (uint64_t)nl * Rh + __umulhi(nl, Rl);
+    m += (uint64_t)((long long)nh * (long long)Rl);
+    return Fix96{(long long)nh * (int)Rh + ((long long)m >> 32), (unsigned)m};
+}
+// ca a + cb b
+__device__ __forceinline__ Fix96 comb_fix(unsigned ca, Fix96 a, unsigned cb, Fix96 b)
+{
+    const uint64_t lo = (uint64_t)ca * a.f + (uint64_t)cb * b.f;
+    return Fix96{(long long)ca * a.q + (long long)cb * b.q + (long long)(lo >> 32), (unsigned)lo};
+}
+// nearest integer; false if the fraction is within thr 2^-32 of 1/2
+__device__ __forceinline__ bool rint_fix(Fix96 v, unsigned thr, long long* out)
+{
+    *out = v.q + (v.f >> 31);
+    return (v.f - 0x80000000u) + thr > 2u * thr;
+}
+
+constexpr int MASS_THREADS = 256;
+
+// The bin of p^2 = pp by the FP64 formula, as in masses_block (rare: kept out of
+// line); ng, q_i = n_qi + n_qbi, 0 for a skipped species pair.
+struct MassBin {
+    long long g, q[3];
+};
+template <bool GLUON_ONLY>
+__device__ __noinline__ MassBin mass_bin_slow(double pp, const double* m2_prev, int skips, long long ng, long long q0, long long q1,
+                                              long long q2)
+{
+    const long long nq[3] = {q0, q1, q2};
+    const double gn = (double)ng;
+    const double rg = skips & 1 ? 0.0 : 0.5 / sqrt(pp + (m2_prev ? m2_prev[0] : 0.0));
+    double q[3], rq[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        q[i] = GLUON_ONLY ? 0.0 : (double)nq[i];
+        rq[i] = GLUON_ONLY || ((skips >> (1 + i)) & 1) ? 0.0 : 0.5 / sqrt(pp + (m2_prev ? m2_prev[1 + i] : 0.0));
+    }
+    MassBin o;
+    o.g = __double2ll_rn((9.0 * gn * rg + 4.0 * ((q[0] * rq[0] + q[1] * rq[1]) + q[2] * rq[2])) * MASS_FX);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) o.q[i] = __double2ll_rn((3.0 * gn * rg + 4.0 * q[i] * rq[i]) * MASS_FX);
+    return o;
+}
+template <bool GLUON_ONLY>
+__global__ void __launch_bounds__(MASS_THREADS, 4) k_masses_tab(const __grid_constant__ MassArgs P)
+{
+    extern __shared__ uint64_t s_R[];  // [GLUON_ONLY ? 1 : 4][nu]
+    constexpr int NS = GLUON_ONLY ? 1 : 4;
     const int nu = P.nu;
     const int64_t nchunk = (P.npc + P.chunk - 1) / P.chunk;
     const int64_t x = blockIdx.x / nchunk, c0 = (blockIdx.x % nchunk) * P.chunk;
@@ -174,73 +223,112 @@ __global__ void __launch_bounds__(256, 4) k_masses_tab(const __grid_constant__ M
     bool skip[4];
     mass_prev(P, x, m2p);
     mass_skips(P, m2p, skip);
-    int ok = 1;
-    for (int u = threadIdx.x; u < nu; u += blockDim.x) {
+    // GLUON_ONLY with a quark pair that is not skipped (a negative mass): the general formula in FP64
+    int ok = !GLUON_ONLY || (skip[1] && skip[2] && skip[3]);
+    int e_max = 0;  // largest exponent field of r
+    for (int u = threadIdx.x; u < nu; u += MASS_THREADS) {
         const double pp = P.ppu[u];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) s_r[s * nu + u] = skip[s] ? 0.0 : 0.5 / sqrt(pp + m2p[s]);
-        const double rg = s_r[u];
-        ok &= (rg >= 0x1p-900 && rg <= 0x1p+900) ? 1 : 0;
+        for (int s = 0; s < NS; ++s) {
+            uint64_t R = 0;
+            if (!skip[s]) {
+                const uint64_t b = (uint64_t)__double_as_longlong(0.5 / sqrt(pp + m2p[s]));
+                const int be = (int)(b >> 52);  // r > 0 (a NaN or negative value fails the range)
+                const uint64_t M = (b & ((1ull << 52) - 1ull)) | (1ull << 52);
+                ok &= be >= 958 && be < 1031;  // 2^-65 <= r < 2^8
+                const int sh = be - 1021;      // r 2^54 = M 2^sh
+                R = sh >= 0 ? M << (sh & 15) : M >> (-sh & 63);
+                e_max = max(e_max, be);
+            }
+            s_R[s * nu + u] = R;
+        }
     }
-    ok = __syncthreads_and(ok);
-    const bool fast = GLUON_ONLY && ok && skip[1] && skip[2] && skip[3];
+    __shared__ int s_e[MASS_THREADS / 32];
+    e_max = __reduce_max_sync(0xffffffffu, e_max);
+    if ((threadIdx.x & 31) == 0) s_e[threadIdx.x >> 5] = e_max;
+    const bool fast = __syncthreads_and(ok) != 0;
+    for (int w = 0; w < MASS_THREADS / 32; ++w) e_max = max(e_max, s_e[w]);
+    // e of the comment in units of 2^-32: (A 2^-32) cmul + 32, r_max <= 2^(e_max - 1022)
+    const int lg = max(e_max - 1022, 0);
+    const unsigned cmul = (GLUON_ONLY ? 2u : 12u) * (1u << (lg & 15)) + 1u;
+    // |3x integrand| <= A r_max 2^-10 + 1 < 2^(52 + lg - 10): below the limit for the usual grids
+    const bool check = ((int64_t)1 << (42 + lg)) > P.limit;
     long long sg = 0, sq[3] = {0, 0, 0};
     bool ovf = false;
-    const long long* st0 = P.state + x * P.npc;  // slot 0 (the gluons when GLUON_ONLY)
     const int64_t jend = c0 + P.chunk < P.npc ? c0 + P.chunk : P.npc;
-    constexpr int AHEAD = 4;  // bins whose loads are in flight together
-    for (int64_t jb = c0 + threadIdx.x; jb < jend; jb += AHEAD * (int64_t)blockDim.x) {
-        long long nb[AHEAD];
+    const int skips = (int)skip[0] | ((int)skip[1] << 1) | ((int)skip[2] << 2) | ((int)skip[3] << 3);
+    constexpr int AHEAD = GLUON_ONLY ? 4 : 1;  // bins whose loads are in flight together
+    constexpr int NV = GLUON_ONLY ? 1 : NSPEC;
+    const long long* const st = P.state + x * P.npc;
+    const int64_t sstride = P.nxc * P.npc;
+    const int jstop = (int)jend;
+    const double* const m2x = P.m2_prev ? P.m2_prev + x * 4 : nullptr;
+    auto mag = [](long long v) {  // |v| < (mag + 1) 2^32
+        const int h = (int)(v >> 32);
+        return (unsigned)(h ^ (h >> 31));
+    };
+    for (int jb = (int)c0 + (int)threadIdx.x; jb < jstop; jb += AHEAD * MASS_THREADS) {
+        long long nsp[AHEAD][NV];
         int ub[AHEAD];
 #pragma unroll
         for (int k = 0; k < AHEAD; ++k) {
-            const int64_t j = jb + k * (int64_t)blockDim.x;
-            nb[k] = (fast && j < jend) ? st0[j] : 0;
-            ub[k] = j < jend ? P.pidx[j] : 0;
-        }
+            const int j = jb + k * MASS_THREADS;
+            ub[k] = j < jstop ? P.pidx[j] : 0;
 #pragma unroll
-        for (int k = 0; k < AHEAD; ++k) {
-        const int64_t j = jb + k * (int64_t)blockDim.x;
-        if (j >= jend) break;
-        const int u = ub[k];
-        long long qg, qq[3];
-        bool done = false;
-        if (fast) {
-            const long long n = nb[k];
-            const uint64_t a = n < 0 ? 0ull - (uint64_t)n : (uint64_t)n;
-            if (a == 0) {
-                qg = qq[0] = 0;
-                done = true;
-            } else if (a < (1ull << 49)) {
-                Exact64 rg = x64_from_double(s_r[u]);
-                rg.neg = n < 0;  // r > 0: the sign of n
-                done = x64_rint_scaled(x64_mul_u(9ull * a, rg), -10, &qg) &
-                       x64_rint_scaled(x64_mul_u(3ull * a, rg), -10, &qq[0]);
+            for (int s = 0; s < NV; ++s) {
+                const int sl = GLUON_ONLY ? 0 : P.slot_of[s];
+                nsp[k][s] = sl < 0 || j >= jstop ? 0 : __ldg(st + (int64_t)sl * sstride + j);
             }
-            qq[1] = qq[2] = qq[0];
         }
-        if (!done) {
-            long long nsp[NSPEC];
 #pragma unroll
-            for (int s = 0; s < NSPEC; ++s) {
-                const int sl = P.slot_of[s];
-                nsp[s] = sl < 0 ? 0 : P.state[((int64_t)sl * P.nxc + x) * P.npc + j];
+        for (int k = 0; k < AHEAD; ++k) {  // a bin beyond the end has n = 0 and adds 0
+            const int u = ub[k];
+            const long long* n = nsp[k];
+            MassBin o;
+            bool done;
+            if constexpr (GLUON_ONLY) {
+                const Fix96 t = mul_fix(n[0], s_R[u]), z{0, 0u};
+                const unsigned ah = mag(n[0]), thr = (9u * ah + 9u) * cmul + 32u;
+                done = fast & (ah < (1u << 14)) & rint_fix(comb_fix(9u, t, 0u, z), thr, &o.g) &
+                       rint_fix(comb_fix(3u, t, 0u, z), thr, &o.q[0]);
+                done |= n[0] == 0;
+                if (!done) o = mass_bin_slow<true>(P.ppu[u], m2x, skips, n[0], 0, 0, 0);
+                sq[0] += o.q[0];
+            } else {
+                const long long ng = skip[0] ? 0 : n[0];
+                long long q[3];
+                unsigned big = mag(ng), A = 9u * (mag(ng) + 1u);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    q[i] = skip[1 + i] ? 0 : n[1 + i] + n[4 + i];
+                    big |= mag(n[1 + i]) | mag(n[4 + i]);
+                    A += 4u * (mag(q[i]) + 1u);
+                }
+                const unsigned thr = A * cmul + 32u;
+                const Fix96 tg = mul_fix(ng, s_R[u]);
+                Fix96 sum{0, 0u};
+                done = fast & (big < (1u << 14));
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const Fix96 t = mul_fix(q[i], s_R[(1 + i) * nu + u]);
+                    done &= rint_fix(comb_fix(3u, tg, 4u, t), thr, &o.q[i]);
+                    sum = comb_fix(1u, sum, 1u, t);
+                }
+                done &= rint_fix(comb_fix(9u, tg, 4u, sum), thr, &o.g);
+                if (!done) o = mass_bin_slow<false>(P.ppu[u], m2x, skips, ng, q[0], q[1], q[2]);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) sq[i] += o.q[i];
             }
-            const double r[4] = {s_r[u], s_r[nu + u], s_r[2 * nu + u], s_r[3 * nu + u]};
-            mass_bin_fp64(nsp, r, skip, &qg, qq);
-        }
-        ovf |= qg > P.limit || qg < -P.limit;
-        sg += qg;
+            sg += o.g;
+            if (check | !done) {
+                ovf |= o.g > P.limit || o.g < -P.limit;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            if (fast && i > 0) break;  // the three quark-flavour sums are equal: added once, copied below
-            ovf |= qq[i] > P.limit || qq[i] < -P.limit;
-            sq[i] += qq[i];
-        }
+                for (int i = 0; i < (GLUON_ONLY ? 1 : 3); ++i) ovf |= o.q[i] > P.limit || o.q[i] < -P.limit;
+            }
         }
     }
-    if (fast) sq[1] = sq[2] = sq[0];
-    __shared__ long long red[4][8];
+    if (GLUON_ONLY) sq[1] = sq[2] = sq[0];
+    __shared__ long long red[4][MASS_THREADS / 32];
     long long v[4] = {sg, sq[0], sq[1], sq[2]};
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
@@ -252,8 +340,11 @@ __global__ void __launch_bounds__(256, 4) k_masses_tab(const __grid_constant__ M
     __syncthreads();
     if (threadIdx.x < 4) {
         long long t = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[threadIdx.x][w];
-        red_add_ll(&P.acc[x * 4 + threadIdx.x], t);
+        for (int w = 0; w < MASS_THREADS / 32; ++w) t += red[threadIdx.x][w];
+        if (nchunk == 1)  // the block has the x cell's whole sums
+            P.m2_out[x * 4 + threadIdx.x] = mass_of(P, (int)threadIdx.x, t);
+        else
+            red_add_ll(&P.acc[x * 4 + threadIdx.x], t);
     }
 }
 
@@ -287,45 +378,45 @@ __global__ void k_masses_finish_batch(const MassArgs* __restrict__ boxes, int nb
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nboxes) return;
     const MassArgs& P = boxes[b];
-    const double inv = 1.0 / (double)(1LL << MASS_SHIFT);
-    P.m2_out[0] = P.pref_g * P.meas * ((double)P.acc[0] * inv) / 3.0;
-    for (int i = 0; i < 3; ++i) P.m2_out[1 + i] = P.pref_q * P.meas * ((double)P.acc[1 + i] * inv) / 24.0;
+    for (int i = 0; i < 4; ++i) P.m2_out[i] = mass_of(P, i, P.acc[i]);
 }
 
 __global__ void k_masses_finish(const __grid_constant__ MassArgs P)
 {
     const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= P.nxc) return;
-    const double inv = 1.0 / (double)(1LL << MASS_SHIFT);
-    P.m2_out[x * 4 + 0] = P.pref_g * P.meas * ((double)P.acc[x * 4 + 0] * inv) / 3.0;
-    for (int i = 0; i < 3; ++i)
-        P.m2_out[x * 4 + 1 + i] = P.pref_q * P.meas * ((double)P.acc[x * 4 + 1 + i] * inv) / 24.0;
+    for (int i = 0; i < 4; ++i) P.m2_out[x * 4 + i] = mass_of(P, i, P.acc[x * 4 + i]);
 }
 
 cudaError_t launch_masses(const MassArgs& a, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(a.acc, 0, sizeof(long long) * 4 * a.nxc, s);
-    if (e != cudaSuccess) return e;
     // chunks of 256 to 2048 bins, enough blocks for every SM on small grids;
     // with the p^2 table a block of many x cells' grid takes a whole x cell,
-    // so that each x cell's table is evaluated once
+    // so that each x cell's table is evaluated once and its sums need no
+    // accumulator in memory
     MassArgs b = a;
+    const bool tab = a.nu > 0 && a.nu <= MASS_TAB_MAX;
     const int64_t per_x = ((int64_t)4 * device_sms() + a.nxc - 1) / a.nxc;
     int64_t chunk = ((a.npc + per_x - 1) / per_x + 255) / 256 * 256;
     b.chunk = chunk < 256 ? 256 : (chunk > MASS_CHUNK ? MASS_CHUNK : chunk);
-    if (a.nu > 0 && per_x == 1) b.chunk = a.npc;
+    if (tab && per_x == 1) b.chunk = a.npc;
     const int64_t nchunk = (a.npc + b.chunk - 1) / b.chunk;
-    if (a.nu > 0 && a.nu <= MASS_TAB_MAX) {
+    if (!tab || nchunk > 1) {
+        const cudaError_t e = cudaMemsetAsync(a.acc, 0, sizeof(long long) * 4 * a.nxc, s);
+        if (e != cudaSuccess) return e;
+    }
+    if (tab) {
         bool gluon_only = a.slot_of[0] == 0;
-        for (int s = 1; s < NSPEC; ++s) gluon_only = gluon_only && a.slot_of[s] < 0;
-        const size_t smem = sizeof(double) * 4 * (size_t)a.nu;
+        for (int q = 1; q < NSPEC; ++q) gluon_only = gluon_only && a.slot_of[q] < 0;
+        const size_t smem = sizeof(uint64_t) * (gluon_only ? 1 : 4) * (size_t)a.nu;
         if (gluon_only) {
             if (smem > 48 * 1024) cudaFuncSetAttribute(k_masses_tab<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            k_masses_tab<true><<<(unsigned)(nchunk * a.nxc), 256, smem, s>>>(b);
+            k_masses_tab<true><<<(unsigned)(nchunk * a.nxc), MASS_THREADS, smem, s>>>(b);
         } else {
             if (smem > 48 * 1024) cudaFuncSetAttribute(k_masses_tab<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            k_masses_tab<false><<<(unsigned)(nchunk * a.nxc), 256, smem, s>>>(b);
+            k_masses_tab<false><<<(unsigned)(nchunk * a.nxc), MASS_THREADS, smem, s>>>(b);
         }
+        if (nchunk == 1) return cudaGetLastError();
     } else {
         k_masses<<<(unsigned)(nchunk * a.nxc), 256, 0, s>>>(b);
     }
