@@ -42,7 +42,6 @@ struct bz_handle_s {
     int nu = 0;                    // their count (0: no table)
     float* d_inv_e = nullptr;      // drift scratch: 1/E of every cell (inhomogeneous grids)
     float* d_gforce = nullptr;     // force-term scratch: g_i per (x cell, mass slot, axis)
-    float* d_m2f = nullptr;        // drift scratch: FP32 m^2 per (x cell, mass slot)
     unsigned long long* d_counter = nullptr;  // FP32 collision: units handed out
     double* d_m2prev = nullptr;    // energy source: the caller's previous masses [x][4]
     long long* d_mom_part = nullptr;  // moments: exact partial sums of the p-cell chunks
@@ -204,8 +203,6 @@ static void free_scratch(bz_handle h)
     h->d_inv_e = nullptr;
     cudaFree(h->d_gforce);
     h->d_gforce = nullptr;
-    cudaFree(h->d_m2f);
-    h->d_m2f = nullptr;
     cudaFree(h->d_counter);
     h->d_counter = nullptr;
     cudaFree(h->d_m2prev);
@@ -261,8 +258,6 @@ static int alloc_scratch(bz_handle h)
         return fail(h, BZ_ENOMEM, "cannot allocate %lld bytes for the drift", (long long)(4 * h->ncell));
     if (h->nxc > 1 && !h->d_gforce && cudaMalloc(&h->d_gforce, sizeof(float) * 12 * h->nxc) != cudaSuccess)
         return fail(h, BZ_ENOMEM, "cannot allocate the force-term scratch");
-    if (h->nxc > 1 && !h->d_m2f && cudaMalloc(&h->d_m2f, sizeof(float) * 4 * h->nxc) != cudaSuccess)
-        return fail(h, BZ_ENOMEM, "cannot allocate the drift's mass table");
     return BZ_OK;
 }
 
@@ -962,9 +957,11 @@ static int fill_drift(bz_handle h, DriftArgs& a, const long long* in, long long*
         double dp = dp_of(h, d);
         for (int j = 0; j < h->g.np[d]; ++j) a.pf[d][j] = (float)(-h->g.L + ((double)j + 0.5) * dp);
     }
+    momentum_octets(a);
+    a.dv_n2 = div_magic((uint32_t)a.np[2]);
+    a.dv_h1 = div_magic((uint32_t)((a.np[1] + 1) / 2));
     a.jtab = h->d_jtab;
     a.inv_e = h->d_inv_e;
-    a.m2f = h->d_m2f;
     // the force needs a mass gradient: none with one x cell or the massless dispersion
     a.force = h->force && h->nxc > 1 && h->mass_mode != BZ_MASS_MASSLESS;
     a.gforce = h->d_gforce;

@@ -508,20 +508,6 @@ __device__ __forceinline__ int rint_split(float w)
 }
 
 
-__device__ __forceinline__ long long flux_n(long long n, int C)
-{
-    return flux32((int)(n >> 32), (unsigned)n, C);
-}
-
-// Courant integer of the narrow form, rint((p_d inv) K) with K = dt/dx 2^30,
-// round half even by the hardware conversion (|w| < 2^31 in the narrow form):
-// the exact power-of-two factor folded into K gives the same float as
-// ((p_d inv) dt/dx) 2^30 wherever the rounded value can be nonzero.
-__device__ __forceinline__ int courant_cvt(float pd, float inv, float K)
-{
-    return __float2int_rn((pd * inv) * K);
-}
-
 // Force term of Eq. (left handside), -div_p[(grad_x E) f]: along p_i the p
 // cells of an x cell all move with dp_i/dt = -dE/dx_i = -g_i / E, where
 // g_i = (m^2(x + e_i) - m^2(x - e_i)) / (4 dx) is half the central difference
@@ -659,54 +645,72 @@ __global__ void __launch_bounds__(DRIFT_THREADS) k_drift(const __grid_constant__
     }
 }
 
-constexpr int PLANE_THREADS = 128;
-constexpr int PLANE_MAX_NZ = 40;  // y-face buffer: n_z x PLANE_THREADS int64 of dynamic shared memory
-#ifndef BZ_PLANE_THREADS_PER_SM
-#define BZ_PLANE_THREADS_PER_SM 2048
-#endif
-#ifndef BZ_PLANE_XFAST
-#define BZ_PLANE_XFAST 1  // 1: blocks of all (slot, x index, segment) of a p tile run together (x neighbours in L2)
-#endif
-#ifndef BZ_HW_CVT
-#define BZ_HW_CVT 0       // 1: f conversion with the hardware int64 -> float instruction (slower here)
-#endif
-
-// Asynchronous global -> shared copies (cp.async): the streaming drift keeps
-// its state loads BZ_DPIPE cells ahead of their use without holding registers.
-// Each thread copies and later reads only its own words, so completion of its
-// own groups (wait_group) is the only ordering needed.
-__device__ __forceinline__ void cp_async8(void* dst, const void* src)
+// Half-grid indices of octet o (momentum_octets).
+template <typename Args>
+__device__ __forceinline__ void octet_index(const Args& P, int o, int h[3])
 {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+    h[0] = (int)udiv((uint32_t)o, P.dv_h12);
+    const int r = o - h[0] * (P.half[1] * P.half[2]);
+    h[1] = (int)udiv((uint32_t)r, P.dv_h2);
+    h[2] = r - h[1] * P.half[2];
 }
 
-#ifndef BZ_DPIPE
-#define BZ_DPIPE 2  // cells in flight per thread (cp.async groups)
-#endif
+// ---------------------------------------------------------------------------
+// Drift by mirrored p cells: the integer fluxes of k_drift, in a form that leaves
+// few instructions a cell.
+//
+// A thread takes the four cells (+-p_x, +-p_y, p_z): they share 1/E and, up to its
+// sign, every Courant number, so it reads one 1/E for its x cell and one for each
+// neighbour (a table of 1/E per x cell and octet, written first) instead of
+// evaluating a square root and a division per face, and rounds 8 Courant numbers
+// for 4 cells; consecutive threads are consecutive along p_z, so that every access
+// is coalesced (octets of 8 cells, half as many rounded numbers but 80-byte runs
+// and 128 registers: 558 us).  With C >= 0 the rounded flux n C 2^-30 of a cell
+// moving up, and minus that of a cell moving down, are (n C + 2^29) >> 30 and
+// (n C + 2^29 - 1) >> 30: two wide multiplications and two shifts, the outflow of
+// the own cell and the inflow from the upwind neighbour (lower for a cell moving
+// up, else upper).  Both sides of a face evaluate the same integer.
+// A warp takes 32 such threads' cells, one (slot, x index, y segment) and its x
+// cells in order, the block's warps on consecutive z: the z and y neighbours' rows
+// come from L1, the x neighbours' from L2 (blocks of one tile run together), so the
+// state is read from memory once.  A walk along z and y that carried each face's
+// flux (4 fluxes a cell instead of 6) took 312 instructions a cell and 357 us on
+// the 16^3 x 20^3 gluon box (no f written), this form 273 us.
+// ---------------------------------------------------------------------------
+constexpr int DOCT_WARPS = 4, DRIFT_MINB = 8;  // warps per block, blocks per SM
 
-// FP32 m^2 of every (x cell, mass slot) for the streaming drift, the same
-// rounding as k_inv_energy's per-row value.
-__global__ void k_mass_table(const __grid_constant__ DriftArgs P)
+__global__ void __launch_bounds__(256) k_inv_octet(const __grid_constant__ DriftArgs P)
 {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < P.nxc * 4) P.m2f[t] = P.mass_mode == 1 ? 0.0f : (float)P.m2[t];
+    const int64_t row = blockIdx.x;  // slot, x cell
+    const int sl = (int)(row / P.nxc);
+    const int64_t x = row - (int64_t)sl * P.nxc;
+    const float m = P.mass_mode == 1 ? 0.0f : (float)P.m2[x * 4 + P.slot_mslot[sl]];
+    float* out = P.inv_e + row * P.noct;
+    for (int o = threadIdx.x; o < P.noct; o += 256) {
+        int h[3];
+        octet_index(P, o, h);
+        const float p0 = P.pf[0][h[0]], p1 = P.pf[1][h[1]], p2 = P.pf[2][h[2]];
+        out[o] = 1.0f / sqrtf((p0 * p0 + p1 * p1) + p2 * p2 + m);
+    }
 }
 
-// Force-term part of the update of cell j of one (slot, x) row, as
-// force_acc, with the inverse energy of the cell behind computed in place:
-// it differs from cell j only in its p_i, and shares the x cell's m^2.
-__device__ __forceinline__ long long force_acc_inline(const DriftArgs& P, const float* g3, int jp, int j,
-                                                      const long long* in_row, long long n, float inv,
-                                                      const float (*pf)[MAX_NP], float m)
+// int64 to the nearest float: n = a 2^23 + b with |a| <= 2^22, b < 2^23 both exact
+// in FP32, one rounding; larger n by integer instructions
+__device__ __forceinline__ float ll2float_fast(long long n)
 {
-    const int jv[3] = {jp & 0xff, (jp >> 8) & 0xff, jp >> 16};
+    const int hi = (int)(n >> 32);
+    if ((unsigned)(hi ^ (hi >> 31)) >= (1u << 13)) return ll2float_rn(n);  // |n| >= 2^45
+    const int a = (int)(n >> 23);
+    const float fa = __int_as_float(a + 0x4B400000) - 12582912.0f;
+    const float fb = __uint_as_float(((unsigned)n & 0x7fffffu) | 0x4B000000u) - 8388608.0f;
+    return fmaf(fa, 8388608.0f, fb);
+}
+
+// Force-term part of the update of one cell (p indices jv), as force_acc, with
+// 1/E of the cell behind from the octet table.
+__device__ __noinline__ long long force_acc_octet(const DriftArgs& P, const float* g3, const int jv[3], int j,
+                                            const long long* in_row, const float* inv_row, long long n, float inv)
+{
     const int stride[3] = {P.np[1] * P.np[2], P.np[2], 1};
     long long acc = 0;
 #pragma unroll
@@ -717,160 +721,193 @@ __device__ __forceinline__ long long force_acc_inline(const DriftArgs& P, const 
         const int jo = jv[i] + (up ? 1 : -1), jb = jv[i] + (up ? -1 : 1);
         long long own = 0, behind = 0;
         if (jo >= 0 && jo < P.np[i]) own = force_flux(n, g, inv, P.Kp[i]);
-        if (jb >= 0 && jb < P.np[i] && bz_in(j + (up ? -stride[i] : stride[i]), P.npc)) {
+        if (jb >= 0 && jb < P.np[i]) {
             const int jj = j + (up ? -stride[i] : stride[i]);
-            const float q0 = pf[0][i == 0 ? jb : jv[0]], q1 = pf[1][i == 1 ? jb : jv[1]], q2 = pf[2][i == 2 ? jb : jv[2]];
-            const float invb = 1.0f / sqrtf((q0 * q0 + q1 * q1) + q2 * q2 + m);
-            behind = force_flux(__ldg(in_row + jj), g, invb, P.Kp[i]);
+            int h[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int jd = d == i ? jb : jv[d];
+                h[d] = min(jd, P.np[d] - 1 - jd);
+            }
+            const int o = (h[0] * P.half[1] + h[1]) * P.half[2] + h[2];
+            if (bz_in(jj, P.npc) & bz_in(o, P.noct)) behind = force_flux(__ldg(in_row + jj), g, __ldg(inv_row + o), P.Kp[i]);
         }
         acc += up ? own - behind : behind - own;
     }
     return acc;
 }
 
-// Drift by (y, z) planes, streaming: the integer fluxes of k_drift with every
-// face flux of the two inner x axes computed once per step.  A thread owns
-// one p cell of one (slot, x index ix) and walks a segment of y rows and each
-// row's z cells in the upwind order of its own p_y and p_z, so the flux into
-// the current cell is the one it computed for the previous cell (z, in a
-// register) or for the previous row (y, per z cell in shared memory); each
-// row starts with its periodic wrap cell.  The x axis reads the upwind
-// neighbour.  1/E = 1/sqrt(p^2 + m^2(x)) is computed in place (IEEE FP32, as
-// k_inv_energy) from the p cell's p^2 and the x cell's FP32 m^2, and the
-// state is streamed through a cp.async ring BZ_DPIPE cells ahead, so a step
-// reads the state once (the x neighbours from L2) and writes it and f once.
-// Face fluxes per cell: 4 + 1/n_z + 1/(rows per segment), against 6 in
-// k_drift.  Integer sums do not depend on their order: the result is the
-// bits of k_drift.
-template <bool FORCE>
-__global__ void __launch_bounds__(PLANE_THREADS) k_drift_stream(const __grid_constant__ DriftArgs P, int nseg, float K)
-{
-    constexpr int D = BZ_DPIPE;
-    __shared__ float s_pf[3][MAX_NP];
-    extern __shared__ long long s_dyn[];  // y-face buffer [n_z][PLANE_THREADS], then the ring [D][2][PLANE_THREADS]
-    for (int d = 0; d < 3; ++d)
-        for (int i = threadIdx.x; i < P.np[d]; i += blockDim.x) s_pf[d][i] = P.pf[d][i];
-    __syncthreads();
-    const int npc = (int)P.npc;
-    const unsigned bj = BZ_PLANE_XFAST ? blockIdx.y : blockIdx.x, bs = BZ_PLANE_XFAST ? blockIdx.x : blockIdx.y;
-    const int j = bj * PLANE_THREADS + threadIdx.x;
-    if (j >= npc) return;
-    const int nx0 = P.nx[0], ny = P.nx[1], nz = P.nx[2];
-    const int seg = (int)(bs % (unsigned)nseg);
-    const int rest = (int)(bs / (unsigned)nseg);
-    const int ix = rest % nx0, sl = rest / nx0;
-    const int jp = __ldg(P.jtab + j);
-    const float p0 = s_pf[0][jp & 0xff], p1 = s_pf[1][(jp >> 8) & 0xff], p2 = s_pf[2][jp >> 16];
-    const float pp = (p0 * p0 + p1 * p1) + p2 * p2;
-    const bool sx = p0 > 0.0f, sy = p1 > 0.0f, sz = p2 > 0.0f;  // p_d > 0: the upwind neighbour is the lower one
-    const int ixu = sx ? (ix == 0 ? nx0 - 1 : ix - 1) : (ix == nx0 - 1 ? 0 : ix + 1);
-    const int64_t plane = (int64_t)ny * nz * P.npc;  // cells of one x index
-    const int64_t zs = P.npc;                         // cells between z neighbours
-    const int64_t b_own = (int64_t)sl * P.nxc * P.npc + (int64_t)ix * plane + j;
-    const int64_t dup = (int64_t)(ixu - ix) * plane;  // to the x-upwind cell
-    const int ms = P.slot_mslot[sl];
-    const float* m2f = P.m2f + ms;                    // [x * 4]
-    const int xo = ix * ny * nz, xuo = ixu * ny * nz;   // x cell = (ix n_y + iy) n_z + iz
-    const long long* in = P.in;
-    long long* fy = s_dyn + threadIdx.x;
-    long long* ring = s_dyn + (size_t)nz * PLANE_THREADS + threadIdx.x;
-    const bool mx = nx0 > 1, my = ny > 1, mz = nz > 1;
-    const int t0 = (int)((int64_t)seg * ny / nseg), t1 = (int)((int64_t)(seg + 1) * ny / nseg);
-    const int W = mz ? 1 : 0, per_row = nz + W, nr = t1 - t0;
-    if (my) {  // y-face fluxes of the row upwind of the segment's first row
-        const int tw = t0 == 0 ? ny - 1 : t0 - 1;
-        const int iy = sy ? tw : ny - 1 - tw;
-        const int64_t rw = b_own + (int64_t)iy * nz * zs;
-        for (int iz = 0; iz < nz; ++iz) {
-            const int xw = xo + iy * nz + iz;
-            const int64_t ow = rw + iz * zs;
-            if (!(bz_in(xw, P.nxc) & bz_in(ow, P.ncell))) continue;
-            const float inv = 1.0f / sqrtf(pp + __ldg(m2f + xw * 4));
-            fy[iz * PLANE_THREADS] = flux_n(__ldg(in + ow), courant_cvt(p1, inv, K));
-        }
+// Sum of rounded fluxes sum_i +-((n_i C_i + half_i) >> 30), 0 <= C_i: with n = nh
+// 2^32 + nl (nl unsigned) each is 4 nh C + s, s = (nl C + half) >> 30; the first
+// parts add up in one wide multiply-accumulate each, and where C < 2^30 (UNIT:
+// dt/dx < 0.999) s is the high word of nl (4 C) + 4 half, so that a flux takes two
+// wide multiplications and an add.  The low 64 bits are those of the exact sum.
+template <bool UNIT>
+struct FluxSum {
+    long long hi = 0;
+    unsigned long long lo = 0;
+    __device__ __forceinline__ static unsigned long long low(unsigned nl, unsigned C, unsigned half)
+    {
+        if (UNIT) return ((unsigned long long)nl * (4u * C) + 4ull * half) >> 32;
+        return ((unsigned long long)nl * C + half) >> 30;
     }
-    // item i of a row: i < W the wrap cell, else the (i - W)-th cell in upwind order
-    int pr = 0, pi = 0, ps = 0;  // next item to copy and its ring slot
-    auto issue = [&]() {
-        if (pr < nr) {
-            const int iy = sy ? t0 + pr : ny - 1 - t0 - pr;
-            int k = pi - W;
-            const bool wrap = k < 0;
-            if (wrap) k = nz - 1;
-            const int iz = sz ? k : nz - 1 - k;
-            const int64_t o = b_own + ((int64_t)iy * nz + iz) * zs;
-            if (bz_in(o, P.ncell)) cp_async8(ring + (2 * ps) * PLANE_THREADS, in + o);
-            if (mx && !wrap && bz_in(o + dup, P.ncell)) cp_async8(ring + (2 * ps + 1) * PLANE_THREADS, in + o + dup);
-            if (++pi == per_row) {
-                pi = 0;
-                ++pr;
-            }
-        }
-        cp_async_commit();
-        ps = ps + 1 == D ? 0 : ps + 1;
-    };
+    __device__ __forceinline__ void in(long long n, unsigned C, unsigned half)
+    {
+        hi += (long long)(int)(n >> 32) * (int)C;
+        lo += low((unsigned)n, C, half);
+    }
+    __device__ __forceinline__ void out(long long n, unsigned C, unsigned half)
+    {
+        hi += (long long)(int)(n >> 32) * -(int)C;
+        lo -= low((unsigned)n, C, half);
+    }
+};
+
+template <bool FORCE, bool UNIT>
+__global__ void __launch_bounds__(32 * DOCT_WARPS, FORCE ? 5 : DRIFT_MINB) k_drift_mirror(const __grid_constant__ DriftArgs P, int nseg, float K)
+{
+    const int lane = threadIdx.x & 31, warp = (int)__reduce_or_sync(0xffffffffu, threadIdx.x >> 5);  // uniform registers
+    const int n1 = P.np[1], n2 = P.np[2];
+    const int t = blockIdx.y * 32 + lane;
+    const bool in_range = t < P.half[0] * P.half[1] * n2;
+    const int hxy = (int)udiv((uint32_t)(in_range ? t : 0), P.dv_n2), z = (in_range ? t : 0) - hxy * n2;
+    const int hx = (int)udiv((uint32_t)hxy, P.dv_h1), hy = hxy - hx * P.half[1];
+    const int ux = P.np[0] - 1 - hx, uy = n1 - 1 - hy;
+    const unsigned oct = (unsigned)((hx * P.half[1] + hy) * P.half[2] + min(z, n2 - 1 - z));
+    const int nx0 = P.nx[0], ny = P.nx[1], nz = P.nx[2];
+    const int seg = (int)(blockIdx.x % (unsigned)nseg), rest = (int)(blockIdx.x / (unsigned)nseg);
+    const int ix = rest % nx0, sl = rest / nx0;
+    // |p_x|, |p_y|, |p_z| times K's power of two is folded in K; p_z > 0: moves up, fed from below
+    const float pax = P.pf[0][ux], pay = P.pf[1][uy], paz = fabsf(P.pf[2][z]);
+    const bool zup = P.pf[2][z] > 0.0f;
+    constexpr unsigned HUP = 1u << 29, HDN = (1u << 29) - 1u;
+    const unsigned zhalf = zup ? HUP : HDN;
+    // the cells, bit 0: upper along x, bit 1: upper along y; a mirror plane's cell is its lower one
+    const unsigned off[4] = {(unsigned)((hx * n1 + hy) * n2 + z), (unsigned)((ux * n1 + hy) * n2 + z),
+                             (unsigned)((hx * n1 + uy) * n2 + z), (unsigned)((ux * n1 + uy) * n2 + z)};
+    const bool live[4] = {in_range, in_range && ux != hx, in_range && uy != hy, in_range && ux != hx && uy != hy};
+    unsigned off8[4];  // byte offsets inside a row of the state
 #pragma unroll
-    for (int q = 0; q < D - 1; ++q) issue();
-    long long fz_up = 0;  // z flux of the previous cell of the walk (the upwind one)
-    int cr = 0, ci = 0, cs = 0;
-#pragma unroll 1
-    for (int g = 0, G = nr * per_row; g < G; ++g) {
-        issue();
-        cp_async_wait<D - 1>();
-        const long long n = ring[(2 * cs) * PLANE_THREADS];
-        const int iy = sy ? t0 + cr : ny - 1 - t0 - cr;
-        int k = ci - W;
-        const bool wrap = k < 0;
-        if (wrap) k = nz - 1;
-        const int iz = sz ? k : nz - 1 - k;
-        const int xr = iy * nz + iz;
-        const float m = bz_in(xo + xr, P.nxc) ? __ldg(m2f + (xo + xr) * 4) : 0.0f;
-        const float inv = 1.0f / sqrtf(pp + m);
-        if (wrap) {
-            fz_up = flux_n(n, courant_cvt(p2, inv, K));
-        } else {
-            long long acc = 0;
-            // p_d > 0: outflow through the upper face, inflow from below; else the mirror
-            if (mz) {
-                const long long f2 = flux_n(n, courant_cvt(p2, inv, K));
-                acc += sz ? f2 - fz_up : fz_up - f2;
-                fz_up = f2;
+    for (int k = 0; k < 4; ++k) off8[k] = off[k] * 8u;
+    const unsigned oct4 = oct * 4u;
+    // byte distances between rows of the state; rows of the 1/E table are row_e bytes
+    const int64_t row_n = P.npc * 8, row_e = (int64_t)P.noct * 4;
+    const int64_t dxlo = (int64_t)(ix == 0 ? nx0 - 1 : -1) * ny * nz, dxup = (int64_t)(ix == nx0 - 1 ? 1 - nx0 : 1) * ny * nz;
+    const int y0 = (int)((int64_t)seg * ny / nseg), y1 = (int)((int64_t)(seg + 1) * ny / nseg);
+    const bool zsplit = nz >= DOCT_WARPS;  // the warps share the z cells of a row, or the rows
+    const int64_t rows = P.ncell / P.npc;
+    for (int iy = y0 + (zsplit ? 0 : warp); iy < y1; iy += zsplit ? 1 : DOCT_WARPS) {
+        const int64_t r0 = (int64_t)sl * P.nxc + ((int64_t)ix * ny + iy) * nz;  // row of (ix, iy, 0)
+        const int64_t dylo = (int64_t)(iy == 0 ? ny - 1 : -1) * nz, dyup = (int64_t)(iy == ny - 1 ? 1 - ny : 1) * nz;
+        const int iz0 = zsplit ? warp : 0, dz = zsplit ? DOCT_WARPS : 1;
+        const char* pn = reinterpret_cast<const char*>(P.in) + (r0 + iz0) * row_n;
+        const char* pe = reinterpret_cast<const char*>(P.inv_e) + (r0 + iz0) * row_e;
+        int64_t po = (r0 + iz0) * row_n;
+        for (int iz = iz0; iz < nz; iz += dz, pn += dz * row_n, pe += dz * row_e, po += dz * row_n) {
+            const int64_t dzlo = iz == 0 ? nz - 1 : -1, dzhi = iz == nz - 1 ? 1 - nz : 1;
+            const int64_t x = r0 + iz;
+            if (!(bz_in(x, rows) & bz_in(x + dxlo, rows) & bz_in(x + dxup, rows) & bz_in(x + dylo, rows) &
+                  bz_in(x + dyup, rows) & bz_in(x + dzlo, rows) & bz_in(x + dzhi, rows) & bz_in(off[3], P.npc) &
+                  bz_in(oct, P.noct)))
+                continue;
+            auto at = [](const char* row, unsigned o) { return __ldg(reinterpret_cast<const long long*>(row + o)); };
+            auto ie = [&](const char* row) { return __ldg(reinterpret_cast<const float*>(row + oct4)); };
+            const char *xl = pn + dxlo * row_n, *xu = pn + dxup * row_n, *yl = pn + dylo * row_n, *yu = pn + dyup * row_n;
+            const char* zn = pn + (zup ? dzlo : dzhi) * row_n;
+            long long n[4], bx[4], by[4], bz[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                n[k] = live[k] ? at(pn, off8[k]) : 0;
+                bx[k] = live[k] && nx0 > 1 ? at(k & 1 ? xl : xu, off8[k]) : 0;
+                by[k] = live[k] && ny > 1 ? at(k & 2 ? yl : yu, off8[k]) : 0;
+                bz[k] = live[k] && nz > 1 ? at(zn, off8[k]) : 0;
             }
-            if (my) {
-                const long long f1 = flux_n(n, courant_cvt(p1, inv, K));
-                const long long fu = fy[iz * PLANE_THREADS];
-                acc += sy ? f1 - fu : fu - f1;
-                fy[iz * PLANE_THREADS] = f1;
+            const float inv = ie(pe);
+            auto courant = [&](float pa, float e) { return (unsigned)__float2int_rn((pa * e) * K); };  // rint((|p| / E) dt/dx 2^30)
+            FluxSum<UNIT> f[4];
+            if (nx0 > 1) {
+                const unsigned C = courant(pax, inv), Clo = courant(pax, ie(pe + dxlo * row_e)), Cup = courant(pax, ie(pe + dxup * row_e));
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    f[k].in(bx[k], k & 1 ? Clo : Cup, k & 1 ? HUP : HDN);
+                    f[k].out(n[k], C, k & 1 ? HUP : HDN);
+                }
             }
-            if (mx) {
-                const long long nu = ring[(2 * cs + 1) * PLANE_THREADS];
-                const float invu = 1.0f / sqrtf(pp + (bz_in(xuo + xr, P.nxc) ? __ldg(m2f + (xuo + xr) * 4) : 0.0f));
-                const long long f0 = flux_n(n, courant_cvt(p0, inv, K));
-                const long long fu = flux_n(nu, courant_cvt(p0, invu, K));
-                acc += sx ? f0 - fu : fu - f0;
+            if (ny > 1) {
+                const unsigned C = courant(pay, inv), Clo = courant(pay, ie(pe + dylo * row_e)), Cup = courant(pay, ie(pe + dyup * row_e));
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    f[k].in(by[k], k & 2 ? Clo : Cup, k & 2 ? HUP : HDN);
+                    f[k].out(n[k], C, k & 2 ? HUP : HDN);
+                }
             }
-            const int64_t oc = b_own + (int64_t)xr * zs;
-            if (bz_in(oc, P.ncell) & bz_in(xo + xr, P.nxc)) {
-                if (FORCE)
-                    acc += force_acc_inline(P, P.gforce + ((int64_t)(xo + xr) * 4 + ms) * 3, jp, j, in + (oc - j), n,
-                                            inv, s_pf, m);
-                P.out[oc] = n - acc;
+            if (nz > 1) {
+                const unsigned C = courant(paz, inv), Cn = courant(paz, ie(pe + (zup ? dzlo : dzhi) * row_e));
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    f[k].in(bz[k], Cn, zhalf);
+                    f[k].out(n[k], C, zhalf);
+                }
+            }
+            // force term: along p_i all cells of the x cell move with -g_i / E; own outflow and
+            // inflow from the cell behind, each through a face inside the box, as the x fluxes
+            FluxSum<false> ff[4];
+            bool wide = false;  // a Courant number of 2 or more: by force_acc_octet below
+            const float* const g3 = FORCE ? P.gforce + ((x - (int64_t)sl * P.nxc) * 4 + P.slot_mslot[sl]) * 3 : nullptr;
+            if (FORCE) {
+                const int hv[3] = {hx, hy, min(z, n2 - 1 - z)}, os[3] = {P.half[1] * P.half[2], P.half[2], 1}, js[3] = {n1 * n2, n2, 1};
+                const int nx[3] = {nx0, ny, nz};
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    if (nx[i] == 1) continue;
+                    const float g = __ldg(g3 + i);
+                    const bool up = (-g) > 0.0f;
+                    const unsigned half = up ? HUP : HDN;
+                    // 1/E one half-grid step outwards and inwards (the cells behind are at either)
+                    const float* e0 = reinterpret_cast<const float*>(pe) + oct;
+                    const float eo = hv[i] > 0 ? __ldg(e0 - os[i]) : inv;
+                    const int in = min(hv[i] + 1, P.np[i] - 2 - hv[i]);
+                    const float ei = in >= 0 ? __ldg(e0 + (in - hv[i]) * os[i]) : inv;
+                    const float w = ((-g) * inv) * P.Kp[i], wo = ((-g) * eo) * P.Kp[i], wi = ((-g) * ei) * P.Kp[i];
+                    wide |= !(fabsf(w) < 2147483648.0f) | !(fabsf(wo) < 2147483648.0f) | !(fabsf(wi) < 2147483648.0f);
+                    const unsigned C = (unsigned)__float2int_rn(fabsf(w)), Co = (unsigned)__float2int_rn(fabsf(wo));
+                    const unsigned Ci = (unsigned)__float2int_rn(fabsf(wi));
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int j = i == 0 ? (k & 1 ? ux : hx) : (i == 1 ? (k & 2 ? uy : hy) : z);
+                        const int jo = up ? j + 1 : j - 1, jb = up ? j - 1 : j + 1;
+                        if (live[k] && jo >= 0 && jo < P.np[i]) ff[k].out(n[k], C, half);
+                        if (live[k] && jb >= 0 && jb < P.np[i]) {
+                            const long long nb = at(pn, off8[k] + (unsigned)((jb - j) * js[i]) * 8u);
+                            ff[k].in(nb, min(jb, P.np[i] - 1 - jb) < hv[i] ? Co : (min(jb, P.np[i] - 1 - jb) == hv[i] ? C : Ci), half);
+                        }
+                    }
+                }
+            }
+            char* const out = reinterpret_cast<char*>(P.out) + po;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (!live[k]) continue;
+                long long r = (long long)((unsigned long long)n[k] + 4ull * (unsigned long long)f[k].hi + f[k].lo);
+                if (FORCE) {
+                    const int jv[3] = {k & 1 ? ux : hx, k & 2 ? uy : hy, z};
+                    if (!wide)
+                        r += (long long)(4ull * (unsigned long long)ff[k].hi + ff[k].lo);
+                    else
+                        r -= force_acc_octet(P, g3, jv, (int)off[k], reinterpret_cast<const long long*>(pn),
+                                             reinterpret_cast<const float*>(pe), n[k], inv);
+                }
+                *reinterpret_cast<long long*>(out + off8[k]) = r;
                 if (P.freal) {
                     if (P.freal_double)
-                        static_cast<double*>(P.freal)[oc] = (double)n * TWO_POW_M40 / P.deg[sl];
+                        *reinterpret_cast<double*>(static_cast<char*>(P.freal) + po + off8[k]) = (double)n[k] * TWO_POW_M40 / P.deg[sl];
                     else
-                        static_cast<float*>(P.freal)[oc] =
-                            (BZ_HW_CVT ? __ll2float_rn(n) : ll2float_rn(n)) * P.fscale[sl];
+                        *reinterpret_cast<float*>(static_cast<char*>(P.freal) + (po >> 1) + (off8[k] >> 1)) =
+                            ll2float_fast(n[k]) * P.fscale[sl];
                 }
             }
         }
-        if (++ci == per_row) {
-            ci = 0;
-            ++cr;
-        }
-        cs = cs + 1 == D ? 0 : cs + 1;
     }
-    cp_async_wait<0>();
 }
 
 static int device_sms()
@@ -905,32 +942,31 @@ cudaError_t launch_drift(const DriftArgs& a, cudaStream_t s)
     const int64_t tiles = (a.npc + DRIFT_TILE - 1) / DRIFT_TILE;
     if (rows < 1 || rows > 2147483647LL || tiles > 65535) return cudaErrorInvalidConfiguration;
     const bool moving = a.nx[0] > 1 || a.nx[1] > 1 || a.nx[2] > 1;
-    if (moving && !(a.inv_e && a.m2f)) return cudaErrorInvalidValue;  // scratch of the moving forms
+    if (moving && !a.inv_e) return cudaErrorInvalidValue;  // scratch of the moving forms
     if (a.force && !(a.gforce && moving)) return cudaErrorInvalidValue;
     if (a.force) k_force_grad<<<(unsigned)((a.nxc * 4 + 127) / 128), 128, 0, s>>>(a);
     const int64_t nslots = rows / a.nxc;
-    if (moving && a.dtdxf < 1.99f && a.nx[2] <= PLANE_MAX_NZ) {
-        // y segments: enough threads for every SM at full occupancy
-        const int64_t base = nslots * a.nx[0] * a.npc;
-        int64_t nseg = ((int64_t)device_sms() * BZ_PLANE_THREADS_PER_SM + base - 1) / base;
+    // |C| <= 2^30 dt/dx < 2^31, mirrored cells: by octets; else (long time steps, cell
+    // centres that are no exact mirror images in FP32) by rows.  16^3 x 20^3 gluons: 359 -> 273 us without f
+    // (some 205 instructions a cell, multiplications and addresses the largest parts), 842 -> 693 us with the force
+    if (moving && a.dtdxf < 1.99f && a.noct > 0) {
+        const int64_t tiles_m = ((int64_t)a.half[0] * a.half[1] * a.np[2] + 31) / 32, base = nslots * a.nx[0] * tiles_m;
+        int64_t nseg = ((int64_t)device_sms() * 8 + base - 1) / base;  // y segments: 8 blocks per SM
         nseg = nseg < 1 ? 1 : (nseg > a.nx[1] ? a.nx[1] : nseg);
-        const int64_t gs = nslots * a.nx[0] * nseg, gj = (a.npc + PLANE_THREADS - 1) / PLANE_THREADS;
-        const int64_t gx = BZ_PLANE_XFAST ? gs : gj, gy = BZ_PLANE_XFAST ? gj : gs;
-        if (gy <= 65535 && gx <= 2147483647LL) {
-            const size_t smem = sizeof(long long) * PLANE_THREADS * ((size_t)a.nx[2] + 2 * BZ_DPIPE);
-            if (smem > 48 * 1024) {
-                const cudaError_t e =
-                    a.force ? cudaFuncSetAttribute(k_drift_stream<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                            : cudaFuncSetAttribute(k_drift_stream<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return e;
-            }
-            const dim3 grid((unsigned)gx, (unsigned)gy);
+        const int64_t gx = nslots * a.nx[0] * nseg;
+        if (tiles_m <= 65535 && gx <= 2147483647LL) {
+            k_inv_octet<<<(unsigned)rows, 256, 0, s>>>(a);
+            const dim3 grid((unsigned)gx, (unsigned)tiles_m);
             const float K = a.dtdxf * 1073741824.0f;
-            k_mass_table<<<(unsigned)((a.nxc * 4 + 255) / 256), 256, 0, s>>>(a);
-            if (a.force)
-                k_drift_stream<true><<<grid, PLANE_THREADS, smem, s>>>(a, (int)nseg, K);
+            const bool unit = a.dtdxf < 0.999f;  // C < 2^30
+            if (a.force && unit)
+                k_drift_mirror<true, true><<<grid, 32 * DOCT_WARPS, 0, s>>>(a, (int)nseg, K);
+            else if (a.force)
+                k_drift_mirror<true, false><<<grid, 32 * DOCT_WARPS, 0, s>>>(a, (int)nseg, K);
+            else if (unit)
+                k_drift_mirror<false, true><<<grid, 32 * DOCT_WARPS, 0, s>>>(a, (int)nseg, K);
             else
-                k_drift_stream<false><<<grid, PLANE_THREADS, smem, s>>>(a, (int)nseg, K);
+                k_drift_mirror<false, false><<<grid, 32 * DOCT_WARPS, 0, s>>>(a, (int)nseg, K);
             return cudaGetLastError();
         }
     }
@@ -1043,14 +1079,6 @@ struct Octet {
     int h[3];
     unsigned hi;  // the high words, or-ed
 };
-template <typename Args>
-__device__ __forceinline__ void octet_index(const Args& P, int o, int h[3])
-{
-    h[0] = (int)udiv((uint32_t)o, P.dv_h12);
-    const int r = o - h[0] * (P.half[1] * P.half[2]);
-    h[1] = (int)udiv((uint32_t)r, P.dv_h2);
-    h[2] = r - h[1] * P.half[2];
-}
 __device__ __forceinline__ void load_octet(const MomentArgs& P, const long long* st, int o, Octet& q)
 {
     octet_index(P, o, q.h);
