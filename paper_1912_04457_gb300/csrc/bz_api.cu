@@ -19,6 +19,8 @@
 
 using namespace bz;
 
+constexpr int LOSS_CAP = 4096;
+
 struct bz_handle_s {
     bz_grid g{};
     int device = 0;
@@ -60,9 +62,10 @@ struct bz_handle_s {
     unsigned long long* d_qitems = nullptr;
     int64_t q_warps = 0, q_items = 0;
     // learned proposal: FP32 master parameters, Adam moments, gradient, per-anchor parameters
-    float *d_prop = nullptr, *d_prop_g = nullptr, *d_prop_m = nullptr, *d_prop_v = nullptr;
+    float *d_prop = nullptr, *d_prop_m = nullptr, *d_prop_v = nullptr;
     float* d_anchor_prm = nullptr;
     float* d_loss = nullptr;
+    float* d_losses = nullptr;         // [LOSS_CAP] losses of a training call's steps
     double* d_wsum = nullptr;          // [sum_weights_scratch()]: the sum, then the per-warp partial sums
     float* d_prop_part = nullptr;      // per-block gradients [4 nsm][nparam] and losses [4 nsm]
     float* d_loss_part = nullptr;
@@ -220,11 +223,12 @@ static void free_scratch(bz_handle h)
     cudaFree(h->d_qcount);
     cudaFree(h->d_qitems);
     cudaFree(h->d_prop);
-    cudaFree(h->d_prop_g);
     cudaFree(h->d_prop_m);
     cudaFree(h->d_prop_v);
     cudaFree(h->d_anchor_prm);
     cudaFree(h->d_loss);
+    cudaFree(h->d_losses);
+    h->d_losses = nullptr;
     cudaFree(h->d_wsum);
     cudaFree(h->d_prop_part);
     cudaFree(h->d_loss_part);
@@ -233,7 +237,7 @@ static void free_scratch(bz_handle h)
     h->d_prop_err = nullptr;
     cudaFree(h->d_rec_count);
     h->d_rec_count = nullptr;
-    h->d_prop = h->d_prop_g = h->d_prop_m = h->d_prop_v = h->d_anchor_prm = h->d_loss = nullptr;
+    h->d_prop = h->d_prop_m = h->d_prop_v = h->d_anchor_prm = h->d_loss = nullptr;
     h->d_wsum = nullptr;
     h->d_qcount = nullptr;
     h->d_qitems = nullptr;
@@ -1754,12 +1758,11 @@ static int prop_alloc(bz_handle h)
 {
     const int n = mlp_nparam();
     if (h->d_prop) return BZ_OK;
-    if (!dalloc(&h->d_prop, n) || !dalloc(&h->d_prop_g, n) || !dalloc(&h->d_prop_m, n) ||
+    if (!dalloc(&h->d_prop, n) || !dalloc(&h->d_losses, LOSS_CAP) || !dalloc(&h->d_prop_m, n) ||
         !dalloc(&h->d_prop_v, n) || !dalloc(&h->d_loss, 1) || !dalloc(&h->d_wsum, sum_weights_scratch()) ||
         !dalloc(&h->d_prop_part, (size_t)4 * h->nsm * n) || !dalloc(&h->d_loss_part, (size_t)4 * h->nsm) ||
         !dalloc(&h->d_prop_err, 1))
         return fail(h, BZ_ENOMEM, "cannot allocate the proposal network");
-    CK(h, cudaMemset(h->d_prop_g, 0, sizeof(float) * n));
     CK(h, cudaMemset(h->d_prop_m, 0, sizeof(float) * n));
     CK(h, cudaMemset(h->d_prop_v, 0, sizeof(float) * n));
     return BZ_OK;
@@ -1868,18 +1871,23 @@ extern "C" int bz_proposal_train(bz_handle h, const void* records, int64_t n, in
     if (!(wsum > 0)) return fail(h, BZ_EINVAL, "records carry no weight");
     const double wbar = wsum / (double)n;
     const ProposalArgs A = prop_args(h);
-    const int np = mlp_nparam();
-    CK(h, cudaMemsetAsync(h->d_prop_g, 0, sizeof(float) * np, s));
     // each step's minibatch: b records drawn independently and uniformly from all n
-    // (the record buffer is in arrival order, i.e. clustered by anchor)
+    // (the record buffer is in arrival order, i.e. clustered by anchor); the losses
+    // stay on the device, up to LOSS_CAP of them, until the steps are enqueued (a copy
+    // to pageable memory per step would wait for it)
     CK(h, cudaMemsetAsync(h->d_prop_err, 0, sizeof(int), s));
-    for (int k = 0; k < steps; ++k) {
-        const int64_t b = batch;
-        const uint64_t key = ((uint64_t)(h->adam_step + 1) << 32) * 0x9E3779B97F4A7C15ull;
-        CK(h, launch_mlp_grad(h->d_prop, A, rec, b, (float)(1.0 / (wbar * (double)b)), h->d_prop_g, h->d_loss, h->nsm,
-                              h->d_prop_part, h->d_loss_part, h->d_prop_err, s, n, key));
-        CK(h, launch_adam(h->d_prop, h->d_prop_g, h->d_prop_m, h->d_prop_v, np, (float)lr, ++h->adam_step, s));
-        if (losses_host) CK(h, cudaMemcpyAsync(&losses_host[k], h->d_loss, sizeof(float), cudaMemcpyDeviceToHost, s));
+    for (int k0 = 0; k0 < steps; k0 += LOSS_CAP) {
+        const int kn = std::min(steps - k0, LOSS_CAP);
+        for (int k = 0; k < kn; ++k) {
+            const int64_t b = batch;
+            const uint64_t key = ((uint64_t)(h->adam_step + 1) << 32) * 0x9E3779B97F4A7C15ull;
+            CK(h, launch_mlp_grad(h->d_prop, A, rec, b, (float)(1.0 / (wbar * (double)b)), nullptr,
+                                  losses_host ? h->d_losses + k : h->d_loss, h->nsm, h->d_prop_part, h->d_loss_part, h->d_prop_err,
+                                  s, n, key, h->d_prop, h->d_prop_m, h->d_prop_v, (float)lr, h->adam_step + 1, k > 0));
+            ++h->adam_step;
+        }
+        if (losses_host)
+            CK(h, cudaMemcpyAsync(losses_host + k0, h->d_losses, sizeof(float) * kn, cudaMemcpyDeviceToHost, s));
     }
     int herr = 0;
     CK(h, cudaMemcpyAsync(&herr, h->d_prop_err, sizeof(int), cudaMemcpyDeviceToHost, s));

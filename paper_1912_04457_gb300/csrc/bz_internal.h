@@ -359,10 +359,12 @@ int mlp_nparam();
 // part [grid][nparam], part_loss [grid]: per-block scratch, added in block order into grad (+=) and loss (=);
 // err (device int): incremented by a block whose tensor-core wait timed out.  At most `grid` blocks, one
 // per SM (each holds 512 columns of tensor memory).
+// p set: the gradient is taken as step `step` of Adam on the parameters p with moments m, v instead of added to grad.
+// chained: the launch before this one on s is the update of such a step, and nothing since has written rec.
 cudaError_t launch_mlp_grad(const float* params, const ProposalArgs& A, const ProposalRecord* rec, int64_t n,
                             float inv_wsum, float* grad, float* loss, int grid, float* part, float* part_loss, int* err,
-                            cudaStream_t s, int64_t ntot = 0, uint64_t key = 0);
-cudaError_t launch_adam(float* p, float* g, float* m, float* v, int n, float lr, int step, cudaStream_t s);
+                            cudaStream_t s, int64_t ntot = 0, uint64_t key = 0, float* p = nullptr, float* m = nullptr,
+                            float* v = nullptr, float lr = 0.0f, int step = 0, bool chained = false);
 // err (device int, zeroed by the caller): incremented by a CTA whose tensor-core wait timed out
 cudaError_t launch_mlp_infer(const float* params, const ProposalArgs& A, int64_t nanchor, float* out, int grid,
                              int* err, cudaStream_t s);

@@ -1,0 +1,68 @@
+"""Proposal network at the edges of its work split: chunks of 128 records over at
+most one block per SM, tiles of 128 anchors, updates chained on one stream."""
+import numpy as np
+import pytest
+
+from oracle import mlp
+
+pytestmark = pytest.mark.gpu
+
+REC = np.dtype([("a", "<i8"), ("w", "<f4"), ("y", "<f4", (5,))])
+
+
+def _records(n, na, seed):
+    import torch
+    rng = np.random.default_rng(seed)
+    r = np.zeros(n, dtype=REC)
+    r["a"], r["w"], r["y"] = rng.integers(0, na, n), rng.uniform(0.1, 2.0, n), rng.uniform(-1, 1, (n, 5))
+    return r, torch.from_numpy(r.view(np.uint8).copy()).cuda()
+
+
+def _rel(a, b):
+    return float(np.linalg.norm(np.asarray(a, float) - np.asarray(b, float)) / np.linalg.norm(np.asarray(b, float)))
+
+
+@pytest.mark.parametrize("n", [1, 127, 129, 128 * 8 + 1, 128 * 152, 128 * 152 + 1, 128 * 400 + 77])
+def test_gradient(n):
+    from paper_1912_04457_gb300 import bz
+    np_ = (6, 6, 6)
+    h = bz.Handle(np_=np_, L=2.0, species_mask=0x7F)
+    params = mlp.init_params(7)
+    h.set_proposal_params(params)
+    r, dev = _records(n, 7 * 216, n)
+    grad, loss = h.proposal_grad(dev, n)
+    X = mlp.features(r["a"], np_, 2.0, 1, list(range(7)))
+    lo, go = mlp.loss_grad(params.astype(np.float64), X, r["y"].astype(np.float64), r["w"].astype(np.float64), bf=True)
+    # a rounding to BF16 that falls the other way moves an activation by 2^-8; over n records the
+    # gradients of such roundings add as random signs: the bar of 1e-3 holds for 1000 records
+    assert _rel(grad.cpu().numpy(), go) <= max(1e-3, 1e-3 * (1000 / n) ** 0.5)
+    assert float(loss.item()) == pytest.approx(lo, rel=1e-4 if n > 100 else 1e-3)
+
+
+@pytest.mark.parametrize("batch", [100, 16384, 40000])
+def test_chained_steps_equal_single_steps(batch):
+    from paper_1912_04457_gb300 import bz
+    out = []
+    _, dev = _records(30000, 7 * 216, 5)
+    for calls in ([6], [1] * 6):
+        h = bz.Handle(np_=(6, 6, 6), L=2.0, species_mask=0x7F)
+        h.set_proposal_params(mlp.init_params(7))
+        losses = np.concatenate([h.proposal_train(dev, 30000, k, batch, 1e-3) for k in calls])
+        out.append((losses, h.proposal_params()))
+    assert np.array_equal(out[0][0], out[1][0])
+    assert np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("np_,mask", [((1, 1, 2), 1), ((4, 4, 8), 1), ((3, 43, 2), 1), ((20, 20, 20), 0x7F)])
+def test_inference(np_, mask):
+    from paper_1912_04457_gb300 import bz
+    h = bz.Handle(np_=np_, L=2.0, species_mask=mask)
+    params = mlp.init_params(11)
+    h.set_proposal_params(params)
+    h.proposal_infer()
+    got = h.anchor_params()
+    a = np.arange(h.ncell)
+    X = mlp.features(a, np_, 2.0, 1, [0] if mask == 1 else list(range(7)))
+    O_, _ = mlp.forward(params.astype(np.float64), X)
+    ref = mlp.head(O_[:, :6])
+    assert np.abs(got[:, :6] - ref[:, :6]).max() < 5e-3
