@@ -293,7 +293,7 @@ cudaError_t launch_sum_ll(const long long* a, int64_t n, long long* out, cudaStr
 cudaError_t launch_collide_f32(const CollideArgs<float>& a, int grid, unsigned long long* counter, cudaStream_t s);
 int collide_f32_resident_blocks(const CollideArgs<float>& a);  // per SM, for the instantiation `a` runs
 // FP32 path, uniform sampler: re-evaluation of the queued terms with an FP64
-// root solve (one warp per queue segment)
+// root solve (nseg queue segments)
 cudaError_t launch_fixup_f32(const CollideArgs<float>& a, int nseg, cudaStream_t s);
 cudaError_t launch_fixup_f32_batch(const CollideArgs<float>* boxes, const int* qcount, const unsigned long long* qitems,
                                    int64_t qcap, const int* step_dev, int nseg, cudaStream_t s);

@@ -46,8 +46,11 @@ constexpr int RING = 128;         // pending roots per warp (power of 2)
 // 14.7 with 128; 7 species, 32^3: 15.5 and 17.5).
 template <bool GROUPS> constexpr int SLOTS = GROUPS ? 64 : 128;
 constexpr int WARPS = F32_WARPS;  // warps per block
-#ifndef BZ_FIX_SPLIT_MAX
-#define BZ_FIX_SPLIT_MAX 8  // most warps sharing one queue segment
+#ifndef BZ_FIX_GROUP
+#define BZ_FIX_GROUP 32  // queue segments read as one list, at most 32
+#endif
+#ifndef BZ_FIX_SLICES_MAX
+#define BZ_FIX_SLICES_MAX 32  // most blocks sharing one list
 #endif
 #ifndef BZ_FIX_MINB
 #define BZ_FIX_MINB 4  // resident blocks of 256 threads per SM the fixup's register budget is cut for (64 registers)
@@ -1205,24 +1208,61 @@ __device__ __noinline__ long long fixup_term_ff(const CollideArgs<float>& P, int
     return own;
 }
 
-// `split` warps per queue segment (the items of a segment are dealt over
-// their 32 split lanes).  The learned form gives each lane a contiguous run
-// of items, so that its cached per-anchor constants are reused.
+// The queue's segments (one per collision warp) hold from none to some hundred
+// items.  Groups of up to 32 neighbouring segments are read as one list (a scan
+// of their counts) dealt over `slices` blocks of 256 threads: with warps that
+// belong to one segment, segments of few items left most lanes idle and those of
+// uneven counts left some warps working alone (10 x 9 x 12 cells of 5 x 3 x 7 x cells:
+// 71 -> 43 us; 16^3, seven species, learned: 94 -> 76 us; a 20^3 gluon box's step
+// 61 -> 58 us).  What is left there is one term's chain of dependent operations.
+struct FixupGroup {
+    int pre[33];  // first item of each segment of the group in its list; [n] = all
+    int total;
+};
+__device__ __forceinline__ void fixup_group(FixupGroup& G, const int* qcount, int seg0, int n)
+{
+    if (threadIdx.x < 32) {
+        const int lane = (int)threadIdx.x;
+        const int c = lane < n ? qcount[seg0 + lane] : 0;
+        int t = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += u;
+        }
+        G.pre[lane] = t - c;
+        if (lane == 31) G.pre[32] = G.total = t;
+    }
+    __syncthreads();
+}
+// the item's segment within the group: the last one with pre <= i
+__device__ __forceinline__ int fixup_segment(const FixupGroup& G, int i)
+{
+    int lo = 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        if (G.pre[lo + o] <= i) lo += o;
+    return lo;
+}
+
+// The learned form gives each thread a contiguous run of items, so that its
+// cached per-anchor constants are reused.
 template <bool LEARNED>
 __global__ void __launch_bounds__(256, BZ_FIX_MINB) k_fixup_f32(const __grid_constant__ CollideArgs<float> P, const int* qcount,
-                                                   const unsigned long long* qitems, int64_t qcap, int nseg, int split)
+                                                                const unsigned long long* qitems, int64_t qcap, int nseg,
+                                                                int gsz, int slices)
 {
-    const int64_t gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int64_t seg = gw / split;
-    if (seg >= nseg) return;
-    const int n = qcount[seg];
-    const int slots = 32 * split, slot = (int)(gw - seg * split) * 32 + (threadIdx.x & 31);
+    __shared__ FixupGroup G;
+    const int seg0 = (int)(blockIdx.x / slices) * gsz, slot = (int)(blockIdx.x % slices) * 256 + (int)threadIdx.x;
+    fixup_group(G, qcount, seg0, min(gsz, nseg - seg0));
+    const int n = G.total, slots = 256 * slices;
     const int run = LEARNED ? (n + slots - 1) / slots : 1;
-    const int i0 = LEARNED ? slot * run : slot, i1 = LEARNED ? min(n, i0 + run) : n, di = LEARNED ? 1 : slots;
+    const int i0 = slot * run, i1 = LEARNED ? min(n, i0 + run) : n, di = LEARNED ? 1 : slots;
     PropCache pc;
     const int step = P.step_dev ? *P.step_dev : P.step;
     for (int i = i0; i < i1; i += di) {
-        const unsigned long long it = qitems[seg * qcap + i];
+        const int k = fixup_segment(G, i);
+        const unsigned long long it = qitems[(seg0 + k) * qcap + (i - G.pre[k])];
         const int64_t a = (int64_t)(it >> 24);
         const int smp = (int)((it >> 4) & 0xFFFFFu), ti = (int)(it & 0xFu);
         const long long own = fixup_term_ff<LEARNED>(P, a, smp, ti, step, pc);
@@ -1233,18 +1273,18 @@ __global__ void __launch_bounds__(256, BZ_FIX_MINB) k_fixup_f32(const __grid_con
 // Batch form: the item carries its box (bits 48..63); the step is read from
 // device memory.
 __global__ void __launch_bounds__(256, BZ_FIX_MINB) k_fixup_f32_batch(const CollideArgs<float>* __restrict__ boxes,
-                                                         const int* qcount, const unsigned long long* qitems,
-                                                         int64_t qcap, const int* step_dev, int nseg, int split)
+                                                                      const int* qcount, const unsigned long long* qitems,
+                                                                      int64_t qcap, const int* step_dev, int nseg, int gsz,
+                                                                      int slices)
 {
-    const int64_t gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int64_t seg = gw / split;
-    if (seg >= nseg) return;
-    const int n = qcount[seg];
-    const int slots = 32 * split, slot = (int)(gw - seg * split) * 32 + (threadIdx.x & 31);
+    __shared__ FixupGroup G;
+    const int seg0 = (int)(blockIdx.x / slices) * gsz, slot = (int)(blockIdx.x % slices) * 256 + (int)threadIdx.x;
+    fixup_group(G, qcount, seg0, min(gsz, nseg - seg0));
     const int step = *step_dev;
     PropCache pc;
-    for (int i = slot; i < n; i += slots) {
-        const unsigned long long it = qitems[seg * qcap + i];
+    for (int i = slot; i < G.total; i += 256 * slices) {
+        const int k = fixup_segment(G, i);
+        const unsigned long long it = qitems[(seg0 + k) * qcap + (i - G.pre[k])];
         const CollideArgs<float>& P = boxes[(int)(it >> 48)];
         const int64_t a = (int64_t)((it >> 24) & 0xFFFFFFull);
         const long long own = fixup_term_ff<false>(P, a, (int)((it >> 4) & 0xFFFFFu), (int)(it & 0xFu), step, pc);
@@ -1252,9 +1292,9 @@ __global__ void __launch_bounds__(256, BZ_FIX_MINB) k_fixup_f32_batch(const Coll
     }
 }
 
-// Warps per queue segment: enough warps for about two full waves of the
-// fixup's resident warps (BZ_FIX_MINB blocks of 8 warps per SM).
-static int fixup_split(int nseg)
+// Blocks per group of segments: enough for about two full waves of the fixup's
+// resident blocks (BZ_FIX_MINB per SM); blocks beyond a short list end at once.
+static int fixup_slices(int ngroups)
 {
     static int nsm = 0;
     if (!nsm) {
@@ -1263,32 +1303,33 @@ static int fixup_split(int nseg)
                                                       cudaSuccess || nsm < 1)
             nsm = 1;
     }
-    const int64_t want = 2ll * nsm * BZ_FIX_MINB * 8;
-    const int64_t sp = (want + nseg - 1) / (nseg > 0 ? nseg : 1);
-    return (int)(sp < 1 ? 1 : (sp > BZ_FIX_SPLIT_MAX ? BZ_FIX_SPLIT_MAX : sp));
+    const int64_t want = 2ll * nsm * BZ_FIX_MINB;
+    const int64_t sl = (want + ngroups - 1) / (ngroups > 0 ? ngroups : 1);
+    return (int)(sl < 1 ? 1 : (sl > BZ_FIX_SLICES_MAX ? BZ_FIX_SLICES_MAX : sl));
 }
 
 cudaError_t launch_fixup_f32(const CollideArgs<float>& a, int nseg, cudaStream_t s)
 {
-    // the learned form keeps one warp per segment: longer runs per lane reuse
-    // its cached per-anchor constants more (measured: split 3 was 3% slower)
-    const int split = a.sampler == SAMPLER_LEARNED ? 1 : fixup_split(nseg);
-    const unsigned grid = (unsigned)(((int64_t)nseg * split + 7) / 8);
-    if (a.sampler == SAMPLER_LEARNED)
-        k_fixup_f32<true><<<grid, 256, 0, s>>>(a, a.qcount, a.qitems, a.qcap, nseg, split);
+    // the learned form keeps one thread per collision lane (groups of 8 segments, one
+    // block each): longer runs per thread reuse its cached per-anchor constants more
+    const bool learned = a.sampler == SAMPLER_LEARNED;
+    const int gsz = learned ? 8 : BZ_FIX_GROUP, groups = (nseg + gsz - 1) / gsz;
+    const int slices = learned ? 1 : fixup_slices(groups);
+    const unsigned grid = (unsigned)((int64_t)groups * slices);
+    if (learned)
+        k_fixup_f32<true><<<grid, 256, 0, s>>>(a, a.qcount, a.qitems, a.qcap, nseg, gsz, slices);
     else
-        k_fixup_f32<false><<<grid, 256, 0, s>>>(a, a.qcount, a.qitems, a.qcap, nseg, split);
+        k_fixup_f32<false><<<grid, 256, 0, s>>>(a, a.qcount, a.qitems, a.qcap, nseg, gsz, slices);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fixup_f32_batch(const CollideArgs<float>* boxes, const int* qcount, const unsigned long long* qitems,
                                    int64_t qcap, const int* step_dev, int nseg, cudaStream_t s)
 {
-    const int split = fixup_split(nseg);
-    k_fixup_f32_batch<<<(unsigned)(((int64_t)nseg * split + 7) / 8), 256, 0, s>>>(boxes, qcount, qitems, qcap, step_dev,
-                                                                                 nseg, split);
+    const int groups = (nseg + BZ_FIX_GROUP - 1) / BZ_FIX_GROUP, slices = fixup_slices(groups);
+    k_fixup_f32_batch<<<(unsigned)((int64_t)groups * slices), 256, 0, s>>>(boxes, qcount, qitems, qcap, step_dev, nseg,
+                                                                          BZ_FIX_GROUP, slices);
     return cudaGetLastError();
 }
-
 
 }  // namespace bz
