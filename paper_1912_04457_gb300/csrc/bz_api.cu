@@ -182,6 +182,12 @@ static void drop_step_graph(bz_handle h, int parity)
     h->sg[parity].exec = nullptr;
 }
 
+// d_acc: the masses' sums [x][4], then (zero between launches, like the sums) their
+// block counters [x] and the moments' chunk counters of fewer than 2 nsm rows
+static size_t acc_bytes(bz_handle h) { return sizeof(long long) * (5 * h->nxc + h->nsm); }
+static unsigned* mass_counters(bz_handle h) { return reinterpret_cast<unsigned*>(h->d_acc + 4 * h->nxc); }
+static unsigned* mom_counters(bz_handle h) { return reinterpret_cast<unsigned*>(h->d_acc + 5 * h->nxc); }
+
 static void free_scratch(bz_handle h)
 {
     drop_step_graph(h, 0);
@@ -381,7 +387,7 @@ extern "C" int bz_init_grid(bz_handle* out, const bz_grid* g)
     int rc;
     if (cudaMalloc(&h->d_m2[0], sizeof(double) * 4 * h->nxc) != cudaSuccess ||
         cudaMalloc(&h->d_m2[1], sizeof(double) * 4 * h->nxc) != cudaSuccess ||
-        cudaMalloc(&h->d_acc, sizeof(long long) * 4 * h->nxc) != cudaSuccess ||
+        cudaMalloc(&h->d_acc, acc_bytes(h)) != cudaSuccess ||
         cudaMalloc(&h->d_flags, sizeof(long long) * 4) != cudaSuccess ||
         cudaMalloc(&h->d_sflags, sizeof(long long) * 2) != cudaSuccess ||
         cudaMalloc(&h->d_jtab, sizeof(int) * h->npc) != cudaSuccess) {
@@ -406,6 +412,7 @@ extern "C" int bz_init_grid(bz_handle* out, const bz_grid* g)
         delete h;
         return rc;
     }
+    cudaMemset(h->d_acc, 0, acc_bytes(h));
     cudaMemset(h->d_flags, 0, sizeof(long long) * 4);
     cudaMemset(h->d_sflags, 0, sizeof(long long) * 2);
     cudaMemset(h->d_m2[0], 0, sizeof(double) * 4 * h->nxc);
@@ -654,7 +661,16 @@ static void fill_masses(bz_handle h, MassArgs& a, const long long* state, long l
     a.nu = h->nu;
 }
 
-static int compute_masses(bz_handle h, const long long* state, cudaStream_t s)
+// The masses' kernel is the one with the table of p^2 values, which can also copy
+// the state and advance a step graph's indices.
+static bool masses_by_table(bz_handle h)
+{
+    return h->mass_mode != BZ_MASS_FIXED && h->nu > 0 && h->nu <= MASS_TAB_MAX;
+}
+
+// drift: with one x cell its copy and f conversion by the same launch (masses_by_table), or null
+static int compute_masses(bz_handle h, const long long* state, cudaStream_t s, const DriftArgs* drift = nullptr,
+                          int* step_dev = nullptr)
 {
     if (h->mass_mode == BZ_MASS_FIXED) {
         if (!h->have_masses) return fail(h, BZ_EINVAL, "mass mode FIXED needs bz_set_masses first");
@@ -663,6 +679,17 @@ static int compute_masses(bz_handle h, const long long* state, cudaStream_t s)
     MassArgs a{};
     fill_masses(h, a, state, h->d_acc, h->d_m2[h->cur ^ 1],
                 (h->have_masses && h->mass_mode != BZ_MASS_MASSLESS) ? h->d_m2[h->cur] : nullptr);
+    a.done = mass_counters(h);
+    a.step_dev = step_dev;
+    if (drift) {
+        a.copy = drift->out;
+        a.freal = drift->freal;
+        a.freal_double = drift->freal_double;
+        for (int sl = 0; sl < NSPEC; ++sl) {
+            a.deg[sl] = drift->deg[sl];
+            a.fscale[sl] = drift->fscale[sl];
+        }
+    }
     {
         ProfScope ps(h, BZ_K_MASSES, s);
         CK(h, launch_masses(a, s));
@@ -1014,6 +1041,7 @@ static int fill_moments(bz_handle h, MomentArgs& a, const long long* state, doub
                 return fail(h, BZ_ENOMEM, "cannot allocate the moments scratch");
             h->mom_part_cap = need;
         }
+        a.done = mom_counters(h);
         a.part = h->d_mom_part;
     }
     a.nchunk = (int)nch;
@@ -1235,15 +1263,21 @@ extern "C" int bz_energy_source(bz_handle h, const int64_t* state, const double*
 // (with f of cur for the lookups), collision deposits into nxt, moments of
 // nxt.  Eager (step_dev null): step index `step`, moments at mom; inside a
 // captured graph: the step index and the moments slot of mom are read from
-// the device words step_dev[0], step_dev[1], advanced after the step.
+// the device words step_dev[0], step_dev[1], advanced by the step (before their use if the
+// masses' kernel does it, else at the end).
 static int one_step(bz_handle h, long long* cur, long long* nxt, double dt, int nsamples, int prec, int step,
                     double* mom, const int* step_dev, cudaStream_t s)
 {
     int rc;
-    if ((rc = compute_masses(h, cur, s))) return rc;
+    void* const freal = h->analytic ? nullptr : h->d_freal;
+    // one x cell: the drift is the identity, and the masses' kernel copies and converts the
+    // state (a launch less: 6 us of a 20^3 gluon step); profiles keep the launches apart
+    const bool table = masses_by_table(h), fused = table && h->nxc == 1 && !h->prof;
     DriftArgs d{};
-    fill_drift(h, d, cur, nxt, dt, h->analytic ? nullptr : h->d_freal, prec == BZ_PREC_F64);
-    {
+    if (fused) fill_drift(h, d, cur, nxt, dt, freal, prec == BZ_PREC_F64);
+    if ((rc = compute_masses(h, cur, s, fused ? &d : nullptr, table ? const_cast<int*>(step_dev) : nullptr))) return rc;
+    if (!fused) {
+        fill_drift(h, d, cur, nxt, dt, freal, prec == BZ_PREC_F64);
         ProfScope ps(h, BZ_K_DRIFT, s);
         CK(h, launch_drift(d, s));
     }
@@ -1258,7 +1292,7 @@ static int one_step(bz_handle h, long long* cur, long long* nxt, double dt, int 
         ProfScope ps(h, BZ_K_MOMENTS, s);
         CK(h, launch_moments(m, s));
     }
-    if (step_dev) CK(h, launch_step_advance(const_cast<int*>(step_dev), const_cast<int*>(step_dev) + 1, s));
+    if (step_dev && !table) CK(h, launch_step_advance(const_cast<int*>(step_dev), const_cast<int*>(step_dev) + 1, s));
     return BZ_OK;
 }
 
@@ -1328,7 +1362,8 @@ extern "C" int bz_step(bz_handle h, int64_t* state, double dt, int32_t nsteps, i
             G.sampler = h->step_sampler;
             G.gen = h->gen;
         }
-        CK(h, launch_set_step(h->d_step_idx, step0 + k, h->d_step_idx + 1, k, s));
+        const int back = masses_by_table(h) ? 1 : 0;  // the masses' kernel advances the indices first
+        CK(h, launch_set_step(h->d_step_idx, step0 + k - back, h->d_step_idx + 1, k - back, s));
         for (; nsteps - k >= 2; k += 2) CK(h, cudaGraphLaunch(G.exec, s));
     }
     while (k < nsteps)

@@ -199,7 +199,11 @@ inline bool momentum_octets(Args& a)
 
 struct MassArgs {
     const long long* state;
-    long long* acc;         // [x][4] fixed-point sums (zeroed by the caller)
+    long long* acc;         // [x][4] fixed-point sums
+    // [x] blocks that have added theirs, or null.  With it acc and done are zero between
+    // launches: the x cell's last block takes the sums, writes the masses and clears acc;
+    // without it the launch clears acc first and a second kernel writes the masses.
+    unsigned* done;
     double* m2_out;         // [x][4]
     const double* m2_prev;  // [x][4] or null (E = |p|)
     long long* flags;
@@ -216,6 +220,13 @@ struct MassArgs {
     const double* ppu;
     const unsigned short* pidx;  // [npc]
     int nu;
+    // with copy set (launches with the table): the state is copied to it, and to freal (float, or double) as f
+    long long* copy;
+    void* freal;
+    int freal_double;
+    double deg[NSPEC];      // per slot: N_s, FP32 rounding of 2^-40 / N_s
+    float fscale[NSPEC];
+    int* step_dev;          // with the table: step index and moments slot of a replayed step graph to advance, or null
 };
 constexpr int MASS_TAB_MAX = 6144;  // 4 x 6144 doubles of 1/(2E) per block in shared memory
 
@@ -267,6 +278,7 @@ struct MomentArgs {
     // ([x][slot][chunk][5] 128-bit as (lo, hi) int64 pairs) when nchunk > 1
     int nchunk;
     long long* part;
+    unsigned* done;         // [x][slot] chunks that have written theirs; zero between launches
     // grids whose FP32 cell centres are mirror images, pf[n-1-j] = -pf[j]: octets of mirrored cells
     // (momentum_octets), noct = 0 otherwise
     int noct, half[3];

@@ -119,6 +119,18 @@ __device__ __forceinline__ void masses_block(const MassArgs& P, int64_t x, int64
     }
 }
 
+// int64 to the nearest float: n = a 2^23 + b with |a| <= 2^22, b < 2^23 both exact
+// in FP32, one rounding; larger n by integer instructions
+__device__ __forceinline__ float ll2float_fast(long long n)
+{
+    const int hi = (int)(n >> 32);
+    if ((unsigned)(hi ^ (hi >> 31)) >= (1u << 13)) return ll2float_rn(n);  // |n| >= 2^45
+    const int a = (int)(n >> 23);
+    const float fa = __int_as_float(a + 0x4B400000) - 12582912.0f;
+    const float fb = __uint_as_float(((unsigned)n & 0x7fffffu) | 0x4B000000u) - 8388608.0f;
+    return fmaf(fa, 8388608.0f, fb);
+}
+
 // Thermal masses with the table of distinct p^2 values: the same sums as
 // masses_block, bit for bit, on the integer pipe.
 //
@@ -211,9 +223,12 @@ __device__ __noinline__ MassBin mass_bin_slow(double pp, const double* m2_prev, 
     for (int i = 0; i < 3; ++i) o.q[i] = __double2ll_rn((3.0 * gn * rg + 4.0 * q[i] * rq[i]) * MASS_FX);
     return o;
 }
-template <bool GLUON_ONLY>
+// COPY (one x cell: its drift is the identity): the state is also written to
+// P.copy and as f to P.freal, in the place of a launch that reads it again.
+template <bool GLUON_ONLY, bool COPY>
 __global__ void __launch_bounds__(MASS_THREADS, 4) k_masses_tab(const __grid_constant__ MassArgs P)
 {
+    if (P.step_dev && blockIdx.x == 0 && threadIdx.x < 2) P.step_dev[threadIdx.x] += 1;
     extern __shared__ uint64_t s_R[];  // [GLUON_ONLY ? 1 : 4][nu]
     constexpr int NS = GLUON_ONLY ? 1 : 4;
     const int nu = P.nu;
@@ -284,6 +299,20 @@ __global__ void __launch_bounds__(MASS_THREADS, 4) k_masses_tab(const __grid_con
         for (int k = 0; k < AHEAD; ++k) {  // a bin beyond the end has n = 0 and adds 0
             const int u = ub[k];
             const long long* n = nsp[k];
+            if (COPY && jb + k * MASS_THREADS < jstop) {
+#pragma unroll
+                for (int s = 0; s < NV; ++s) {
+                    const int sl = GLUON_ONLY ? 0 : P.slot_of[s];
+                    if (sl < 0) continue;
+                    const int64_t cell = (int64_t)sl * sstride + x * P.npc + jb + k * MASS_THREADS;
+                    P.copy[cell] = n[s];
+                    if (!P.freal) continue;
+                    if (P.freal_double)
+                        static_cast<double*>(P.freal)[cell] = (double)n[s] * TWO_POW_M40 / P.deg[sl];
+                    else
+                        static_cast<float*>(P.freal)[cell] = ll2float_fast(n[s]) * P.fscale[sl];
+                }
+            }
             MassBin o;
             bool done;
             if constexpr (GLUON_ONLY) {
@@ -338,14 +367,25 @@ __global__ void __launch_bounds__(MASS_THREADS, 4) k_masses_tab(const __grid_con
     }
     if (ovf) red_add_ll(&P.flags[2], 1);
     __syncthreads();
-    if (threadIdx.x < 4) {
-        long long t = 0;
-        for (int w = 0; w < MASS_THREADS / 32; ++w) t += red[threadIdx.x][w];
-        if (nchunk == 1)  // the block has the x cell's whole sums
-            P.m2_out[x * 4 + threadIdx.x] = mass_of(P, (int)threadIdx.x, t);
-        else
-            red_add_ll(&P.acc[x * 4 + threadIdx.x], t);
+    if (threadIdx.x >= 32) return;
+    long long t = 0;
+    if (lane < 4)
+        for (int w = 0; w < MASS_THREADS / 32; ++w) t += red[lane][w];
+    if (nchunk > 1) {
+        if (lane < 4) {
+            red_add_ll(&P.acc[x * 4 + lane], t);
+            __threadfence();
+        }
+        if (!P.done) return;
+        __syncwarp();
+        unsigned before = lane == 0 ? atomicInc(P.done + x, (unsigned)nchunk - 1u) : 0u;  // wraps to 0
+        before = __shfl_sync(0xffffffffu, before, 0);
+        if (before != (unsigned)nchunk - 1u) return;
+        __threadfence();
+        if (lane < 4) t = (long long)atomicExch(reinterpret_cast<unsigned long long*>(&P.acc[x * 4 + lane]), 0ull);
     }
+    // the block has the x cell's whole sums, or is the last of its blocks
+    if (lane < 4) P.m2_out[x * 4 + lane] = mass_of(P, lane, t);
 }
 
 __global__ void __launch_bounds__(256, BZ_MASS_MINB) k_masses(const __grid_constant__ MassArgs P)
@@ -401,7 +441,8 @@ cudaError_t launch_masses(const MassArgs& a, cudaStream_t s)
     b.chunk = chunk < 256 ? 256 : (chunk > MASS_CHUNK ? MASS_CHUNK : chunk);
     if (tab && per_x == 1) b.chunk = a.npc;
     const int64_t nchunk = (a.npc + b.chunk - 1) / b.chunk;
-    if (!tab || nchunk > 1) {
+    if (!tab) b.done = nullptr;
+    if (!tab || (nchunk > 1 && !b.done)) {
         const cudaError_t e = cudaMemsetAsync(a.acc, 0, sizeof(long long) * 4 * a.nxc, s);
         if (e != cudaSuccess) return e;
     }
@@ -409,14 +450,15 @@ cudaError_t launch_masses(const MassArgs& a, cudaStream_t s)
         bool gluon_only = a.slot_of[0] == 0;
         for (int q = 1; q < NSPEC; ++q) gluon_only = gluon_only && a.slot_of[q] < 0;
         const size_t smem = sizeof(uint64_t) * (gluon_only ? 1 : 4) * (size_t)a.nu;
-        if (gluon_only) {
-            if (smem > 48 * 1024) cudaFuncSetAttribute(k_masses_tab<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            k_masses_tab<true><<<(unsigned)(nchunk * a.nxc), MASS_THREADS, smem, s>>>(b);
-        } else {
-            if (smem > 48 * 1024) cudaFuncSetAttribute(k_masses_tab<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            k_masses_tab<false><<<(unsigned)(nchunk * a.nxc), MASS_THREADS, smem, s>>>(b);
-        }
-        if (nchunk == 1) return cudaGetLastError();
+        auto run = [&](auto kernel) {
+            if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            kernel<<<(unsigned)(nchunk * a.nxc), MASS_THREADS, smem, s>>>(b);
+        };
+        if (gluon_only)
+            b.copy ? run(k_masses_tab<true, true>) : run(k_masses_tab<true, false>);
+        else
+            b.copy ? run(k_masses_tab<false, true>) : run(k_masses_tab<false, false>);
+        if (nchunk == 1 || b.done) return cudaGetLastError();
     } else {
         k_masses<<<(unsigned)(nchunk * a.nxc), 256, 0, s>>>(b);
     }
@@ -692,18 +734,6 @@ __global__ void __launch_bounds__(256) k_inv_octet(const __grid_constant__ Drift
         const float p0 = P.pf[0][h[0]], p1 = P.pf[1][h[1]], p2 = P.pf[2][h[2]];
         out[o] = 1.0f / sqrtf((p0 * p0 + p1 * p1) + p2 * p2 + m);
     }
-}
-
-// int64 to the nearest float: n = a 2^23 + b with |a| <= 2^22, b < 2^23 both exact
-// in FP32, one rounding; larger n by integer instructions
-__device__ __forceinline__ float ll2float_fast(long long n)
-{
-    const int hi = (int)(n >> 32);
-    if ((unsigned)(hi ^ (hi >> 31)) >= (1u << 13)) return ll2float_rn(n);  // |n| >= 2^45
-    const int a = (int)(n >> 23);
-    const float fa = __int_as_float(a + 0x4B400000) - 12582912.0f;
-    const float fb = __uint_as_float(((unsigned)n & 0x7fffffu) | 0x4B000000u) - 8388608.0f;
-    return fmaf(fa, 8388608.0f, fb);
 }
 
 // Force-term part of the update of one cell (p indices jv), as force_acc, with
@@ -1263,7 +1293,7 @@ __device__ __forceinline__ void moments_block(const MomentArgs& P, int64_t x, in
         __int128 t[5] = {0, 0, 0, 0, 0};
         for (int w = 0; w < MOM_THREADS / 32; ++w)
             for (int i = 0; i < 5; ++i) t[i] += red[i][w];
-        if (part) {  // exact partial sums of this chunk, combined by k_moments_finish
+        if (part) {  // exact partial sums of this chunk, added by the last block
             for (int i = 0; i < 5; ++i) {
                 part[2 * i] = (long long)(unsigned long long)t[i];
                 part[2 * i + 1] = (long long)(t[i] >> 64);
@@ -1275,7 +1305,8 @@ __device__ __forceinline__ void moments_block(const MomentArgs& P, int64_t x, in
 }
 
 // Block = (x cell, slot, chunk of the p cells); with one chunk the block
-// writes the moments, else its exact partial sums for k_moments_finish.
+// writes the moments, else its exact partial sums, which the last of the (x cell,
+// slot)'s blocks adds (a second kernel with a thread per (x cell, slot): 7 us).
 __global__ void __launch_bounds__(MOM_THREADS, 7) k_moments(const __grid_constant__ MomentArgs P)
 {
     const int nch = P.nchunk > 1 ? P.nchunk : 1;
@@ -1284,21 +1315,27 @@ __global__ void __launch_bounds__(MOM_THREADS, 7) k_moments(const __grid_constan
     const int64_t x = row / P.nslots;
     const int sl = (int)(row % P.nslots);
     double* out = P.out + (P.kidx ? (int64_t)*P.kidx * P.kstride : 0);
-    moments_block(P, x, sl, c, nch, out + (x * P.nslots + sl) * 5, nch > 1 ? P.part + (int64_t)blockIdx.x * 10 : nullptr);
-}
-
-// Adds the chunks' partial sums of each (x cell, slot) in chunk order.
-__global__ void k_moments_finish(const __grid_constant__ MomentArgs P)
-{
-    const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= P.nxc * P.nslots) return;
-    __int128 t[5] = {0, 0, 0, 0, 0};
-    for (int c = 0; c < P.nchunk; ++c) {
-        const long long* q = P.part + (row * P.nchunk + c) * 10;
-        for (int i = 0; i < 5; ++i)
-            t[i] += (__int128)(((unsigned __int128)(unsigned long long)q[2 * i + 1] << 64) | (unsigned long long)q[2 * i]);
+    double* o = out + (x * P.nslots + sl) * 5;
+    moments_block(P, x, sl, c, nch, o, nch > 1 ? P.part + (int64_t)blockIdx.x * 10 : nullptr);
+    if (nch == 1 || threadIdx.x >= 32) return;
+    const int lane = (int)threadIdx.x;
+    unsigned before = 0;
+    if (lane == 0) {  // the thread that wrote the sums
+        __threadfence();
+        before = atomicInc(P.done + row, (unsigned)nch - 1u);  // wraps to 0
     }
-    moments_out(P, t, P.out + (P.kidx ? (int64_t)*P.kidx * P.kstride : 0) + row * 5);
+    before = __shfl_sync(0xffffffffu, before, 0);
+    if (before != (unsigned)nch - 1u) return;
+    __threadfence();
+    __int128 t[5] = {0, 0, 0, 0, 0};  // exact sums: any order gives the same bits
+    for (int k = lane; k < nch; k += 32) {
+        const long long* q = P.part + (row * nch + k) * 10;
+        for (int i = 0; i < 5; ++i)
+            t[i] += (__int128)(((unsigned __int128)(unsigned long long)__ldcg(q + 2 * i + 1) << 64) |
+                               (unsigned long long)__ldcg(q + 2 * i));
+    }
+    for (int i = 0; i < 5; ++i) t[i] = warp_sum_i128(t[i]);
+    if (lane == 0) moments_out(P, t, o);
 }
 
 cudaError_t launch_moments(const MomentArgs& a, cudaStream_t s)
@@ -1307,7 +1344,6 @@ cudaError_t launch_moments(const MomentArgs& a, cudaStream_t s)
     MomentArgs b = a;
     b.nchunk = nch;
     k_moments<<<(unsigned)(a.nxc * a.nslots * nch), MOM_THREADS, 0, s>>>(b);
-    if (nch > 1) k_moments_finish<<<(unsigned)((a.nxc * a.nslots + 127) / 128), 128, 0, s>>>(b);
     return cudaGetLastError();
 }
 
