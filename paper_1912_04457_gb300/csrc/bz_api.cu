@@ -65,6 +65,7 @@ struct bz_handle_s {
     float *d_prop = nullptr, *d_prop_m = nullptr, *d_prop_v = nullptr;
     float* d_anchor_prm = nullptr;
     float* d_loss = nullptr;
+    char* d_prop_img = nullptr;        // the network's weights as BF16 operands (training)
     float* d_losses = nullptr;         // [LOSS_CAP] losses of a training call's steps
     double* d_wsum = nullptr;          // [sum_weights_scratch()]: the sum, then the per-warp partial sums
     float* d_prop_part = nullptr;      // per-block gradients [4 nsm][nparam] and losses [4 nsm]
@@ -234,7 +235,9 @@ static void free_scratch(bz_handle h)
     cudaFree(h->d_anchor_prm);
     cudaFree(h->d_loss);
     cudaFree(h->d_losses);
+    cudaFree(h->d_prop_img);
     h->d_losses = nullptr;
+    h->d_prop_img = nullptr;
     cudaFree(h->d_wsum);
     cudaFree(h->d_prop_part);
     cudaFree(h->d_loss_part);
@@ -1793,7 +1796,8 @@ static int prop_alloc(bz_handle h)
 {
     const int n = mlp_nparam();
     if (h->d_prop) return BZ_OK;
-    if (!dalloc(&h->d_prop, n) || !dalloc(&h->d_losses, LOSS_CAP) || !dalloc(&h->d_prop_m, n) ||
+    if (!dalloc(&h->d_prop, n) || !dalloc(&h->d_losses, LOSS_CAP) ||
+        !dalloc(&h->d_prop_img, mlp_image_bytes()) || !dalloc(&h->d_prop_m, n) ||
         !dalloc(&h->d_prop_v, n) || !dalloc(&h->d_loss, 1) || !dalloc(&h->d_wsum, sum_weights_scratch()) ||
         !dalloc(&h->d_prop_part, (size_t)4 * h->nsm * n) || !dalloc(&h->d_loss_part, (size_t)4 * h->nsm) ||
         !dalloc(&h->d_prop_err, 1))
@@ -1883,7 +1887,7 @@ extern "C" int bz_proposal_grad(bz_handle h, const void* records, int64_t n, flo
     CK(h, cudaMemsetAsync(grad, 0, sizeof(float) * mlp_nparam(), s));
     CK(h, cudaMemsetAsync(loss, 0, sizeof(float), s));
     CK(h, cudaMemsetAsync(h->d_prop_err, 0, sizeof(int), s));
-    CK(h, launch_mlp_grad(h->d_prop, prop_args(h), rec, n, (float)(1.0 / wsum), grad, loss, h->nsm, h->d_prop_part,
+    CK(h, launch_mlp_grad(h->d_prop, h->d_prop_img, prop_args(h), rec, n, (float)(1.0 / wsum), grad, loss, h->nsm, h->d_prop_part,
                           h->d_loss_part, h->d_prop_err, s));
     int herr = 0;
     CK(h, cudaMemcpyAsync(&herr, h->d_prop_err, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1916,7 +1920,7 @@ extern "C" int bz_proposal_train(bz_handle h, const void* records, int64_t n, in
         for (int k = 0; k < kn; ++k) {
             const int64_t b = batch;
             const uint64_t key = ((uint64_t)(h->adam_step + 1) << 32) * 0x9E3779B97F4A7C15ull;
-            CK(h, launch_mlp_grad(h->d_prop, A, rec, b, (float)(1.0 / (wbar * (double)b)), nullptr,
+            CK(h, launch_mlp_grad(h->d_prop, h->d_prop_img, A, rec, b, (float)(1.0 / (wbar * (double)b)), nullptr,
                                   losses_host ? h->d_losses + k : h->d_loss, h->nsm, h->d_prop_part, h->d_loss_part, h->d_prop_err,
                                   s, n, key, h->d_prop, h->d_prop_m, h->d_prop_v, (float)lr, h->adam_step + 1, k > 0));
             ++h->adam_step;

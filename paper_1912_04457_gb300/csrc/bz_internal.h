@@ -366,14 +366,16 @@ inline int f32_unit_chunks(int64_t items, int64_t warps)
     return (int)(c < 8 ? 8 : (c > 32 ? 32 : c));
 }
 int mlp_nparam();
+int mlp_image_bytes();
 // ntot > 0: minibatch position r reads record splitmix64(key + r) mod ntot of rec
 // (i.i.d. draws from all ntot records); ntot = 0: records [0, n) in order
 // part [grid][nparam], part_loss [grid]: per-block scratch, added in block order into grad (+=) and loss (=);
 // err (device int): incremented by a block whose tensor-core wait timed out.  At most `grid` blocks, one
 // per SM (each holds 512 columns of tensor memory).
+// img: mlp_image_bytes() of scratch, the weights as BF16 operands.
 // p set: the gradient is taken as step `step` of Adam on the parameters p with moments m, v instead of added to grad.
 // chained: the launch before this one on s is the update of such a step, and nothing since has written rec.
-cudaError_t launch_mlp_grad(const float* params, const ProposalArgs& A, const ProposalRecord* rec, int64_t n,
+cudaError_t launch_mlp_grad(const float* params, void* img, const ProposalArgs& A, const ProposalRecord* rec, int64_t n,
                             float inv_wsum, float* grad, float* loss, int grid, float* part, float* part_loss, int* err,
                             cudaStream_t s, int64_t ntot = 0, uint64_t key = 0, float* p = nullptr, float* m = nullptr,
                             float* v = nullptr, float lr = 0.0f, int step = 0, bool chained = false);

@@ -91,18 +91,31 @@ __device__ __forceinline__ float t2_tail(float z)
     return 1.0f / (s * (s + fabsf(z)));
 }
 
-// One factor of q: density g of component i (0, 1: k1; 2..4: k3) and d log g / d (mu, sigma)
-__device__ __forceinline__ void factor_grad(float mu, float s, float y, float& g, float& dm, float& ds)
+// The truncation of a factor of q with centre mu and scale s
+struct FactorEnds {
+    float za, zb, pa, pb, sZ;
+};
+__device__ __forceinline__ FactorEnds factor_ends(float mu, float s)
 {
-    const float z = (y - mu) / s, za = (-1.0f - mu) / s, zb = (1.0f - mu) / s;
+    FactorEnds e;
+    e.za = (-1.0f - mu) / s;
+    e.zb = (1.0f - mu) / s;
     // za < 0 < zb: Z = F(zb) - F(za) = 1 - tail(zb) - tail(za)
-    const float Z = (1.0f - t2_tail(zb)) - t2_tail(za);
-    const float pa = t2_pdf(za), pb = t2_pdf(zb);
-    g = t2_pdf(z) / (s * Z);
+    const float Z = (1.0f - t2_tail(e.zb)) - t2_tail(e.za);
+    e.pa = t2_pdf(e.za);
+    e.pb = t2_pdf(e.zb);
+    e.sZ = s * Z;
+    return e;
+}
+// One factor of q at y: density g and d log g / d (mu, s)
+__device__ __forceinline__ void factor_grad(const FactorEnds& e, float mu, float s, float y, float& g, float& dm, float& ds)
+{
+    const float z = (y - mu) / s;
+    g = t2_pdf(z) / e.sZ;
     // d log g / d mu and d log g / d s, with d log f / dz = -3 z / (2 + z^2)
     const float dlf = -3.0f * z / (2.0f + z * z);
-    dm = -dlf / s + (pb - pa) / (s * Z);
-    ds = -dlf * z / s - 1.0f / s + (pb * zb - pa * za) / (s * Z);
+    dm = -dlf / s + (e.pb - e.pa) / e.sZ;
+    ds = -dlf * z / s - 1.0f / s + (e.pb * e.zb - e.pa * e.za) / e.sZ;
 }
 
 // log q(y) and d log q / d o (6) of one record from its parameters (head) and
@@ -330,9 +343,9 @@ constexpr uint32_t C_T = 0, C_O = 128, C_S = 160, C_S3 = 416, C_W2 = 256, C_W3 =
 struct TrainSmem {
     __nv_bfloat16 W1[NIN * H];  // op_off(f, i, H)
     __nv_bfloat16 W3[H * 16];   // op_off(i, j, 16), outputs 8..15 zero
+    __nv_bfloat16 W2[H * H];    // op_off(i, n, H); W1, W3, W2 in one piece are the weight image
     __nv_bfloat16 X[RB * NIN];  // op_off(r, f, NIN)
     __nv_bfloat16 dO[RB * 16];  // op_off(r, j, 16)
-    __nv_bfloat16 W2[H * H];    // op_off(i, n, H)
     __nv_bfloat16 H1[RB * H], H2[RB * H], Z1[RB * H], Z2[RB * H];  // op_off(r, i, H); Z1, Z2 later hold dZ1, dZ2
     float b1[H], b2[H], b3[16];
     float yv[RB * 5], wv[RB];
@@ -356,18 +369,43 @@ __device__ __forceinline__ uint64_t dmn(uint32_t base, int C, int kk)
 }
 }  // namespace tc
 
+// The weights as MMA operands, in BF16 and in the order of TrainSmem: an update writes
+// the parameters and this image of them, so that a block copies 40 KB instead of
+// converting 79 KB (each of 128 blocks: 6000 cycles of the kernel's 36000).
+constexpr int IMG_W3 = NIN * H, IMG_W2 = IMG_W3 + H * 16, IMG_N = IMG_W2 + H * H;
+static_assert(IMG_N * 2 == 5 * 16 * 512, "five 16-byte words per thread");
+__device__ __forceinline__ int image_offset(int k)  // of parameter k, or -1 (a bias)
+{
+    using tc::op_off;
+    if (k < NIN * H) return op_off(k / H, k % H, H);
+    k -= NIN * H + H;
+    if (k < 0) return -1;
+    if (k < H * H) return IMG_W2 + op_off(k / H, k % H, H);
+    k -= H * H + H;
+    if (k < 0 || k >= H * NOUT) return -1;
+    return IMG_W3 + op_off(k / NOUT, k % NOUT, 16);
+}
+__global__ void __launch_bounds__(256) k_weight_image(const float* __restrict__ params, __nv_bfloat16* __restrict__ img)
+{
+    const int k = blockIdx.x * 256 + threadIdx.x;
+    const int o = k < NPARAM ? image_offset(k) : -1;
+    if (o < 0) return;
+    img[o] = __float2bfloat16_rn(params[k]);
+    if (o >= IMG_W3 && o < IMG_W2) img[o + 64] = __float2bfloat16_rn(0.0f);  // operand columns 8..15: the next core matrix
+}
+
 // 512 threads: warp w reads lane quarter w mod 4 of an accumulator (rows 32 (w mod
 // 4) ..) and its columns 32 (w / 4) .., and stores activations as 16-byte words.  A
 // 16384-record minibatch is one chunk per block and a chain of ten dependent stages
 // (product, epilogue, barrier), so that a stage's latency is the time: 128 threads
 // with 128 columns each and 2-byte stores took 97 us, this 26 us.  What is left
 // is SiLU (128 per scheduler and layer at some 40 issue cycles: exponential and
-// division), the weights' 79 KB per block and the gradient's 79 KB.  SiLU' is taken
+// division), the weights' 40 KB per block and the gradient's 79 KB.  SiLU' is taken
 // with SiLU and kept in FP32 until the backward pass (one layer in registers, one in
 // tensor memory): with the exponential evaluated again there 31 us.
 constexpr int GRAD_THREADS = 512;
 
-__global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(const float* __restrict__ params, const ProposalArgs A,
+__global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(const float* params, const __nv_bfloat16* img, const ProposalArgs A,
                                                               const ProposalRecord* __restrict__ rec, int64_t n,
                                                               float inv_wsum, float* __restrict__ part,
                                                               float* __restrict__ part_loss, int64_t ntot, uint64_t key, int* err)
@@ -384,6 +422,19 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(const float* __res
         R.a = -1;
         if (cg == 0 && r < n) R = rec[ntot > 0 ? (int64_t)(splitmix64(key + (uint64_t)r) % (uint64_t)ntot) : r];
     };
+    const int64_t nchunks = (n + RB - 1) / RB;
+    auto inputs = [&](int64_t c) {  // one record per row; then the next chunk's on the way
+        if (cg != 0) return;
+        float f[NIN];
+        if (R.a >= 0)
+            anchor_features(A, R.a, f);
+        else
+            for (int i = 0; i < NIN; ++i) f[i] = 0.0f;
+        for (int i = 0; i < 5; ++i) S.yv[row * 5 + i] = R.y[i];
+        S.wv[row] = R.w * inv_wsum;
+        store_x(S.X, row, f);
+        if (c + gridDim.x < nchunks) fetch(c + gridDim.x);
+    };
     fetch(blockIdx.x);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&S.mbar)) : "memory");
@@ -394,19 +445,21 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(const float* __res
                      "r"(TRAIN_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    inputs(blockIdx.x);
     // the previous step's parameters; the update may still run beside this block and pass
     // through the same L1, so that they are read from L2
     asm volatile("griddepcontrol.wait;" ::: "memory");
     {
-        const float* W1 = params;
-        const float* b1 = W1 + NIN * H;
-        const float* W2 = b1 + H;
-        const float* b2 = W2 + H * H;
-        const float* W3 = b2 + H;
-        const float* b3 = W3 + H * NOUT;
-        load_weights<H, H, GRAD_THREADS>(S.W2, W2);
-        load_weights<NIN, H, GRAD_THREADS>(S.W1, W1);
-        load_w3(S.W3, W3);
+        const float* b1 = params + NIN * H;
+        const float* b2 = b1 + H + H * H;
+        const float* b3 = b2 + H + H * NOUT;
+        const uint4* src = reinterpret_cast<const uint4*>(img);
+        uint4* dst = reinterpret_cast<uint4*>(S.W1);
+        uint4 v[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) v[k] = __ldcg(src + tid + k * GRAD_THREADS);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) dst[tid + k * GRAD_THREADS] = v[k];
         if (tid < H) {
             S.b1[tid] = __ldcg(b1 + tid);
             S.b2[tid] = __ldcg(b2 + tid);
@@ -436,21 +489,9 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(const float* __res
         fence_async_smem();
         __syncthreads();
     };
-    const int64_t nchunks = (n + RB - 1) / RB;
     bool first = true;
     for (int64_t c = blockIdx.x; c < nchunks && ok; c += gridDim.x, first = false) {
-        // ---- inputs: one record per row ----
-        if (cg == 0) {
-            float f[NIN];
-            if (R.a >= 0)
-                anchor_features(A, R.a, f);
-            else
-                for (int i = 0; i < NIN; ++i) f[i] = 0.0f;
-            for (int i = 0; i < 5; ++i) S.yv[row * 5 + i] = R.y[i];
-            S.wv[row] = R.w * inv_wsum;
-            store_x(S.X, row, f);
-            if (c + gridDim.x < nchunks) fetch(c + gridDim.x);
-        }
+        if (!first) inputs(c);
         sync_operands();
         // ---- hidden layers ----
         // Z + b rounded to BF16, H = SiLU; SiLU' stays in FP32: of Z1 in tensor memory, of Z2 in registers
@@ -513,9 +554,10 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(const float* __res
         {
             const float* y = S.yv + row * 5;
             float f[3];
+            const float mu = cg == 0 ? 0.0f : (cg == 1 ? prm[0] : (cg == 2 ? prm[1] : prm[2])), sg = cg == 0 ? prm[4] : prm[3];
+            const FactorEnds e = factor_ends(mu, sg);
             for (int i = cg == 0 ? 0 : cg + 1; i <= cg + 1; ++i) {
-                const float mu = cg == 0 ? 0.0f : (cg == 1 ? prm[0] : (cg == 2 ? prm[1] : prm[2]));
-                factor_grad(mu, cg == 0 ? prm[4] : prm[3], y[i], f[0], f[1], f[2]);
+                factor_grad(e, mu, sg, y[i], f[0], f[1], f[2]);
 #pragma unroll
                 for (int k = 0; k < 3; ++k) S.fac[(3 * i + k) * RB + row] = f[k];
             }
@@ -681,6 +723,7 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(const float* __res
 // Adam's constants of one step (c1, c2: the bias corrections).
 struct AdamStep {
     float *p, *m, *v;
+    __nv_bfloat16* img;
     float lr, b1, b2, eps, c1, c2;
 };
 
@@ -725,7 +768,10 @@ __global__ void __launch_bounds__(128) k_grad_reduce(const float* __restrict__ p
             const float vk = U.b2 * __ldcg(U.v + k) + (1.0f - U.b2) * g * g;
             U.m[k] = mk;
             U.v[k] = vk;
-            U.p[k] = __ldcg(U.p + k) - U.lr * (mk / U.c1) / (sqrtf(vk / U.c2) + U.eps);
+            const float pk = __ldcg(U.p + k) - U.lr * (mk / U.c1) / (sqrtf(vk / U.c2) + U.eps);
+            U.p[k] = pk;
+            const int o = image_offset(k);
+            if (o >= 0) U.img[o] = __float2bfloat16_rn(pk);
         } else {
             grad[k] += g;
         }
@@ -953,7 +999,9 @@ cudaError_t launch_sort_records(ProposalRecord* rec, int64_t n, cudaStream_t s)
 
 int mlp_nparam() { return NPARAM; }
 
-cudaError_t launch_mlp_grad(const float* params, const ProposalArgs& A, const ProposalRecord* rec, int64_t n,
+int mlp_image_bytes() { return IMG_N * 2; }
+
+cudaError_t launch_mlp_grad(const float* params, void* img, const ProposalArgs& A, const ProposalRecord* rec, int64_t n,
                             float inv_wsum, float* grad, float* loss, int grid, float* part, float* part_loss, int* err,
                             cudaStream_t s, int64_t ntot, uint64_t key, float* p, float* m, float* v, float lr, int step, bool chained)
 {
@@ -976,7 +1024,9 @@ cudaError_t launch_mlp_grad(const float* params, const ProposalArgs& A, const Pr
     lc.stream = s;
     lc.attrs = &at;
     lc.numAttrs = chained ? 1 : 0;
-    cudaError_t le = cudaLaunchKernelEx(&lc, k_mlp_grad, params, A, rec, n, inv_wsum, part, part_loss, ntot, key, err);
+    __nv_bfloat16* const im = static_cast<__nv_bfloat16*>(img);
+    if (!chained) k_weight_image<<<(NPARAM + 255) / 256, 256, 0, s>>>(params, im);
+    cudaError_t le = cudaLaunchKernelEx(&lc, k_mlp_grad, params, (const __nv_bfloat16*)im, A, rec, n, inv_wsum, part, part_loss, ntot, key, err);
     if (le != cudaSuccess) return le;
     lc.gridDim = dim3((NPARAM + 63) / 64);
     lc.blockDim = dim3(128);
@@ -984,7 +1034,7 @@ cudaError_t launch_mlp_grad(const float* params, const ProposalArgs& A, const Pr
     lc.numAttrs = 1;
     if (p) {
         const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-        const AdamStep U{p, m, v, lr, b1, b2, eps, 1.0f - powf(b1, (float)step), 1.0f - powf(b2, (float)step)};
+        const AdamStep U{p, m, v, im, lr, b1, b2, eps, 1.0f - powf(b1, (float)step), 1.0f - powf(b2, (float)step)};
         le = cudaLaunchKernelEx(&lc, k_grad_reduce<true>, (const float*)part, (const float*)part_loss, g, (float*)nullptr, loss, U);
     } else {
         le = cudaLaunchKernelEx(&lc, k_grad_reduce<false>, (const float*)part, (const float*)part_loss, g, grad, loss, AdamStep{});
