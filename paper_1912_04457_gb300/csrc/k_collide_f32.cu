@@ -83,7 +83,7 @@ template <int MODE, bool GROUPS> struct WarpSmem {
     // | bin of Pz - z << 16 | first term << 24 | (terms - 1) << 28
     float4 ring[RING];
     // this unit's terms: masses of the legs and sym, packed leg slots / flags / row
-    float4 tm[GROUPS ? MAX_TERMS : 1];  // (ma2, mb2, mc2, sym)
+    float4 tm[GROUPS ? MAX_TERMS : 1];  // (ma2, mb2, mc2, sym; learned: -sym if the next term shares leg 2)
     int tinfo[GROUPS ? MAX_TERMS : 1];  // slot0 | slot1 << 3 | slot2 << 6 | quark0..3 << 9..12 | cls << 13
     int tgn[GROUPS ? MAX_TERMS : 1];    // terms of the kinematic group the term opens (0: not a group's first)
 };
@@ -289,6 +289,12 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
     float m2v = __shfl_sync(0xffffffffu, mv, 2), m3 = __shfl_sync(0xffffffffu, mv, 3);
     if (P.mass_mode == 1) m0 = m1 = m2v = m3 = 0.0f;
 
+    // A group's terms often share leg 2 ((q, d, q) and (qbar, d, qbar)).  Adding such terms'
+    // deposits to its cell first leaves one atomic in ten out: the learned sampler, most
+    // of whose roots deposit, gains (16^3, seven species: 990 -> 952 us with 6 blocks per SM);
+    // the uniform one gains where f is of order 1 everywhere (32^3: 15.2 -> 14.7 ms) and
+    // loses where most of its roots deposit nothing (12.5 -> 13.1 ms), so it does not.
+    constexpr bool MERGE = MODE == M_LEARNED;
     const int nt = GROUPS ? P.nterms[d] : 1;
     if constexpr (GROUPS) {
         // kinematic groups: consecutive terms with equal leg masses (the first
@@ -297,12 +303,14 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
         const unsigned firsts = __ballot_sync(0xffffffffu, gfirst);
         if (lane < nt) {
             const TermDev& T = P.terms[d][lane];
+            const unsigned after = firsts & ~((2u << lane) - 1u);
+            const int end = after ? __ffs(after) - 1 : nt;
+            const bool share = lane + 1 < end && P.terms[d][lane + 1].slot[1] == T.slot[1];
             S.tm[lane] = make_float4(sel4(T.mslot[0], m0, m1, m2v, m3), sel4(T.mslot[1], m0, m1, m2v, m3),
-                                     sel4(T.mslot[2], m0, m1, m2v, m3), (float)T.sym);
+                                     sel4(T.mslot[2], m0, m1, m2v, m3), MERGE && share ? -(float)T.sym : (float)T.sym);
             S.tinfo[lane] = T.slot[0] | (T.slot[1] << 3) | (T.slot[2] << 6) | (T.quark[0] << 9) | (T.quark[1] << 10)
                             | (T.quark[2] << 11) | (T.quark[3] << 12) | (T.cls << 13);
-            const unsigned after = firsts & ~((2u << lane) - 1u);
-            S.tgn[lane] = gfirst ? (after ? __ffs(after) - 1 : nt) - lane : 0;
+            S.tgn[lane] = gfirst ? end - lane : 0;
         }
     }
     const float md2 = sel4(P.terms[d][0].mslot[3], m0, m1, m2v, m3);
@@ -342,15 +350,46 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
             const int t0 = GROUPS ? (tg >> 24) & 15 : 0, tn = GROUPS ? (int)(tg >> 28) + 1 : 1;
             src_rec = src;
             const float z = rv.x, E3 = rv.y, sqH = rv.z;
+            const float4 ga = S.ga[src];
+            const float Ep = ga.x;
+            const uint32_t i4 = __float_as_uint(ga.y);
+            const int2 gc = S.gc[src];
+            const unsigned lin1 = (gc.y & 0xffff) * P.np[2] + ((tg >> 8) & 0xff);
+            const unsigned lin2 = ((unsigned)gc.y >> 16) * P.np[2] + ((tg >> 16) & 0xff);
+            const unsigned lin3 = gc.x;
+            // the cells and occupations of a term's legs; a single term's, and the anchor's
+            // occupation, are loaded ahead of the arithmetic that comes before their use (20^3
+            // gluons, 64 samples: 20.7 -> 18.9 us; 32^3, seven species: 13.0 -> 12.5 ms; the first
+            // term of a group's as well, and each next one's ahead: 3% slower)
+            unsigned i1, i2, i3;
+            float f1 = 0.0f, f2 = 0.0f, f3 = 0.0f, fpp = 0.0f;
+            int info = 0;
+            auto legs = [&](int ti) {
+                i1 = lin1;
+                i2 = lin2;
+                i3 = lin3;
+                if constexpr (GROUPS) {
+                    info = S.tinfo[ti];
+                    i1 += (unsigned)(info & 7) * slot_stride;
+                    i2 += (unsigned)((info >> 3) & 7) * slot_stride;
+                    i3 += (unsigned)((info >> 6) & 7) * slot_stride;
+                }
+                if (!P.analytic && (bz_in(xoff + (int64_t)i1, P.ncell) & bz_in(xoff + (int64_t)i2, P.ncell) &
+                                    bz_in(xoff + (int64_t)i3, P.ncell))) {
+                    f1 = __ldg(f_x + i1);
+                    f2 = __ldg(f_x + i2);
+                    f3 = __ldg(f_x + i3);
+                }
+            };
+            if (!GROUPS) legs(t0);
+            if (!P.analytic) fpp = __ldg(f_row + i4);
             float ma2 = md2, mc2 = md2;
             if constexpr (GROUPS) {
                 const float4 tmv0 = S.tm[t0];  // leg masses shared by the group's terms
                 ma2 = tmv0.x;
                 mc2 = tmv0.z;
             }
-            const float4 ga = S.ga[src], gb = S.gb[src];
-            const float Ep = ga.x;
-            const uint32_t i4 = __float_as_uint(ga.y);
+            const float4 gb = S.gb[src];
             const float E = Ep + E3;
             const float a2 = ga.w + ma2;
             const float E1 = sqrtf(a2 + z * z);
@@ -362,11 +401,7 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
             if (s <= 0.0f || t - mg2 >= 0.0f || uu - mg2 >= 0.0f) {
                 red_add(&P.flags[0], tn);
             } else {
-                const int2 gc = S.gc[src];
-                const unsigned lin1 = (gc.y & 0xffff) * P.np[2] + ((tg >> 8) & 0xff);
-                const unsigned lin2 = ((unsigned)gc.y >> 16) * P.np[2] + ((tg >> 16) & 0xff);
-                const unsigned lin3 = gc.x;
-                const float fpp = P.analytic ? f_equilibrium(P, d, Ep) : __ldg(f_row + i4);
+                if (P.analytic) fpp = f_equilibrium(P, d, Ep);
                 // |J| E1 E2 = sqrt(H) at a root of Eq. (work out delta E)
                 const float den = P.twopi5 * 16.0f * sqH * E3 * Ep;
                 if (MODE != M_RECORD && i4 != own_a) {
@@ -374,50 +409,42 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
                     own = 0;
                     own_a = i4;
                 }
+                long long q2 = 0;  // deposits to leg 2 of the terms that share it with the next one (sym < 0)
                 for (int k = 0; k < tn; ++k) {  // the group's terms: |M|^2, leg species, statistics
-                    float sym, M2;
-                    unsigned i1 = lin1, i2 = lin2, i3 = lin3;
-                    int info = 0;
+                    if (GROUPS) legs(t0 + k);
+                    const unsigned c1 = i1, c2 = i2, c3 = i3;
+                    float g1 = f1, g2 = f2, g3 = f3, sym, M2;
+                    const int tinfo = info;
                     if constexpr (GROUPS) {
-                        const int ti = t0 + k;
-                        sym = S.tm[ti].w;
-                        info = S.tinfo[ti];
-                        M2 = msq<float>(info >> 13, P, s, t, uu, mg2);
-                        i1 += (unsigned)(info & 7) * slot_stride;
-                        i2 += (unsigned)((info >> 3) & 7) * slot_stride;
-                        i3 += (unsigned)((info >> 6) & 7) * slot_stride;
+                        sym = S.tm[t0 + k].w;
+                        M2 = msq<float>(tinfo >> 13, P, s, t, uu, mg2);
                     } else {
                         sym = 0.5f;  // gg -> gg or qq -> qq: identical initial particles
                         M2 = msq<float>(d == 0 ? M_GG : M_QQ, P, s, t, uu, mg2);
                     }
-                    if (!(bz_in(xoff + (int64_t)i1, P.ncell) & bz_in(xoff + (int64_t)i2, P.ncell) &
-                          bz_in(xoff + (int64_t)i3, P.ncell) & bz_in(row + (int64_t)i4, P.ncell)))
+                    if (!(bz_in(xoff + (int64_t)c1, P.ncell) & bz_in(xoff + (int64_t)c2, P.ncell) &
+                          bz_in(xoff + (int64_t)c3, P.ncell) & bz_in(row + (int64_t)i4, P.ncell)))
                         continue;
-                    float f1, f2, f3;
                     if (P.analytic) {
                         const float E2 = E - E1;
-                        f1 = f_equilibrium(P, GROUPS ? P.slot_species[info & 7] : d, E1);
-                        f2 = f_equilibrium(P, GROUPS ? P.slot_species[(info >> 3) & 7] : d, E2);
-                        f3 = f_equilibrium(P, GROUPS ? P.slot_species[(info >> 6) & 7] : d, E3);
-                    } else {
-                        f1 = __ldg(f_x + i1);
-                        f2 = __ldg(f_x + i2);
-                        f3 = __ldg(f_x + i3);
+                        g1 = f_equilibrium(P, GROUPS ? P.slot_species[tinfo & 7] : d, E1);
+                        g2 = f_equilibrium(P, GROUPS ? P.slot_species[(tinfo >> 3) & 7] : d, E2);
+                        g3 = f_equilibrium(P, GROUPS ? P.slot_species[(tinfo >> 6) & 7] : d, E3);
                     }
                     float F1, F2, F3, Fp;
                     if constexpr (GROUPS) {
-                        F1 = (info & (1 << 9)) ? 1.0f - f1 : 1.0f + f1;
-                        F2 = (info & (1 << 10)) ? 1.0f - f2 : 1.0f + f2;
-                        F3 = (info & (1 << 11)) ? 1.0f - f3 : 1.0f + f3;
-                        Fp = (info & (1 << 12)) ? 1.0f - fpp : 1.0f + fpp;
+                        F1 = (tinfo & (1 << 9)) ? 1.0f - g1 : 1.0f + g1;
+                        F2 = (tinfo & (1 << 10)) ? 1.0f - g2 : 1.0f + g2;
+                        F3 = (tinfo & (1 << 11)) ? 1.0f - g3 : 1.0f + g3;
+                        Fp = (tinfo & (1 << 12)) ? 1.0f - fpp : 1.0f + fpp;
                     } else {
-                        F1 = fmaf(bf, f1, 1.0f);
-                        F2 = fmaf(bf, f2, 1.0f);
-                        F3 = fmaf(bf, f3, 1.0f);
+                        F1 = fmaf(bf, g1, 1.0f);
+                        F2 = fmaf(bf, g2, 1.0f);
+                        F3 = fmaf(bf, g3, 1.0f);
                         Fp = fmaf(bf, fpp, 1.0f);
                     }
-                    const float W = f1 * f2 * F3 * Fp - F1 * F2 * f3 * fpp;
-                    const float ct = div_approx(sym * W * M2, den);
+                    const float W = g1 * g2 * F3 * Fp - F1 * F2 * g3 * fpp;
+                    const float ct = div_approx(fabsf(sym) * W * M2, den);
                     const float wq = ct * P.Kown * (MODE == M_LEARNED ? S.wfac[src] : 1.0f);
                     if (MODE == M_RECORD) {  // record mode: sum |c~| per sample, no deposits
                         w_root += fabsf(ct);
@@ -432,9 +459,16 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
                         }
                         own += q;
                         if (q != 0 && P.sampler != 1) {
-                            red_add(&A_x[i3], q);
-                            red_add(&A_x[i1], -q);
-                            red_add(&A_x[i2], -q);
+                            red_add(&A_x[c3], q);
+                            red_add(&A_x[c1], -q);
+                            if (!MERGE) red_add(&A_x[c2], -q);
+                        }
+                        if (MERGE) {
+                            q2 += q;
+                            if (sym > 0.0f && q2 != 0 && P.sampler != 1) {
+                                red_add(&A_x[c2], -q2);
+                                q2 = 0;
+                            }
                         }
                     }
                 }
@@ -847,7 +881,7 @@ __device__ __forceinline__ void collide_unit(const CollideArgs<float>& P, int64_
 // block in the constant bank, the batch with each box's block in global
 // memory): a box gives the same bits alone or inside a batch.
 template <int MODE, bool GROUPS, bool BATCH>
-__global__ void __launch_bounds__(32 * WARPS, (GROUPS && !BATCH) ? BZ_F32_MIN_BLOCKS_GROUPED : BZ_F32_MIN_BLOCKS)
+__global__ void __launch_bounds__(32 * WARPS, (GROUPS && !BATCH && MODE != M_LEARNED) ? BZ_F32_MIN_BLOCKS_GROUPED : BZ_F32_MIN_BLOCKS)
     k_collide_f32(const __grid_constant__ CollideArgs<float> one, const CollideArgs<float>* __restrict__ boxes,
                   const int64_t* __restrict__ prefix, int nboxes, unsigned long long* counter, const int* step_dev,
                   int chunk, int* qcount, unsigned long long* qitems, long long qcap)
