@@ -1380,7 +1380,7 @@ extern "C" int bz_step(bz_handle h, int64_t* state, double dt, int32_t nsteps, i
 // Batched ensemble: independent homogeneous boxes of any grid size, species
 // set, coupling and sample count, stepped together.  Per step: thermal
 // masses of every box (one launch), f of the concatenated state (one
-// launch), collision of every (box, anchor, 32 samples) unit in one
+// launch), collision of every box's units of samples in one
 // persistent launch with dynamic work distribution, float-float fixup of queued
 // terms, moments, and the end-of-step bookkeeping; the step is captured
 // once as a CUDA graph and replayed, the step index living in device memory.

@@ -5,7 +5,8 @@
 // roundTiesToEven) for finite operands whose results stay normal; the
 // callers keep to that range and fall back to FP64 instructions outside it.
 // On this GPU FP64 instructions, conversions included, issue at 1/64 of the
-// FP32 rate, so the thermal-mass sums take this path for their products.
+// FP32 rate, so the FP64 collision kernel takes this path for the rounding of its
+// weights.
 // The header also compiles as plain C++ (the host unit test checks it
 // against the host's double arithmetic).
 #pragma once

@@ -1069,13 +1069,14 @@ __device__ __noinline__ long long fixup_term_ff(const CollideArgs<float>& P, int
         pc.x = -1;
         pc.L = ff_from_double(P.L64);
         pc.nL = ff_neg(pc.L);
-        pc.twoL = ff_from_double(2.0 * P.L64);
+        pc.twoL = {2.0f * pc.L.hi, 2.0f * pc.L.lo};
         for (int i = 0; i < 3; ++i) pc.dp[i] = ff_from_double(P.dp64[i]);
     }
     if (pc.x != x) {
         pc.x = x;
-        for (int i = 0; i < 4; ++i) pc.m2[i] = P.mass_mode == 1 ? ff{0.0f, 0.0f} : ff_from_double(P.m2[x * 4 + i]);
         pc.mg2 = ff_from_double(P.m2[x * 4]);
+        pc.m2[0] = P.mass_mode == 1 ? ff{0.0f, 0.0f} : pc.mg2;
+        for (int i = 1; i < 4; ++i) pc.m2[i] = P.mass_mode == 1 ? ff{0.0f, 0.0f} : ff_from_double(P.m2[x * 4 + i]);
     }
     const ff L = pc.L, nL = pc.nL, twoL = pc.twoL;
     const ff dp[3] = {pc.dp[0], pc.dp[1], pc.dp[2]};
