@@ -399,12 +399,9 @@ def run_bz(args):
     result = None
     if rank == 0:
         coll_ms, coll_n = prof["collide"]
-        drift_kernels = 2 if w.nxc > 1 else 1   # k_mass_table + the drift kernel on inhomogeneous grids
-        nsm_ = torch.cuda.get_device_properties(local).multi_processor_count
-        # k_moments + k_moments_finish when few (x cell, slot) rows are split into p-cell chunks
-        mom_kernels = 2 if (w.nxc * w.nslots < 2 * nsm_ and w.npc // 1024 > 1) else 1
-        launches = (2 * prof["masses"][1] + drift_kernels * prof["drift"][1] + prof["collide"][1]
-                    + prof["fixup"][1] + mom_kernels * prof["moments"][1] + prof["convert"][1])
+        drift_kernels = 2 if w.nxc > 1 else 1   # the inverse energies + the drift kernel on inhomogeneous grids
+        launches = (prof["masses"][1] + drift_kernels * prof["drift"][1] + prof["collide"][1]
+                    + prof["fixup"][1] + prof["moments"][1] + prof["convert"][1])
         # algorithmic work of one collision launch
         cpu_rate, cpu_anchors, cores, cpu_secs, roots_per_term, cpu_stride = (None,) * 6
         if not args.no_cpu_baseline and world == 1:
@@ -535,7 +532,7 @@ def measured_hbm_gbs():
 
 
 def transport_rooflines(h, w, state, mom, prof, steps, stream, barrier):
-    """Drift (k_mass_table + drift kernel; algorithmic bytes 8 B read + 8 B
+    """Drift (inverse energies + drift kernel; algorithmic bytes 8 B read + 8 B
     write + 4 B f per cell), moments and thermal masses (8 B read per cell
     each) of the timed steps against the HBM peak, and the drift with the
     force term switched on, timed over separate calls."""

@@ -284,7 +284,7 @@ int bz_profile_read(bz_handle h, double* ms_host, int64_t* launches_host, int32_
  * integrand.  Each step runs the whole hot path of every box -- masses
  * (Eqs. mg, mq), collision sampling with symmetrical deposition (Eqs. ca,
  * small c relation) into the state in place, moments -- as one persistent
- * collision launch (warps take chunks of (box, anchor, 32 samples) units
+ * collision launch (warps take chunks of units of a box's samples
  * from a global counter, so ragged boxes share the GPU evenly) inside one
  * captured CUDA graph that is replayed every step.
  * ------------------------------------------------------------------------ */
@@ -392,7 +392,7 @@ int bz_proposal_init(bz_handle h, uint64_t seed);
 int bz_proposal_get_params(bz_handle h, float* host);
 int bz_proposal_set_params(bz_handle h, const float* host);
 /* Uniform FP32 sampling of state in record mode: no deposits, no FP64
- * re-evaluation; for every unit (anchor, 32 samples) whose index is a
+ * re-evaluation; for every unit of an anchor's samples whose index is a
  * multiple of unit_stride one record is appended to records (device,
  * max_records) for each sample with w > 0 (samples whose roots were all
  * rejected or fell outside the box carry no information and are skipped).
@@ -442,7 +442,7 @@ int bz_load(bz_handle h, int64_t* state, int64_t* step, const char* path);
 
 /* Bounds-checked builds (compiled with -DBZ_CHECK=1, a stand-in for a
  * memory sanitizer): the collision (FP64, FP32 and its re-evaluation) and the
- * drift kernels (streaming and row forms) test every index they compute into f, A, the
+ * drift kernels (mirrored and row forms) test every index they compute into f, A, the
  * state and the mass table before the access, skip an access outside its
  * buffer and count it.  count: indices outside their buffers since the
  * last reset (host, may be NULL); first_bad: one of them, -1 if none (host,
