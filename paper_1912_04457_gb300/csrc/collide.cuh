@@ -25,6 +25,7 @@
 #pragma once
 #include <cstdint>
 #include "bz_internal.h"
+#include "exact64.cuh"
 
 namespace bz {
 
@@ -166,9 +167,9 @@ __device__ __forceinline__ R upow(R x, int n)
     return r;
 }
 
-// a / b: FP64 as written; FP32 by the hardware reciprocal (the arguments are
+// a / b: FP64 as written (the same bits by integer instructions); FP32 by the hardware reciprocal (the arguments are
 // far from its range limits), without the scaling of the approximate division.
-__device__ __forceinline__ double div_approx(double a, double b) { return a / b; }
+__device__ __forceinline__ double div_approx(double a, double b) { return div64(a, b); }
 __device__ __forceinline__ float div_approx(float a, float b)
 {
     float r;

@@ -13,7 +13,9 @@
 // root) candidates -- 0.37 a sample and term -- are evaluated by full warps with
 // the operations of eval_term.  Collision kernel: 20^3 gluons, N = 64, 618 ->
 // 133 us; 7 species, 12 x 13 x 10, N = 100, 9.8 -> 1.5 ms; 4^3 x 20^3 gluons, N =
-// 128, 74.6 -> 11.9 ms; about 80% of the FP64 pipe's cycles are then in use.
+// 128, 74.6 -> 11.9 ms; about 80% of the FP64 pipe's cycles were then in use, two
+// fifths of them by divisions and square roots.  Those are evaluated by integer
+// digits (div64, sqrt64: the same bits): 90 us, 0.88 ms and 7.7 ms.
 #include "collide.cuh"
 #include "exact64.cuh"
 
@@ -159,7 +161,7 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
             const bool second = (e >> 12) & 1u;
             const double ma2 = S.tma[ti], mb2 = S.tmb[ti], mc2 = S.tmc[ti];
             const double Ep = S.g[0][src], Pz = S.g[1][src];
-            const double E3 = sqrt(S.g[5][src] + mc2);
+            const double E3 = sqrt64(S.g[5][src] + mc2);
             const double E = Ep + E3;
             const double a2 = S.g[3][src] + ma2;
             const double b2 = S.g[4][src] + mb2;
@@ -170,22 +172,22 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
             const double H = kk - a2 * D;
             bool ok = !(lt0(H) || le0(D));
             const double kp = kap * Pz;
-            const double sq = E * sqrt(ok ? H : 0.0);
+            const double sq = E * sqrt64(ok ? H : 0.0);
             const double Q = ge0(kp) ? kp + sq : kp - sq;
             ok = ok && (dbits(Q) << 1) != 0ull;
             if (ok) {
                 const double zn = second ? EE * a2 - kk : Q, zd = second ? Q : D;
-                const double z = zn / zd;
+                const double z = div64(zn, zd);
                 // 0 < E1 < E with E1 = (kap + Pz z)/E: by the numerator's sign, and against
                 // E^2 unless it is within 256 units in the last place of it
                 const double w = kap + Pz * z;
                 const long long far = (long long)(dbits(EE) - dbits(w));
-                const bool e1ok = (long long)dbits(w) > 0 && (far > 256 || (far >= -256 && w / E < E));
+                const bool e1ok = (long long)dbits(w) > 0 && (far > 256 || (far >= -256 && div64(w, E) < E));
                 const double dz = Pz - z;
                 if (e1ok && in_box64(z, L) && in_box64(dz, L)) {
-                    const double E1 = sqrt(a2 + z * z);
-                    const double E2 = sqrt(b2 + dz * dz);
-                    const double J = z / E1 - dz / E2;
+                    const double E1 = sqrt64(a2 + z * z);
+                    const double E2 = sqrt64(b2 + dz * dz);
+                    const double J = div64(z, E1) - div64(dz, E2);
                     const double s = EE - S.g[2][src];
                     const double k1k3 = S.g[6][src] + z * S.g[7][src];
                     const double k1p = S.g[8][src] + z * S.g[9][src];
@@ -228,7 +230,7 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
                             const double gain = f1 * f2 * F3 * Fp;
                             const double W = gain - F1 * F2 * f3 * fp;
                             const double den = fabs(J) * P.twopi5 * 16.0 * E1 * E2 * E3 * Ep;
-                            const double ct = S.tsym[ti] * W * M2 / den;
+                            const double ct = div64(S.tsym[ti] * W * M2, den);
                             const double wq = ct * P.Kown;
                             long long q = 0;
                             if ((dbits(wq) & ~SIGN64) >= dbits(Ops<double>::LIM)) {
@@ -358,7 +360,7 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
                         const double PP = (Px * Px + Py * Py) + Pz * Pz;
                         const double bx = Px - k[0], by = Py - k[1];
                         const double a2m = k[0] * k[0] + k[1] * k[1], b2m = bx * bx + by * by;
-                        const double Ep = sqrt(pp + md2);
+                        const double Ep = sqrt64(pp + md2);
                         S.g[0][sb] = Ep;
                         S.g[1][sb] = Pz;
                         S.g[2][sb] = PP;
