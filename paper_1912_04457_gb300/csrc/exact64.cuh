@@ -20,10 +20,6 @@
 #define BZ_HD __host__ __device__ __forceinline__
 #endif
 
-#ifndef BZ_DIV64
-#define BZ_DIV64 static __device__ __noinline__
-#endif
-
 namespace bz {
 
 struct Exact64 {
@@ -280,20 +276,55 @@ BZ_HD bool x64_sqrt(uint64_t a, uint64_t& out)
     return true;
 }
 
+// a b; false (out unset) unless one is +-0 and the other finite, or both and the product
+// are safely normal
+BZ_HD bool x64_mul(uint64_t a, uint64_t b, uint64_t& out)
+{
+    const uint32_t ah = (uint32_t)(a >> 32), bh = (uint32_t)(b >> 32), a0 = (uint32_t)a, b0 = (uint32_t)b;
+    const uint32_t ea = (ah >> 20) & 0x7FFu, eb = (bh >> 20) & 0x7FFu, sign = (ah ^ bh) & 0x80000000u;
+    const int e = (int)(ea + eb) - 1023;  // of a product of mantissas in [1, 2)
+    if (ea - 1u >= 2046u || eb - 1u >= 2046u || (unsigned)(e - 2) >= 2043u) {
+        const bool az = (a << 1) == 0, bz = (b << 1) == 0;
+        if (!((az && eb != 0x7FFu) || (bz && ea != 0x7FFu))) return false;
+        out = (uint64_t)sign << 32;
+        return true;
+    }
+    const uint32_t a1 = (ah & 0xFFFFFu) | 0x100000u, b1 = (bh & 0xFFFFFu) | 0x100000u;
+    const uint64_t p0 = (uint64_t)a0 * b0;
+    uint64_t mid = (uint64_t)a1 * b0 + (p0 >> 32);
+    mid = (uint64_t)a0 * b1 + mid;
+    uint64_t top = (uint64_t)a1 * b1 + (mid >> 32);  // product = top 2^64 + (mid mod 2^32) 2^32 + (p0 mod 2^32)
+    const uint32_t lo = (uint32_t)p0, ml = (uint32_t)mid;
+    const int two = (int)((uint32_t)(top >> 41) & 1u);  // mantissa product >= 2
+    const int sh = 20 + two;                            // bits of ml below the result
+    const uint64_t m = (top << (32 - sh)) | (ml >> sh);
+    const uint32_t half = 1u << (sh - 1), rest = ml & (2u * half - 1u);
+    const bool up = rest > half || (rest == half && (lo != 0u || (m & 1u)));
+    out = ((uint64_t)(sign + ((uint32_t)(e - 1 + two) << 20)) << 32) + m + (up ? 1u : 0u);
+    return true;
+}
+
 #ifdef __CUDACC__
+static __device__ __noinline__ double mul64_slow(double a, double b) { return a * b; }
+static __device__ __noinline__ double mul64(double a, double b)
+{
+    uint64_t o;
+    if (x64_mul((uint64_t)__double_as_longlong(a), (uint64_t)__double_as_longlong(b), o)) return __longlong_as_double((long long)o);
+    return mul64_slow(a, b);
+}
 static __device__ __noinline__ double div64_slow(double a, double b) { return a / b; }
 static __device__ __noinline__ double sqrt64_slow(double a) { return sqrt(a); }
 // a / b and sqrt(a) as the FP64 instructions give them, without those: some 70 integer
 // and FP32 instructions (150 cycles) for nine or ten of 64 cycles.  Calls, not inlined: a
 // root's dozen copies overflow the instruction cache (7 species, 12 x 13 x 10: 1.07 against
 // 0.88 ms).
-BZ_DIV64 double div64(double a, double b)
+static __device__ __noinline__ double div64(double a, double b)
 {
     uint64_t o;
     if (x64_div((uint64_t)__double_as_longlong(a), (uint64_t)__double_as_longlong(b), o)) return __longlong_as_double((long long)o);
     return div64_slow(a, b);
 }
-BZ_DIV64 double sqrt64(double a)
+static __device__ __noinline__ double sqrt64(double a)
 {
     uint64_t o;
     if (x64_sqrt((uint64_t)__double_as_longlong(a), o)) return __longlong_as_double((long long)o);

@@ -15,7 +15,9 @@
 // 133 us; 7 species, 12 x 13 x 10, N = 100, 9.8 -> 1.5 ms; 4^3 x 20^3 gluons, N =
 // 128, 74.6 -> 11.9 ms; about 80% of the FP64 pipe's cycles were then in use, two
 // fifths of them by divisions and square roots.  Those are evaluated by integer
-// digits (div64, sqrt64: the same bits): 90 us, 0.88 ms and 7.7 ms.
+// digits (div64, sqrt64: the same bits): 90 us, 0.88 ms and 7.7 ms.  The products of
+// the geometry, which every live sample takes, too (mul64): 88 us, 0.87 ms and 7.1 ms;
+// with the roots' products as well 102 us, 0.94 ms and 8.0 ms.
 #include "collide.cuh"
 #include "exact64.cuh"
 
@@ -354,12 +356,12 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
                         for (int i = 0; i < 3; ++i) p[i] = ac.p[i] + P.dp[i] * (one_plus_u(w[i], half) - 1.5);  // u - 1/2, exact
 #pragma unroll
                         for (int i = 0; i < 5; ++i) k[i] = -L + twoL * (one_plus_u(w[3 + i], half) - 1.0);  // k1x, k1y, k3
-                        const double pp = (p[0] * p[0] + p[1] * p[1]) + p[2] * p[2];
-                        const double kk3 = (k[2] * k[2] + k[3] * k[3]) + k[4] * k[4];
+                        const double pp = (mul64(p[0], p[0]) + mul64(p[1], p[1])) + mul64(p[2], p[2]);
+                        const double kk3 = (mul64(k[2], k[2]) + mul64(k[3], k[3])) + mul64(k[4], k[4]);
                         const double Px = p[0] + k[2], Py = p[1] + k[3], Pz = p[2] + k[4];
-                        const double PP = (Px * Px + Py * Py) + Pz * Pz;
+                        const double PP = (mul64(Px, Px) + mul64(Py, Py)) + mul64(Pz, Pz);
                         const double bx = Px - k[0], by = Py - k[1];
-                        const double a2m = k[0] * k[0] + k[1] * k[1], b2m = bx * bx + by * by;
+                        const double a2m = mul64(k[0], k[0]) + mul64(k[1], k[1]), b2m = mul64(bx, bx) + mul64(by, by);
                         const double Ep = sqrt64(pp + md2);
                         S.g[0][sb] = Ep;
                         S.g[1][sb] = Pz;
@@ -367,9 +369,9 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
                         S.g[3][sb] = a2m;
                         S.g[4][sb] = b2m;
                         S.g[5][sb] = kk3;
-                        S.g[6][sb] = k[0] * k[2] + k[1] * k[3];
+                        S.g[6][sb] = mul64(k[0], k[2]) + mul64(k[1], k[3]);
                         S.g[7][sb] = k[4];
-                        S.g[8][sb] = k[0] * p[0] + k[1] * p[1];
+                        S.g[8][sb] = mul64(k[0], p[0]) + mul64(k[1], p[1]);
                         S.g[9][sb] = p[2];
                         auto bin = [&](uint32_t v, unsigned n) {  // floor(u n), exactly
                             return (int)(((2ull * v + odd) * n) >> 33);

@@ -1,5 +1,5 @@
-// Host check of x64_div and x64_sqrt (exact64.cuh) against the host's IEEE division and
-// square root, with the FP32 estimates off by up to two units in the last place either
+// Host check of x64_mul, x64_div and x64_sqrt (exact64.cuh) against the host's IEEE
+// operations, the latter two with the FP32 estimates off by up to two units in the last place either
 // way.  Prints the number of cases and of mismatches; exit status 1 on any mismatch.
 #include <cmath>
 #include <cstdint>
@@ -61,6 +61,15 @@ int main(int argc, char** argv)
         if (x64_div(a, b, o)) {
             ++taken;
             r = y / x;
+            std::memcpy(&e, &r, sizeof e);
+            bad += o != e;
+        }
+        if (rng() % 64 == 0) b = (uint64_t)(rng() & 1) << 63;
+        std::memcpy(&x, &b, sizeof x);
+        ++cases;
+        if (x64_mul(a, b, o)) {
+            ++taken;
+            r = y * x;
             std::memcpy(&e, &r, sizeof e);
             bad += o != e;
         }
