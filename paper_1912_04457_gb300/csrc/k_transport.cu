@@ -4,6 +4,7 @@
 // which threads accumulate.
 #include <cstdint>
 #include "bz_internal.h"
+#include "exact64.cuh"
 #include "intconv.cuh"
 
 namespace bz {
@@ -83,12 +84,12 @@ __device__ __forceinline__ void masses_block(const MassArgs& P, int64_t x, int64
             nsp[s] = sl < 0 ? 0 : P.state[((int64_t)sl * P.nxc + x) * P.npc + j];
         }
         const double ng = skip_g ? 0.0 : (double)nsp[0];
-        const double rg = skip_g ? 0.0 : 0.5 / sqrt(pp + m2p[0]);
+        const double rg = skip_g ? 0.0 : div64(0.5, sqrt64(pp + m2p[0]));
         double q[3], rq[3];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             q[i] = skip_q[i] ? 0.0 : (double)(nsp[1 + i] + nsp[4 + i]);
-            rq[i] = skip_q[i] ? 0.0 : 0.5 / sqrt(pp + m2p[1 + i]);
+            rq[i] = skip_q[i] ? 0.0 : div64(0.5, sqrt64(pp + m2p[1 + i]));
         }
         const double g3 = 9.0 * ng * rg + 4.0 * ((q[0] * rq[0] + q[1] * rq[1]) + q[2] * rq[2]);
         const long long qg = __double2ll_rn(g3 * MASS_FX);
@@ -148,7 +149,9 @@ __device__ __forceinline__ float ll2float_fast(long long n)
 // which issues for 64 cycles.  The products are 64 x 47 bits, cut to 32 fraction
 // bits.  Gluons only (GLUON_ONLY): one rounding of one product, 9 n R_g and 3 n R_g.
 // 16^3 x 20^3 gluons, all bins nonzero: 410 -> 142 us (99 instructions a bin, a third
-// of them multiplications; 262 MB are read); 8^3 x 16^3, 7 species: 168 -> 78 us.
+// of them multiplications; 262 MB are read); 8^3 x 16^3, 7 species: 168 -> 78 us.  The
+// tables' roots and quotients by integer digits (div64, sqrt64: the same bits): 134 and 61
+// us, a 32^3 grid of 7 species 25 -> 17 us, 64^3 without the table 238 -> 107 us.
 // m_a^2 (i = 0 gluon, 1..3 flavours) from its exact fixed-point sum
 __device__ __forceinline__ double mass_of(const MassArgs& P, int i, long long acc)
 {
@@ -247,7 +250,7 @@ __global__ void __launch_bounds__(MASS_THREADS, 4) k_masses_tab(const __grid_con
         for (int s = 0; s < NS; ++s) {
             uint64_t R = 0;
             if (!skip[s]) {
-                const uint64_t b = (uint64_t)__double_as_longlong(0.5 / sqrt(pp + m2p[s]));
+                const uint64_t b = (uint64_t)__double_as_longlong(div64(0.5, sqrt64(pp + m2p[s])));
                 const int be = (int)(b >> 52);  // r > 0 (a NaN or negative value fails the range)
                 const uint64_t M = (b & ((1ull << 52) - 1ull)) | (1ull << 52);
                 ok &= be >= 958 && be < 1031;  // 2^-65 <= r < 2^8
