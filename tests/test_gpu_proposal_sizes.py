@@ -66,3 +66,17 @@ def test_inference(np_, mask):
     O_, _ = mlp.forward(params.astype(np.float64), X)
     ref = mlp.head(O_[:, :6])
     assert np.abs(got[:, :6] - ref[:, :6]).max() < 5e-3
+
+
+def test_losses_beyond_one_copy():
+    """More steps than the device buffer of losses holds (4096): one call against two."""
+    from paper_1912_04457_gb300 import bz
+    out = []
+    _, dev = _records(5000, 7 * 216, 6)
+    for calls in ([4100], [3000, 1100]):
+        h = bz.Handle(np_=(6, 6, 6), L=2.0, species_mask=0x7F)
+        h.set_proposal_params(mlp.init_params(7))
+        losses = np.concatenate([h.proposal_train(dev, 5000, k, 128, 1e-4) for k in calls])
+        out.append((losses, h.proposal_params()))
+    assert np.array_equal(out[0][0], out[1][0]) and np.all(np.isfinite(out[0][0]))
+    assert np.array_equal(out[0][1], out[1][1])
