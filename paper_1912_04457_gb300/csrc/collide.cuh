@@ -193,10 +193,10 @@ __device__ __forceinline__ R msq_user(const UserRow* row, R s, R t, R u, R mg2)
     return acc;
 }
 
-template <typename R>
+template <typename R, bool USER = true>  // USER: rows may be user-defined
 __device__ __forceinline__ R msq(int cls, const CollideArgs<R>& P, R s, R t, R u, R mg2)
 {
-    if ((P.umask >> cls) & 1u) return msq_user<R>(P.urows + cls, s, t, u, mg2);
+    if (USER && ((P.umask >> cls) & 1u)) return msq_user<R>(P.urows + cls, s, t, u, mg2);
     R tm = t - mg2, um = u - mg2;
     switch (cls) {
     case M_QQP:

@@ -258,7 +258,7 @@ __device__ __forceinline__ uint4 draw(const CollideArgs<float>& P, uint32_t c0, 
     return SINGLE ? philox_tail_ks(c0, head, P.ks) : philox_tail(c0, head, P.key0, P.key1);
 }
 
-template <int MODE, bool GROUPS, bool SINGLE>
+template <int MODE, bool GROUPS, bool SINGLE, bool PLAIN>
 __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t unit, uint32_t a_first, uint32_t a_stop, int c0,
                                             int c1, int step, WarpSmem<MODE, GROUPS>& S, DeferCtx& dq,
                                             unsigned long long box_tag)
@@ -295,6 +295,7 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
     // the uniform one gains where f is of order 1 everywhere (32^3: 15.2 -> 14.7 ms) and
     // loses where most of its roots deposit nothing (12.5 -> 13.1 ms), so it does not.
     constexpr bool MERGE = MODE == M_LEARNED;
+    const bool analytic = !PLAIN && SINGLE && P.analytic;  // (a batch's boxes hold states)
     const int nt = GROUPS ? P.nterms[d] : 1;
     if constexpr (GROUPS) {
         // kinematic groups: consecutive terms with equal leg masses (the first
@@ -374,7 +375,7 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
                     i2 += (unsigned)((info >> 3) & 7) * slot_stride;
                     i3 += (unsigned)((info >> 6) & 7) * slot_stride;
                 }
-                if (!P.analytic && (bz_in(xoff + (int64_t)i1, P.ncell) & bz_in(xoff + (int64_t)i2, P.ncell) &
+                if (!analytic && (bz_in(xoff + (int64_t)i1, P.ncell) & bz_in(xoff + (int64_t)i2, P.ncell) &
                                     bz_in(xoff + (int64_t)i3, P.ncell))) {
                     f1 = __ldg(f_x + i1);
                     f2 = __ldg(f_x + i2);
@@ -382,7 +383,7 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
                 }
             };
             if (!GROUPS) legs(t0);
-            if (!P.analytic) fpp = __ldg(f_row + i4);
+            if (!analytic) fpp = __ldg(f_row + i4);
             float ma2 = md2, mc2 = md2;
             if constexpr (GROUPS) {
                 const float4 tmv0 = S.tm[t0];  // leg masses shared by the group's terms
@@ -401,7 +402,7 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
             if (s <= 0.0f || t - mg2 >= 0.0f || uu - mg2 >= 0.0f) {
                 red_add(&P.flags[0], tn);
             } else {
-                if (P.analytic) fpp = f_equilibrium(P, d, Ep);
+                if (analytic) fpp = f_equilibrium(P, d, Ep);
                 // |J| E1 E2 = sqrt(H) at a root of Eq. (work out delta E)
                 const float den = P.twopi5 * 16.0f * sqH * E3 * Ep;
                 if (MODE != M_RECORD && i4 != own_a) {
@@ -417,15 +418,15 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
                     const int tinfo = info;
                     if constexpr (GROUPS) {
                         sym = S.tm[t0 + k].w;
-                        M2 = msq<float>(tinfo >> 13, P, s, t, uu, mg2);
+                        M2 = msq<float, !PLAIN>(tinfo >> 13, P, s, t, uu, mg2);
                     } else {
                         sym = 0.5f;  // gg -> gg or qq -> qq: identical initial particles
-                        M2 = msq<float>(d == 0 ? M_GG : M_QQ, P, s, t, uu, mg2);
+                        M2 = msq<float, !PLAIN>(d == 0 ? M_GG : M_QQ, P, s, t, uu, mg2);
                     }
                     if (!(bz_in(xoff + (int64_t)c1, P.ncell) & bz_in(xoff + (int64_t)c2, P.ncell) &
                           bz_in(xoff + (int64_t)c3, P.ncell) & bz_in(row + (int64_t)i4, P.ncell)))
                         continue;
-                    if (P.analytic) {
+                    if (analytic) {
                         const float E2 = E - E1;
                         g1 = f_equilibrium(P, GROUPS ? P.slot_species[tinfo & 7] : d, E1);
                         g2 = f_equilibrium(P, GROUPS ? P.slot_species[(tinfo >> 3) & 7] : d, E2);
@@ -458,14 +459,14 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
                                 red_add(&P.flags[1], 1);
                         }
                         own += q;
-                        if (q != 0 && P.sampler != 1) {
+                        if (q != 0 && (PLAIN || P.sampler != 1)) {
                             red_add(&A_x[c3], q);
                             red_add(&A_x[c1], -q);
                             if (!MERGE) red_add(&A_x[c2], -q);
                         }
                         if (MERGE) {
                             q2 += q;
-                            if (sym > 0.0f && q2 != 0 && P.sampler != 1) {
+                            if (sym > 0.0f && q2 != 0 && (PLAIN || P.sampler != 1)) {
                                 red_add(&A_x[c2], -q2);
                                 q2 = 0;
                             }
@@ -839,7 +840,7 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
 }
 
 // The rows of a unit: its anchors (a_offset + i a_stride, increasing) row by row.
-template <int MODE, bool GROUPS, bool SINGLE>
+template <int MODE, bool GROUPS, bool SINGLE, bool PLAIN>
 __device__ __forceinline__ void collide_unit(const CollideArgs<float>& P, int64_t unit, int step, WarpSmem<MODE, GROUPS>& S,
                                              DeferCtx& dq, unsigned long long box_tag)
 {
@@ -861,7 +862,7 @@ __device__ __forceinline__ void collide_unit(const CollideArgs<float>& P, int64_
         // end of a's row: rows are npc cells each, in increasing order
         const uint32_t row_end = (udiv(a, P.dv_npc) + 1) * (uint32_t)P.npc;
         const uint32_t stop = min(row_end, a_end);
-        collide_row<MODE, GROUPS, SINGLE>(P, unit, a, stop, c0, c1, step, S, dq, box_tag);
+        collide_row<MODE, GROUPS, SINGLE, PLAIN>(P, unit, a, stop, c0, c1, step, S, dq, box_tag);
         if (stop == a_end) break;
         a += (stop - a + (uint32_t)P.a_stride - 1) / (uint32_t)P.a_stride * (uint32_t)P.a_stride;
     } while (a < a_end);
@@ -880,7 +881,11 @@ __device__ __forceinline__ void collide_unit(const CollideArgs<float>& P, int64_
 // Both run the same collide_unit source (the single box with its argument
 // block in the constant bank, the batch with each box's block in global
 // memory): a box gives the same bits alone or inside a batch.
-template <int MODE, bool GROUPS, bool BATCH>
+// PLAIN: f from the state, no user-defined |M|^2 row, all legs deposited: without the
+// code of the other forms (what a launch takes is chosen by launch_collide_f32; 32^3,
+// seven species: 12.53 -> 11.81 ms, 5 x 3 x 7 x cells, four species: 3.61 -> 3.48, 16^3 x 20^3 gluons: 101.8 ->
+// 99.7, learned 16^3 of seven species: 861 -> 809 us).
+template <int MODE, bool GROUPS, bool BATCH, bool PLAIN>
 __global__ void __launch_bounds__(32 * WARPS, (GROUPS && !BATCH && MODE != M_LEARNED) ? BZ_F32_MIN_BLOCKS_GROUPED : BZ_F32_MIN_BLOCKS)
     k_collide_f32(const __grid_constant__ CollideArgs<float> one, const CollideArgs<float>* __restrict__ boxes,
                   const int64_t* __restrict__ prefix, int nboxes, unsigned long long* counter, const int* step_dev,
@@ -930,10 +935,10 @@ __global__ void __launch_bounds__(32 * WARPS, (GROUPS && !BATCH && MODE != M_LEA
         // from the constant bank, a batch box from global memory; the
         // arithmetic is the same source, so a box gives the same bits either way
         if (BATCH)
-            collide_unit<MODE, GROUPS, false>(boxes[b], u - prefix[b], step, smem[warp], dq,
+            collide_unit<MODE, GROUPS, false, PLAIN>(boxes[b], u - prefix[b], step, smem[warp], dq,
                                               (unsigned long long)b << 48);
         else
-            collide_unit<MODE, GROUPS, true>(one, u, step, smem[warp], dq, 0ull);
+            collide_unit<MODE, GROUPS, true, PLAIN>(one, u, step, smem[warp], dq, 0ull);
         u += dyn ? 1 : nwarps;
     }
     __syncwarp();
@@ -964,11 +969,13 @@ cudaError_t check_read_collide_f32(unsigned long long out[2], bool reset)
 }
 
 // The instantiation a single-box launch runs, and its resident blocks per SM.
-template <int MODE, bool GROUPS>
+static bool is_plain(const CollideArgs<float>& a) { return !a.analytic && !a.umask && a.sampler != 1; }
+
+template <int MODE, bool GROUPS, bool PLAIN>
 static int resident_blocks()
 {
     static int n = 0;
-    if (!n && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_collide_f32<MODE, GROUPS, false>, 32 * WARPS, 0) !=
+    if (!n && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_collide_f32<MODE, GROUPS, false, PLAIN>, 32 * WARPS, 0) !=
                    cudaSuccess || n < 1))
         n = 1;
     return n;
@@ -976,34 +983,36 @@ static int resident_blocks()
 
 int collide_f32_resident_blocks(const CollideArgs<float>& a)
 {
-    if (a.rec_stride) return resident_blocks<M_RECORD, true>();
-    if (a.sampler == SAMPLER_LEARNED) return resident_blocks<M_LEARNED, true>();
-    return has_groups(a) ? resident_blocks<M_UNIFORM, true>() : resident_blocks<M_UNIFORM, false>();
+    const bool plain = is_plain(a);
+    if (a.rec_stride) return resident_blocks<M_RECORD, true, false>();
+    if (a.sampler == SAMPLER_LEARNED)
+        return plain ? resident_blocks<M_LEARNED, true, true>() : resident_blocks<M_LEARNED, true, false>();
+    if (has_groups(a)) return plain ? resident_blocks<M_UNIFORM, true, true>() : resident_blocks<M_UNIFORM, true, false>();
+    return plain ? resident_blocks<M_UNIFORM, false, true>() : resident_blocks<M_UNIFORM, false, false>();
 }
 
 cudaError_t launch_collide_f32(const CollideArgs<float>& a, int grid, unsigned long long* counter, cudaStream_t s)
 {
+    auto run = [&](auto kernel) {
+        kernel<<<grid, 32 * WARPS, 0, s>>>(a, nullptr, nullptr, 0, counter, nullptr, 1, a.qcount, a.qitems, a.qcap);
+    };
+    const bool plain = is_plain(a);
     if (a.rec_stride)
-        k_collide_f32<M_RECORD, true, false><<<grid, 32 * WARPS, 0, s>>>(a, nullptr, nullptr, 0, counter, nullptr, 1, a.qcount,
-                                                                   a.qitems, a.qcap);
+        run(k_collide_f32<M_RECORD, true, false, false>);
     else if (a.sampler == SAMPLER_LEARNED)
-        k_collide_f32<M_LEARNED, true, false><<<grid, 32 * WARPS, 0, s>>>(a, nullptr, nullptr, 0, counter, nullptr, 1, a.qcount,
-                                                                    a.qitems, a.qcap);
+        plain ? run(k_collide_f32<M_LEARNED, true, false, true>) : run(k_collide_f32<M_LEARNED, true, false, false>);
     else if (has_groups(a))
-        k_collide_f32<M_UNIFORM, true, false><<<grid, 32 * WARPS, 0, s>>>(a, nullptr, nullptr, 0, counter, nullptr, 1, a.qcount,
-                                                                    a.qitems, a.qcap);
+        plain ? run(k_collide_f32<M_UNIFORM, true, false, true>) : run(k_collide_f32<M_UNIFORM, true, false, false>);
     else
-        k_collide_f32<M_UNIFORM, false, false><<<grid, 32 * WARPS, 0, s>>>(a, nullptr, nullptr, 0, counter, nullptr, 1,
-                                                                     a.qcount, a.qitems, a.qcap);
+        plain ? run(k_collide_f32<M_UNIFORM, false, false, true>) : run(k_collide_f32<M_UNIFORM, false, false, false>);
     return cudaGetLastError();
 }
-
 cudaError_t launch_collide_f32_batch(const CollideArgs<float>* boxes, const int64_t* prefix, int nboxes,
                                      unsigned long long* counter, const int* step_dev, int chunk, int grid,
                                      int* qcount, unsigned long long* qitems, long long qcap, cudaStream_t s)
 {
     const CollideArgs<float> none{};
-    k_collide_f32<M_UNIFORM, true, true><<<grid, 32 * WARPS, 0, s>>>(none, boxes, prefix, nboxes, counter, step_dev, chunk, qcount,
+    k_collide_f32<M_UNIFORM, true, true, false><<<grid, 32 * WARPS, 0, s>>>(none, boxes, prefix, nboxes, counter, step_dev, chunk, qcount,
                                                           qitems, qcap);
     return cudaGetLastError();
 }
