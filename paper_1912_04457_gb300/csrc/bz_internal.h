@@ -365,6 +365,17 @@ inline int f32_unit_chunks(int64_t items, int64_t warps)
     const int64_t c = share / 8;
     return (int)(c < 8 ? 8 : (c > 32 ? 32 : c));
 }
+// Work units of the FP64 collision kernel on `warps` resident warps: at most 32 chunks,
+// an even number of units for every warp, whole anchors rounded up.
+inline F32Split f64_split(int64_t n_sel, int nsamples, int64_t warps)
+{
+    const int64_t nchunk = (nsamples + 31) / 32, items = n_sel * nchunk;
+    const int64_t share = items > 0 ? (items + warps - 1) / warps : 1;  // no anchor selected: no units
+    const int64_t rounds = (share + 31) / 32;
+    int64_t chunks = (share + rounds - 1) / rounds;
+    if (chunks > nchunk) chunks = chunks + nchunk - 1 < 32 ? chunks + nchunk - 1 : 32;
+    return f32_split(n_sel, nsamples, chunks < 1 ? 1 : (int)chunks);
+}
 int mlp_nparam();
 int mlp_image_bytes();
 // ntot > 0: minibatch position r reads record splitmix64(key + r) mod ntot of rec

@@ -507,13 +507,7 @@ cudaError_t launch_collide_f64(const CollideArgs<double>& a, int nsm, cudaStream
     int terms = 0;
     for (int d = 0; d < NSPEC; ++d) terms += a.nterms[d];
     const bool one = terms == 1;  // one species
-    // units of at most 32 chunks, an even number of them for every warp
-    const int64_t nchunk = (a.nsamples + 31) / 32, items = a.n_sel * nchunk;
-    const int64_t warps = (int64_t)nsm * (one ? BLOCKS64<128> : BLOCKS64<64>) * W64;
-    const int64_t share = (items + warps - 1) / warps, rounds = (share + 31) / 32;
-    int64_t chunks = (share + rounds - 1) / rounds;
-    if (chunks > nchunk) chunks = chunks + nchunk - 1 < 32 ? chunks + nchunk - 1 : 32;  // whole anchors, rounded up
-    const F32Split f = f32_split(a.n_sel, a.nsamples, chunks < 1 ? 1 : (int)chunks);
+    const F32Split f = f64_split(a.n_sel, a.nsamples, (int64_t)nsm * (one ? BLOCKS64<128> : BLOCKS64<64>) * W64);
     if (a.sampler != SAMPLER_LEARNED && a.param == 0 && !a.p_center && a.ncell < ((int64_t)1 << 31) &&
         f.units < ((int64_t)1 << 31)) {
         CollideArgs<double> b = a;
