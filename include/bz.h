@@ -392,9 +392,10 @@ int bz_proposal_init(bz_handle h, uint64_t seed);
 int bz_proposal_get_params(bz_handle h, float* host);
 int bz_proposal_set_params(bz_handle h, const float* host);
 /* Uniform FP32 sampling of state in record mode: no deposits, no FP64
- * re-evaluation; for every unit of an anchor's samples whose index is a
- * multiple of unit_stride one record is appended to records (device,
- * max_records) for each sample with w > 0 (samples whose roots were all
+ * re-evaluation; the samples are in units of one anchor and up to 256 of its
+ * samples (ceil(nsamples / 256) units an anchor, anchors in order), and for
+ * every unit whose index is a multiple of unit_stride one record is appended
+ * to records (device, max_records) for each sample with w > 0 (samples whose roots were all
  * rejected or fell outside the box carry no information and are skipped).
  * Record order is not deterministic.  *n_written (host) receives the count,
  * at most max_records; synchronises.  Errors: BZ_EINVAL for a NULL pointer,

@@ -903,10 +903,10 @@ static int run_collide(bz_handle h, long long* A, int nsamples, int step, double
     // Cell indices are 32-bit there.
     if (h->ncell >= (int64_t)1 << 31)
         return fail(h, BZ_EINVAL, "the FP32 path needs fewer than 2^31 cells (has %lld)", (long long)h->ncell);
-    const int64_t old_units = f32_split(n_sel, nsamples, F32_RECORD_CHUNKS).units;
-    if (old_units >= ((int64_t)1 << 31))
+    const int64_t anchor_units = f32_anchor_split(n_sel, nsamples).units;
+    if (anchor_units >= ((int64_t)1 << 31))
         return fail(h, BZ_EINVAL, "anchors x samples too large for one FP32 call (%lld work units); use an anchor subset",
-                    (long long)old_units);
+                    (long long)anchor_units);
     CollideArgs<float> a{};
     fill_collide(h, a, A, nsamples, step, dt, sampler);
     a.step_dev = step_dev;
@@ -1521,10 +1521,10 @@ extern "C" int bz_batch_create(bz_batch* out, int32_t nboxes, const bz_box* boxe
         b->slot_prefix[i + 1] = b->slot_prefix[i] + h.nslots;
     }
     const int chunks = f32_unit_chunks(items, (int64_t)b->nsm * 24);
-    int64_t old_units = 0;
+    int64_t anchor_units = 0;
     b->split.resize(nboxes);
     for (int i = 0; i < nboxes; ++i) {
-        old_units += f32_split(b->hb[i].ncell, boxes[i].nsamples, F32_RECORD_CHUNKS).units;
+        anchor_units += f32_anchor_split(b->hb[i].ncell, boxes[i].nsamples).units;
         b->split[i] = f32_split(b->hb[i].ncell, boxes[i].nsamples, chunks);
         b->unit_prefix[i + 1] = b->unit_prefix[i] + b->split[i].units;
     }
@@ -1533,7 +1533,7 @@ extern "C" int bz_batch_create(bz_batch* out, int32_t nboxes, const bz_box* boxe
     b->nmchunks = b->mchunk_prefix[nboxes];
     b->ncchunks = b->cchunk_prefix[nboxes];
     b->total_slots = b->slot_prefix[nboxes];
-    if (b->ncell >= ((int64_t)1 << 31) || old_units >= ((int64_t)1 << 31)) {
+    if (b->ncell >= ((int64_t)1 << 31) || anchor_units >= ((int64_t)1 << 31)) {
         delete b;
         return bfail(nullptr, BZ_EINVAL, "the batch needs fewer than 2^31 cells and work units");
     }
@@ -2008,7 +2008,7 @@ extern "C" int bz_record(bz_handle h, const int64_t* state, int32_t nsamples, in
     unsigned long long* cnt = h->d_rec_count;
     CK(h, cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
     const int64_t n_sel = h->a_offset < h->ncell ? (h->ncell - h->a_offset + h->a_stride - 1) / h->a_stride : 0;
-    const F32Split split = f32_split(n_sel, nsamples, F32_RECORD_CHUNKS);
+    const F32Split split = f32_anchor_split(n_sel, nsamples);
     const int64_t units = split.units;
     if (units >= ((int64_t)1 << 31)) return fail(h, BZ_EINVAL, "anchors x samples too large for one record call");
     int64_t blocks = (units + F32_WARPS - 1) / F32_WARPS;

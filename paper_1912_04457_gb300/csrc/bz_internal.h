@@ -352,7 +352,14 @@ inline F32Split f32_split(int64_t n_sel, int nsamples, int chunks)
     f.units = f.upa > 1 ? (n_sel + f.upa - 1) / f.upa : n_sel * f.gpa;
     return f;
 }
-constexpr int F32_RECORD_CHUNKS = 8;  // record mode: a unit is an anchor and up to 256 of its samples
+// Units of one anchor and up to 256 of its samples each: record mode's (thinned by
+// their index, so that a unit must not join anchors), and what the limit of 2^31 units a
+// call counts.
+inline F32Split f32_anchor_split(int64_t n_sel, int nsamples)
+{
+    const int nchunk = (nsamples + 31) / 32;
+    return f32_split(n_sel, nsamples, nchunk < 8 ? nchunk : 8);
+}
 // Chunks of a unit for a problem of `items` chunks on `warps` resident warps.  A
 // warp's last passes over a unit's samples and roots are short (on average
 // half empty), so units are long -- 32 chunks -- where there are many per

@@ -114,6 +114,29 @@ def test_record_mode():
     assert 0 < n3 < n
 
 
+@pytest.mark.parametrize("N,stride", [(32, 3), (100, 3), (129, 2), (300, 5)])
+def test_record_stride_selects_units_of_one_anchor(N, stride):
+    """unit_stride keeps the records of the units (anchor, part of 256 samples) whose
+    index is a multiple of it, whatever the sample count; a sample's record does not
+    depend on the number of samples, so that an anchor's first part is its records at 256."""
+    import torch
+    from paper_1912_04457_gb300 import bz
+    mask, np_ = 0x03, (8, 6, 4)
+    st = torch.from_numpy(I.encode(I.random_f(np_, 2, 1, 5, 0.0, 0.6), mask).reshape(-1)).cuda()
+
+    def records(nsamples, unit_stride):
+        h = bz.Handle(np_=np_, L=2.0, seed=3, species_mask=mask)
+        rec, n = h.record(st, nsamples, step=4, dt=0.01, unit_stride=unit_stride, max_records=1 << 18)
+        r = rec[: n * 32].cpu().numpy().view(REC)
+        return {(int(x["a"]), x["y"].tobytes(), x["w"].tobytes()) for x in r}
+
+    every, first = records(N, 1), records(min(N, 256), 1)
+    parts = (N + 255) // 256
+    want = {r for r in every if (r[0] * parts + (r not in first)) % stride == 0}
+    assert 0 < len(want) < len(every)
+    assert records(N, stride) == want
+
+
 def test_trained_proposal_lowers_the_error():
     """Record at t = 0 with the uniform sampler, train on the GPU, and compare the
     relative L2 error of the collision term against a high-N oracle reference
