@@ -614,6 +614,11 @@ __device__ __forceinline__ long long force_acc(const DriftArgs& P, const float* 
     return acc;
 }
 
+// Face flux of a Courant number w 2^-30 of any size (out of line: rare)
+__device__ __noinline__ long long wide_flux(long long n, float w) { return flux_fx(n, rint_ll(w)); }
+
+// Rows of p cells, a thread per cell.  NARROW: |C| < 2^31, which dt/dx < 2 gives where m^2 >= 0
+// (|p| <= E); a state with negative cells can have m^2 < 0, so that larger ones take wide_flux.
 template <bool NARROW>
 __global__ void __launch_bounds__(DRIFT_THREADS) k_drift(const __grid_constant__ DriftArgs P)
 {
@@ -653,12 +658,14 @@ __global__ void __launch_bounds__(DRIFT_THREADS) k_drift(const __grid_constant__
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 if (P.nx[d] == 1) continue;
-                const int own_C = rint_split(((pf[d] * inv) * P.dtdxf) * 1073741824.0f);
+                const float own_w = ((pf[d] * inv) * P.dtdxf) * 1073741824.0f;
                 const long long off = s_off[2 * d + (pf[d] > 0.0f ? 0 : 1)];  // the upwind neighbour
                 if (!bz_in(row * P.npc + off + j, P.ncell)) continue;
                 const long long nn = __ldg(in_row + off + j);
-                const int nb_C = rint_split(((pf[d] * __ldg(ie_row + off + j)) * P.dtdxf) * 1073741824.0f);
-                const long long f_own = flux32(nh, nl, own_C), f_nb = flux32((int)(nn >> 32), (unsigned)nn, nb_C);
+                const float nb_w = ((pf[d] * __ldg(ie_row + off + j)) * P.dtdxf) * 1073741824.0f;
+                const long long f_own = fabsf(own_w) >= 2147483648.0f ? wide_flux(ncj, own_w) : flux32(nh, nl, rint_split(own_w));
+                const long long f_nb = fabsf(nb_w) >= 2147483648.0f ? wide_flux(nn, nb_w)
+                                                                   : flux32((int)(nn >> 32), (unsigned)nn, rint_split(nb_w));
                 // p_d > 0: outflow up, inflow from below; p_d < 0: inflow from above, outflow down
                 acc += pf[d] > 0.0f ? f_own - f_nb : f_nb - f_own;
             }
@@ -773,7 +780,7 @@ __device__ __noinline__ long long force_acc_octet(const DriftArgs& P, const floa
 // Sum of rounded fluxes sum_i +-((n_i C_i + half_i) >> 30), 0 <= C_i: with n = nh
 // 2^32 + nl (nl unsigned) each is 4 nh C + s, s = (nl C + half) >> 30; the first
 // parts add up in one wide multiply-accumulate each, and where C < 2^30 (UNIT:
-// dt/dx < 0.999) s is the high word of nl (4 C) + 4 half, so that a flux takes two
+// dt/dx < 0.999 and m^2 >= 0) s is the high word of nl (4 C) + 4 half, so that a flux takes two
 // wide multiplications and an add.  The low 64 bits are those of the exact sum.
 template <bool UNIT>
 struct FluxSum {
@@ -795,6 +802,54 @@ struct FluxSum {
         lo -= low((unsigned)n, C, half);
     }
 };
+
+// A thread's cells again, in all its rows, with exact products.  The launch's dt/dx keeps C in
+// the range of the form it takes where |p| <= E; with m^2 < 0 (a state with negative cells) C may
+// leave it, and a thread that met such a C stores its cells a second time.  It works from the launch's
+// arguments alone, so that the loop before it keeps no register for it but the largest 1/E it met
+// (16^3 x 20^3 gluons: 272 us, 273 without it; the or of all C 277, masses tested ahead of the loop 314, a call out of
+// line 100 bytes of spills).  A C that is no number counts as 0, as in the loop.
+template <bool FORCE>
+__device__ __forceinline__ void mirror_wide(const DriftArgs& P, int nseg, float K)
+{
+    const int t = blockIdx.y * 32 + (threadIdx.x & 31), warp = threadIdx.x >> 5;
+    const int n1 = P.np[1], n2 = P.np[2], ny = P.nx[1], nz = P.nx[2];
+    if (t >= P.half[0] * P.half[1] * n2) return;
+    const int z = t % n2, hx = t / n2 / P.half[1], hy = t / n2 % P.half[1];
+    const int oct = (hx * P.half[1] + hy) * P.half[2] + min(z, n2 - 1 - z);
+    const int seg = (int)(blockIdx.x % (unsigned)nseg), rest = (int)(blockIdx.x / (unsigned)nseg);
+    const int ix = rest % P.nx[0], sl = rest / P.nx[0];
+    const int y0 = (int)((int64_t)seg * ny / nseg), y1 = (int)((int64_t)(seg + 1) * ny / nseg);
+    const bool zsplit = nz >= DOCT_WARPS;
+    const int64_t xs[3] = {(int64_t)ny * nz, nz, 1};
+    for (int iy = y0 + (zsplit ? 0 : warp); iy < y1; iy += zsplit ? 1 : DOCT_WARPS)
+        for (int iz = zsplit ? warp : 0; iz < nz; iz += zsplit ? DOCT_WARPS : 1) {
+            const int xi[3] = {ix, iy, iz};
+            const int64_t x = ((int64_t)ix * ny + iy) * nz + iz, row = (int64_t)sl * P.nxc + x;
+            const long long* in_row = P.in + row * P.npc;
+            const float* inv_row = P.inv_e + row * P.noct;
+            const float inv = inv_row[oct];
+            for (int k = 0; k < 4; ++k) {
+                const int jv[3] = {k & 1 ? P.np[0] - 1 - hx : hx, k & 2 ? n1 - 1 - hy : hy, z};
+                if ((k & 1 && jv[0] == hx) || (k & 2 && jv[1] == hy)) continue;  // a mirror plane
+                const int j = (jv[0] * n1 + jv[1]) * n2 + z;
+                const long long n = in_row[j];
+                long long acc = 0;
+                for (int d = 0; d < 3; ++d) {
+                    if (P.nx[d] == 1) continue;
+                    const float p = P.pf[d][jv[d]];
+                    const int64_t off = xs[d] * (p > 0.0f ? (xi[d] == 0 ? P.nx[d] - 1 : -1) : (xi[d] == P.nx[d] - 1 ? 1 - P.nx[d] : 1));
+                    if (!bz_in((row + off) * P.npc + j, P.ncell)) continue;
+                    const float w = (p * inv) * K, wn = (p * inv_row[off * P.noct + oct]) * K;
+                    const long long own = flux_fx(n, w == w ? rint_ll(w) : 0);
+                    const long long nb = flux_fx(in_row[off * P.npc + j], wn == wn ? rint_ll(wn) : 0);
+                    acc += p > 0.0f ? own - nb : nb - own;
+                }
+                if (FORCE) acc += force_acc_octet(P, P.gforce + (x * 4 + P.slot_mslot[sl]) * 3, jv, j, in_row, inv_row, n, inv);
+                if (bz_in(row * P.npc + j, P.ncell)) P.out[row * P.npc + j] = n - acc;
+            }
+        }
+}
 
 template <bool FORCE, bool UNIT>
 __global__ void __launch_bounds__(32 * DOCT_WARPS, FORCE ? 5 : DRIFT_MINB) k_drift_mirror(const __grid_constant__ DriftArgs P, int nseg, float K)
@@ -829,6 +884,7 @@ __global__ void __launch_bounds__(32 * DOCT_WARPS, FORCE ? 5 : DRIFT_MINB) k_dri
     const int y0 = (int)((int64_t)seg * ny / nseg), y1 = (int)((int64_t)(seg + 1) * ny / nseg);
     const bool zsplit = nz >= DOCT_WARPS;  // the warps share the z cells of a row, or the rows
     const int64_t rows = P.ncell / P.npc;
+    float emax = 0.0f;  // largest 1/E met (see mirror_wide)
     for (int iy = y0 + (zsplit ? 0 : warp); iy < y1; iy += zsplit ? 1 : DOCT_WARPS) {
         const int64_t r0 = (int64_t)sl * P.nxc + ((int64_t)ix * ny + iy) * nz;  // row of (ix, iy, 0)
         const int64_t dylo = (int64_t)(iy == 0 ? ny - 1 : -1) * nz, dyup = (int64_t)(iy == ny - 1 ? 1 - ny : 1) * nz;
@@ -860,6 +916,7 @@ __global__ void __launch_bounds__(32 * DOCT_WARPS, FORCE ? 5 : DRIFT_MINB) k_dri
             FluxSum<UNIT> f[4];
             if (nx0 > 1) {
                 const unsigned C = courant(pax, inv), Clo = courant(pax, ie(pe + dxlo * row_e)), Cup = courant(pax, ie(pe + dxup * row_e));
+                emax = fmaxf(fmaxf(emax, inv), fmaxf(ie(pe + dxlo * row_e), ie(pe + dxup * row_e)));
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     f[k].in(bx[k], k & 1 ? Clo : Cup, k & 1 ? HUP : HDN);
@@ -868,6 +925,7 @@ __global__ void __launch_bounds__(32 * DOCT_WARPS, FORCE ? 5 : DRIFT_MINB) k_dri
             }
             if (ny > 1) {
                 const unsigned C = courant(pay, inv), Clo = courant(pay, ie(pe + dylo * row_e)), Cup = courant(pay, ie(pe + dyup * row_e));
+                emax = fmaxf(fmaxf(emax, inv), fmaxf(ie(pe + dylo * row_e), ie(pe + dyup * row_e)));
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     f[k].in(by[k], k & 2 ? Clo : Cup, k & 2 ? HUP : HDN);
@@ -876,6 +934,7 @@ __global__ void __launch_bounds__(32 * DOCT_WARPS, FORCE ? 5 : DRIFT_MINB) k_dri
             }
             if (nz > 1) {
                 const unsigned C = courant(paz, inv), Cn = courant(paz, ie(pe + (zup ? dzlo : dzhi) * row_e));
+                emax = fmaxf(fmaxf(emax, inv), ie(pe + (zup ? dzlo : dzhi) * row_e));
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     f[k].in(bz[k], Cn, zhalf);
@@ -941,6 +1000,7 @@ __global__ void __launch_bounds__(32 * DOCT_WARPS, FORCE ? 5 : DRIFT_MINB) k_dri
             }
         }
     }
+    if (emax * fmaxf(pax, fmaxf(pay, paz)) * K >= (UNIT ? 1073741824.0f : 2147483648.0f)) mirror_wide<FORCE>(P, nseg, K);
 }
 
 static int device_sms()
@@ -979,7 +1039,7 @@ cudaError_t launch_drift(const DriftArgs& a, cudaStream_t s)
     if (a.force && !(a.gforce && moving)) return cudaErrorInvalidValue;
     if (a.force) k_force_grad<<<(unsigned)((a.nxc * 4 + 127) / 128), 128, 0, s>>>(a);
     const int64_t nslots = rows / a.nxc;
-    // |C| <= 2^30 dt/dx < 2^31, mirrored cells: by octets; else (long time steps, cell
+    // |C| <= 2^30 dt/dx < 2^31 (m^2 >= 0; else checked by the kernels), mirrored cells: by octets; else (long time steps, cell
     // centres that are no exact mirror images in FP32) by rows.  16^3 x 20^3 gluons: 359 -> 273 us without f
     // (some 205 instructions a cell, multiplications and addresses the largest parts), 842 -> 693 us with the force
     if (moving && a.dtdxf < 1.99f && a.noct > 0) {
@@ -991,7 +1051,7 @@ cudaError_t launch_drift(const DriftArgs& a, cudaStream_t s)
             k_inv_octet<<<(unsigned)rows, 256, 0, s>>>(a);
             const dim3 grid((unsigned)gx, (unsigned)tiles_m);
             const float K = a.dtdxf * 1073741824.0f;
-            const bool unit = a.dtdxf < 0.999f;  // C < 2^30
+            const bool unit = a.dtdxf < 0.999f;  // C < 2^30 where |p| <= E
             if (a.force && unit)
                 k_drift_mirror<true, true><<<grid, 32 * DOCT_WARPS, 0, s>>>(a, (int)nseg, K);
             else if (a.force)

@@ -45,3 +45,39 @@ def test_bits(nx, np_, L, mask, dt, rng, force):
     assert np.array_equal(out.cpu().numpy().reshape(st.shape), O.drift(cfg, st, m2, dt).reshape(st.shape))
     src = h.energy_source(dev, dt, 0.9 * m2).cpu().numpy().reshape(nxc, ns, 3)
     assert np.array_equal(src, O.energy_source(cfg, st, m2, 0.9 * m2, dt).reshape(nxc, ns, 3))
+
+
+WIDE = [
+    # nx, np, mask, dt (dx = 0.2), m^2 / (smallest p^2 of the grid), force: Courant numbers beyond dt/dx
+    ((3, 2, 5), (6, 4, 7), 0x03, 0.19, (-0.9, -0.9), True),         # |p| / E up to 3: C above 2^30
+    ((2, 3, 2), (4, 6, 8), 0x01, 0.19, (-0.9999, 0.5), False),      # and above 2^31, next to cells of m^2 > 0
+    ((4, 1, 3), (4, 5, 6), 0x12, 0.3, (-0.9, 0.0), True),           # dt/dx = 1.5
+    ((5, 2, 1), (4, 5, 6), 0x01, 0.3, (-0.9999, 0.0), False),
+    ((2, 1, 1), (256, 256, 130), 0x01, 0.19, (-0.9999, 0.0), False),  # too many tiles: rows of p cells
+]
+
+
+@pytest.mark.parametrize("nx,np_,mask,dt,m2_rng,force", WIDE)
+def test_negative_mass_squared(nx, np_, mask, dt, m2_rng, force):
+    """A state with negative cells can have m^2 < 0, where |p| / E exceeds 1 and Courant
+    numbers leave the range that dt/dx gives: the fluxes stay the exact products."""
+    import torch
+    from paper_1912_04457_gb300 import bz
+    nxc, ns, L = int(np.prod(nx)), bin(mask).count("1"), 2.0
+    pp = sum(min(abs(-L + (j + 0.5) * 2 * L / n) for j in range(n)) ** 2 for n in np_)
+    kw = dict(nx=nx, dx=0.2, np_=np_, L=L, seed=3, species_mask=mask)
+    cfg = O.make_config(force=force, **kw)
+    # the masses are linear in f (E = |p| at the first evaluation): each x cell's largest |m^2| to a share of pp
+    f = I.random_f(np_, ns, nxc, 21, 0.005, 0.01)
+    share = np.linspace(m2_rng[0], m2_rng[1], nxc)
+    f *= (share * pp / O.masses(cfg, I.encode(f, mask)).max(axis=1))[None, :, None]
+    st = I.encode(f, mask)
+    m2 = O.masses(cfg, st)
+    assert m2.min() < -0.89 * pp and m2.min() > -pp
+    h = bz.Handle(**kw)
+    h.set_force_term(force)
+    dev = torch.from_numpy(st.reshape(-1)).cuda()
+    out = torch.empty_like(dev)
+    h.drift(dev, out, dt)
+    assert np.array_equal(h.get_masses(), m2)
+    assert np.array_equal(out.cpu().numpy().reshape(st.shape), O.drift(cfg, st, m2, dt).reshape(st.shape))
