@@ -1166,7 +1166,7 @@ constexpr int MOM_THREADS = 128;  // per (x cell, slot) or chunk of one
 // read; 7 blocks per SM, 72 registers: more bytes in flight than with 94).
 // The eight n as loaded, lower cells first: bit d of the index is set for the
 // upper cell of axis d; a cell on the mirror plane of an odd axis counts as its
-// lower cell only (its momentum component there is 0).
+// lower cell only (its factor 2j + 1 - n there is 0).
 struct Octet {
     long long n[8];
     int h[3];

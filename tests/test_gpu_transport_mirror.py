@@ -22,6 +22,9 @@ CASES = [
     ((2, 2, 3), (6, 5, 6), 0.01, 0x7F, 0.01, (0.0, 0.9), True),        # E below 2^-7: wide 1/E; f / E <= 0.9 / 0.001,
     # so that the masses' fixed-point sums over 180 cells stay below 2^19 (f up to 900 would exceed it)
     ((2, 3, 2), (32, 31, 2), 3.0, 0x11, 0.02, (0.0, 1.0), False),
+    ((3, 2, 2), (7, 4, 11), 7.3, 0x13, 0.05, (-0.2, 0.9), True),       # central cells at 8.9e-16
+    ((2, 2, 3), (6, 33, 4), 7.3, 0x01, 0.3, (0.0, 0.9), False),
+    ((1, 3, 2), (35, 35, 2), 0.7, 0x03, 0.1, (0.0, 2.0), True),
 ]
 
 
