@@ -614,15 +614,14 @@ __device__ __forceinline__ long long force_acc(const DriftArgs& P, const float* 
     return acc;
 }
 
-// Face flux of a Courant number w 2^-30 of any size (out of line: rare)
-__device__ __noinline__ long long wide_flux(long long n, float w) { return flux_fx(n, rint_ll(w)); }
-
 // Rows of p cells, a thread per cell.  NARROW: |C| < 2^31, which dt/dx < 2 gives where m^2 >= 0
-// (|p| <= E); a state with negative cells can have m^2 < 0, so that larger ones take wide_flux.
+// (|p| <= E); a state with negative cells can have m^2 < 0, and a row with it or next to one takes
+// the exact products of the other form.
 template <bool NARROW>
 __global__ void __launch_bounds__(DRIFT_THREADS) k_drift(const __grid_constant__ DriftArgs P)
 {
     __shared__ long long s_off[6];    // cell offsets of the (lower, upper) neighbour rows per axis
+    __shared__ unsigned s_neg[6];     // m^2 < 0 in the row or that neighbour
     __shared__ float s_pf[3][MAX_NP]; // cell-centre momenta (lanes index them at different cells)
     for (int d = 0; d < 3; ++d)
         for (int i = threadIdx.x; i < P.np[d]; i += blockDim.x) s_pf[d][i] = P.pf[d][i];
@@ -636,8 +635,12 @@ __global__ void __launch_bounds__(DRIFT_THREADS) k_drift(const __grid_constant__
         const int xi = (int)((x / xs) % P.nx[d]);
         const int64_t step = up ? (xi == P.nx[d] - 1 ? 1 - P.nx[d] : 1) : (xi == 0 ? P.nx[d] - 1 : -1);
         s_off[threadIdx.x] = step * xs * P.npc;
+        if (NARROW && P.inv_e && P.mass_mode != 1)  // the signs of the row's and its neighbours' masses
+            s_neg[threadIdx.x] = (unsigned)(__double2hiint(P.m2[x * 4 + ms]) | __double2hiint(P.m2[(x + step * xs) * 4 + ms])) >> 31;
     }
     __syncthreads();
+    const bool narrow = NARROW && P.inv_e &&
+                        (P.mass_mode == 1 || !(s_neg[0] | s_neg[1] | s_neg[2] | s_neg[3] | s_neg[4] | s_neg[5]));
     const long long* in_row = P.in + row * P.npc;
     long long* out_row = P.out + row * P.npc;
     const int npc = (int)P.npc;
@@ -650,7 +653,7 @@ __global__ void __launch_bounds__(DRIFT_THREADS) k_drift(const __grid_constant__
         const int jp = __ldg(P.jtab + j);
         const float pf[3] = {s_pf[0][jp & 0xff], s_pf[1][(jp >> 8) & 0xff], s_pf[2][jp >> 16]};
         long long acc = 0;
-        if (NARROW && P.inv_e) {
+        if (narrow) {
             const float* ie_row = P.inv_e + row * P.npc;
             const float inv = __ldg(ie_row + j);
             const int nh = (int)(ncj >> 32);
@@ -658,14 +661,12 @@ __global__ void __launch_bounds__(DRIFT_THREADS) k_drift(const __grid_constant__
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 if (P.nx[d] == 1) continue;
-                const float own_w = ((pf[d] * inv) * P.dtdxf) * 1073741824.0f;
+                const int own_C = rint_split(((pf[d] * inv) * P.dtdxf) * 1073741824.0f);
                 const long long off = s_off[2 * d + (pf[d] > 0.0f ? 0 : 1)];  // the upwind neighbour
                 if (!bz_in(row * P.npc + off + j, P.ncell)) continue;
                 const long long nn = __ldg(in_row + off + j);
-                const float nb_w = ((pf[d] * __ldg(ie_row + off + j)) * P.dtdxf) * 1073741824.0f;
-                const long long f_own = fabsf(own_w) >= 2147483648.0f ? wide_flux(ncj, own_w) : flux32(nh, nl, rint_split(own_w));
-                const long long f_nb = fabsf(nb_w) >= 2147483648.0f ? wide_flux(nn, nb_w)
-                                                                   : flux32((int)(nn >> 32), (unsigned)nn, rint_split(nb_w));
+                const int nb_C = rint_split(((pf[d] * __ldg(ie_row + off + j)) * P.dtdxf) * 1073741824.0f);
+                const long long f_own = flux32(nh, nl, own_C), f_nb = flux32((int)(nn >> 32), (unsigned)nn, nb_C);
                 // p_d > 0: outflow up, inflow from below; p_d < 0: inflow from above, outflow down
                 acc += pf[d] > 0.0f ? f_own - f_nb : f_nb - f_own;
             }

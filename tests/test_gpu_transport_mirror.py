@@ -25,6 +25,10 @@ CASES = [
     ((3, 2, 2), (7, 4, 11), 7.3, 0x13, 0.05, (-0.2, 0.9), True),       # central cells at 8.9e-16
     ((2, 2, 3), (6, 33, 4), 7.3, 0x01, 0.3, (0.0, 0.9), False),
     ((1, 3, 2), (35, 35, 2), 0.7, 0x03, 0.1, (0.0, 2.0), True),
+    ((2, 3, 8), (6, 5, 4), 2.0, 0x12, 0.05, (-0.2, 0.9), True),        # the force by mirrored cells: z cells
+    ((1, 8, 2), (26, 34, 16), 2.0, 0x7F, 0.02, (0.0, 0.9), True),      # or segments that fill the warps
+    ((3, 2, 6), (6, 5, 4), 2.0, 0x12, 0.05, (-0.2, 0.9), True),        # and by rows
+    ((2, 1, 1), (40, 64, 50), 2.0, 0x01, 0.02, (0.0, 0.9), False),     # several blocks for a row's 1/E
 ]
 
 
@@ -55,6 +59,8 @@ WIDE = [
     ((3, 2, 5), (6, 4, 7), 0x03, 0.19, (-0.9, -0.9), True),         # |p| / E up to 3: C above 2^30
     ((2, 3, 2), (4, 6, 8), 0x01, 0.19, (-0.9999, 0.5), False),      # and above 2^31, next to cells of m^2 > 0
     ((4, 1, 3), (4, 5, 6), 0x12, 0.3, (-0.9, 0.0), True),           # dt/dx = 1.5
+    ((2, 3, 8), (6, 4, 8), 0x03, 0.19, (-0.9, -0.9), True),
+    ((2, 2, 4), (4, 5, 6), 0x12, 0.3, (-0.9, 0.0), True),
     ((5, 2, 1), (4, 5, 6), 0x01, 0.3, (-0.9999, 0.0), False),
     ((2, 1, 1), (256, 256, 130), 0x01, 0.19, (-0.9999, 0.0), False),  # too many tiles: rows of p cells
 ]
