@@ -1041,14 +1041,24 @@ cudaError_t launch_drift(const DriftArgs& a, cudaStream_t s)
     if (a.force) k_force_grad<<<(unsigned)((a.nxc * 4 + 127) / 128), 128, 0, s>>>(a);
     const int64_t nslots = rows / a.nxc;
     // |C| <= 2^30 dt/dx < 2^31 (m^2 >= 0; else checked by the kernels), mirrored cells: by octets; else (long time steps, cell
-    // centres that are no exact mirror images in FP32) by rows.  16^3 x 20^3 gluons: 359 -> 273 us without f
-    // (some 205 instructions a cell, multiplications and addresses the largest parts), 842 -> 693 us with the force
+    // centres that are no exact mirror images in FP32) by rows.  16^3 x 20^3 gluons, without f: 242 us, by rows 440
+    // (some 205 instructions a cell, multiplications and addresses the largest parts)
     if (moving && a.dtdxf < 1.99f && a.noct > 0) {
         const int64_t tiles_m = ((int64_t)a.half[0] * a.half[1] * a.np[2] + 31) / 32, base = nslots * a.nx[0] * tiles_m;
-        int64_t nseg = ((int64_t)device_sms() * 8 + base - 1) / base;  // y segments: 8 blocks per SM
+        // y segments of equal length: 40 blocks per SM (five waves, so that the last one matters little: 16^3 x
+        // 20^3 gluons 272 -> 242 us, with 8 per SM); 8 where the warps share a segment's rows, which few z cells need
+        const bool zsplit = a.nx[2] >= DOCT_WARPS;
+        int64_t nseg = ((int64_t)device_sms() * (zsplit ? 40 : 8) + base - 1) / base;
         nseg = nseg < 1 ? 1 : (nseg > a.nx[1] ? a.nx[1] : nseg);
+        while (zsplit && a.nx[1] % nseg) ++nseg;
+        // With the force, whose neighbours along p cost both forms alike, mirrored cells are as fast as rows where
+        // the four warps share their z cells or rows evenly (16^3 x 20^3 gluons: 667 us, rows 675; 4^3 x 32^3:
+        // 52, 59) and slower where some have none (11 x 8 x 5 x (28, 36, 36), three species: 1430, rows 1000;
+        // 3^3 x 32^3: 47, 33)
+        const int64_t share = zsplit ? a.nx[2] : a.nx[1] / nseg, whole = (share + DOCT_WARPS - 1) / DOCT_WARPS * DOCT_WARPS;
+        const bool rows_form = a.force && 5 * whole >= 6 * share;
         const int64_t gx = nslots * a.nx[0] * nseg;
-        if (tiles_m <= 65535 && gx <= 2147483647LL) {
+        if (!rows_form && tiles_m <= 65535 && gx <= 2147483647LL) {
             // blocks of a row's octets: enough for every SM (2 rows of (128, 128, 64) cells: 186 -> 39 us)
             const int64_t per_row = ((int64_t)device_sms() * 8 + rows - 1) / rows, chunks = (a.noct + 255) / 256;
             k_inv_octet<<<dim3((unsigned)rows, (unsigned)(per_row < chunks ? per_row : chunks)), 256, 0, s>>>(a);
