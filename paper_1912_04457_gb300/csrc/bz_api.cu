@@ -930,7 +930,8 @@ static int run_collide(bz_handle h, long long* A, int nsamples, int step, double
     if (dyn && !h->d_counter && cudaMalloc(&h->d_counter, sizeof(unsigned long long)) != cudaSuccess)
         return fail(h, BZ_ENOMEM, "cannot allocate the unit counter");
     const int64_t warps = blocks * F32_WARPS;
-    const int64_t samples_per_warp = ((units + warps - 1) / warps) * 32 * ((int64_t)a.upa * a.cpg);
+    // queue room: a share of the term evaluations of 256 samples for every unit of an anchor
+    const int64_t samples_per_warp = ((anchor_units + warps - 1) / warps) * 256;
     const int64_t qcap = samples_per_warp * MAX_TERMS / DEFER_CAP_DIV + 64;
     if (warps > h->q_warps || warps * qcap > h->q_items) {
         cudaFree(h->d_qcount);
@@ -1538,9 +1539,9 @@ extern "C" int bz_batch_create(bz_batch* out, int32_t nboxes, const bz_box* boxe
         return bfail(nullptr, BZ_EINVAL, "the batch needs fewer than 2^31 cells and work units");
     }
     // persistent grid of up to 32 warps per SM; per-warp queue room for 4% of an
-    // even share at 24 warps per SM (2.7% at 16, 5.3% at 32)
+    // even share at 24 warps per SM (2.7% at 16, 5.3% at 32), 256 samples for every unit of an anchor
     b->qwarps = (int64_t)b->nsm * 32;
-    b->qcap = (items * 32 * MAX_TERMS) / ((int64_t)b->nsm * 24) / 25 + 64;
+    b->qcap = (anchor_units * 256 * MAX_TERMS) / ((int64_t)b->nsm * 24) / 25 + 64;
     bool ok = dalloc(&b->d_f, b->ncell) && dalloc(&b->d_m2_cur, 4 * nboxes) && dalloc(&b->d_m2_prev, 4 * nboxes) &&
               dalloc(&b->d_acc, 4 * nboxes) && dalloc(&b->d_flags, 4) && dalloc(&b->d_have_prev, 1) &&
               dalloc(&b->d_step, 1) && dalloc(&b->d_kidx, 1) && dalloc(&b->d_counter, 1) &&

@@ -336,7 +336,8 @@ constexpr double DEFER_TAU = BZ_DEFER_TAU;  // FP32 terms with |H| < tau kappa^2
 #ifndef BZ_DEFER_CAP_DIV
 #define BZ_DEFER_CAP_DIV 50
 #endif
-constexpr int DEFER_CAP_DIV = BZ_DEFER_CAP_DIV;  // queue room: 1/DIV of a warp's term evaluations
+constexpr int DEFER_CAP_DIV = BZ_DEFER_CAP_DIV;  // queue room: 1/DIV of a warp's term evaluations, were every anchor's
+                                                 // samples (and terms) rounded up to 256 (and MAX_TERMS)
 constexpr int MAX_SAMPLES = 1 << 20;
 // FP32 collision kernel: warps per block.
 constexpr int F32_WARPS = 4;

@@ -39,3 +39,26 @@ def test_no_anchor_selected(prec):
     if prec == 0:
         assert np.all(h.collision_audit(st, A, 64)[4:] == 0.0)
     assert np.all(h.flags() == 0)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("batch", [False, True])
+def test_few_samples_leave_room_in_the_re_evaluation_queue(batch):
+    """Heavy species (thermal masses of a large coupling, some 10 GeV in a box of 2) make every
+    tenth term ill-conditioned.  The queue has room for 256 samples of every unit of an anchor, so that
+    at 32 samples none of them is left to FP32."""
+    import torch
+    from paper_1912_04457_gb300 import bz
+    from paper_1912_04457_gb300 import inputs as I
+    np_, mask, alpha, N = (16, 16, 16), 0x7F, 60.0, 32
+    n = I.encode(I.random_f(np_, 7, 1, 7, 0.0, 0.5), mask).reshape(-1)
+    if batch:
+        b = bz.Batch([dict(np_=np_, L=2.0, species_mask=mask, nsamples=N, alpha_s=alpha)] * 4)
+        st = torch.from_numpy(np.tile(n, 4)).cuda()
+        b.step(st, 1e-9, 1)
+        assert b.flags()[3] == 0
+    else:
+        h = bz.Handle(np_=np_, L=2.0, seed=3, species_mask=mask, alpha_s=alpha)
+        A = torch.empty(n.size, dtype=torch.int64, device="cuda")
+        h.collision_term(torch.from_numpy(n).cuda(), A, N, 0, 1e-9, bz.PREC_F32)
+        assert h.flags()[3] == 0 and int(A.sum().item()) == 0
