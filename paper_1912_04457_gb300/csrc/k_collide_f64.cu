@@ -61,13 +61,20 @@ __device__ __forceinline__ bool in_box64(double v, double L)
 {
     return (dbits(v) & ~SIGN64) < dbits(L) || dbits(v) == (dbits(L) | SIGN64);
 }
-// v truncated to FP32 (0 below its normal range; v within the FP32 range)
-__device__ __forceinline__ float trunc32(double v)
+// Exponent field of FP64 minus that of FP32 for v 2^-e, e in [-800, 800], and v 2^-e
+// truncated to FP32 with it: 0 below FP32's normal range, infinite above it.
+__device__ __forceinline__ int rebias32(int e) { return (896 + e) << 20; }
+__device__ __forceinline__ float trunc32(double v, int rebias)
 {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-    const unsigned mag = hi & 0x7fffffffu;
-    const unsigned m = mag - 0x38000000u;  // exponent rebias 1023 -> 127
-    return mag < 0x38100000u ? 0.0f : __uint_as_float((hi & 0x80000000u) | (m << 3) | (lo >> 29));
+    const int m = (int)(hi & 0x7fffffffu) - rebias;
+    const unsigned mag = m < 0x00100000 ? 0u : (m >= 0x0FF00000 ? 0x7F800000u : ((unsigned)m << 3) | (lo >> 29));
+    return __uint_as_float((hi & 0x80000000u) | mag);
+}
+// v 2^-e for a normal v and result
+__device__ __forceinline__ double scale64(double v, int e)
+{
+    return __hiloint2double(__double2hiint(v) - (e << 20), __double2loint(v));
 }
 
 // 1 + u of a Philox word, exactly: u = (x + 1/2) 2^-32, or ((x >> 9) + 1/2) 2^-23
@@ -91,10 +98,10 @@ __device__ __forceinline__ float sqrt32(float x)
 }
 
 // Bin of the solved coordinate v inside the box: bin_of where FP32 cannot tell
-// it (t within its error bound, some 3e-7 n bins, of an edge).
-__device__ __forceinline__ int solved_bin64(double v, double L, double dp, float Lf, float inv_dp, int n)
+// it (t within its error bound, some 3e-7 n bins, of an edge).  reb1, Lf and inv_dp: the scale of L.
+__device__ __forceinline__ int solved_bin64(double v, double L, double dp, int reb1, float Lf, float inv_dp, int n)
 {
-    const float t = (trunc32(v) + Lf) * inv_dp;
+    const float t = (trunc32(v, reb1) + Lf) * inv_dp;
     const float r = t + 12582912.0f;  // nearest integer by the shifter
     const float d = t - (r - 12582912.0f);
     if (!(fabsf(d) > 1e-6f * (float)n + 1e-6f)) return bin_of<double>(v, L, dp, n);
@@ -111,8 +118,11 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
     const int lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
     const double L = P.L, twoL = P.twoL;
-    const float Lf = (float)P.L;
-    const float inv_dp2 = 1.0f / (float)P.dp[2];
+    // the classification in FP32 works in units of L's power of two, 2^eL: FP32's range is far
+    // from its squares then for any L, and the margins, all relative, are the same
+    const int eL = min(max((__double2hiint(L) >> 20) - 1023, -400), 400), reb1 = rebias32(eL), reb2 = rebias32(2 * eL);
+    const float Lf = (float)scale64(L, eL);
+    const float inv_dp2 = 1.0f / (float)scale64(P.dp[2], eL);
     const uint32_t npc = (uint32_t)P.npc;
     const uint32_t slot_stride = (uint32_t)(P.nxc * P.npc);
     const uint32_t sl = udiv(a_first, P.dv_slot);
@@ -129,7 +139,7 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
         S.tmb[lane] = massless ? 0.0 : m2x[T.mslot[1]];
         S.tmc[lane] = massless ? 0.0 : m2x[T.mslot[2]];
         S.tsym[lane] = T.sym;
-        S.tmf[lane] = make_float4(trunc32(S.tma[lane]), trunc32(S.tmb[lane]), trunc32(S.tmc[lane]), 0.0f);
+        S.tmf[lane] = make_float4(trunc32(S.tma[lane], reb2), trunc32(S.tmb[lane], reb2), trunc32(S.tmc[lane], reb2), 0.0f);
         S.tinfo[lane] = T.slot[0] | (T.slot[1] << 3) | (T.slot[2] << 6) | (T.quark[0] << 9) | (T.quark[1] << 10)
                         | (T.quark[2] << 11) | (T.quark[3] << 12) | (T.cls << 13);
     }
@@ -204,9 +214,9 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
                         const int4 gi = S.gi[src];
                         const double M2 = msq<double>(info >> 13, P, s, t, uu, mg2);
                         const uint32_t i1 = (unsigned)(info & 7) * slot_stride + (unsigned)gi.y * n2
-                                            + (unsigned)solved_bin64(z, L, P.dp[2], Lf, inv_dp2, (int)n2);
+                                            + (unsigned)solved_bin64(z, L, P.dp[2], reb1, Lf, inv_dp2, (int)n2);
                         const uint32_t i2 = (unsigned)((info >> 3) & 7) * slot_stride + (unsigned)gi.z * n2
-                                            + (unsigned)solved_bin64(dz, L, P.dp[2], Lf, inv_dp2, (int)n2);
+                                            + (unsigned)solved_bin64(dz, L, P.dp[2], reb1, Lf, inv_dp2, (int)n2);
                         const uint32_t i3 = (unsigned)((info >> 6) & 7) * slot_stride + (unsigned)gi.x;
                         const uint32_t i4 = (unsigned)gi.w;
                         if (bz_in(xoff + (int64_t)i1, P.ncell) & bz_in(xoff + (int64_t)i2, P.ncell) &
@@ -378,11 +388,11 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
                         };
                         S.gi[sb] = make_int4((bin(w[5], n0) * (int)n1 + bin(w[6], n1)) * (int)n2 + bin(w[7], n2),
                                              bin(w[3], n0) * (int)n1 + bin(w[4], n1), (int)(m >> 16), (int)ac.j);
-                        gEp = trunc32(Ep);
-                        gPz = trunc32(Pz);
-                        ga2 = trunc32(a2m);
-                        gb2 = trunc32(b2m);
-                        gkk3 = trunc32(kk3);
+                        gEp = trunc32(Ep, reb1);
+                        gPz = trunc32(Pz, reb1);
+                        ga2 = trunc32(a2m, reb2);
+                        gb2 = trunc32(b2m, reb2);
+                        gkk3 = trunc32(kk3, reb2);
                     }
                     ti = 0;
                 }
@@ -392,26 +402,27 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
             // FP32 estimate of the two roots of term ti for this lane's sample.  With
             // K = E^2 + a^2 + b^2 every operation's error is below 1e-6 K (kappa, D),
             // 5e-6 K^2 (H); the margins are at least four times what follows from
-            // that.  Roots that may be valid stay: NaNs and overflows count as "may".
+            // that.  Roots that may be valid stay: NaNs and overflows count as "may" (K^2 is taken first:
+            // it overflows before the terms of H do).
             const float4 tmf = S.tmf[ti];
             const float ma2 = tmf.x, mb2 = tmf.y, mc2 = tmf.z;
             const float E3 = sqrt32(gkk3 + mc2);
             const float E = gEp + E3, EE = E * E;
             const float a2 = ga2 + ma2, b2 = gb2 + mb2;
-            const float K = EE + a2 + b2, Pz2 = gPz * gPz;
+            const float K = EE + a2 + b2, KK = K * K, Pz2 = gPz * gPz;
             const float D = EE - Pz2;
             const float kap = (EE + a2 - b2 - Pz2) * 0.5f;
             const float H = kap * kap - a2 * D;
             bool c0r = lane < bcnt, c1r;
             // no root: below the tangency, or E1 < 0 or E2 < 0 (kappa outside (0, D))
-            c0r = c0r && !(H < -1e-4f * K * K) && !(kap < -1e-5f * K) && !(kap > D + 1e-5f * K);
+            c0r = c0r && !(H < -1e-4f * KK) && !(kap < -1e-5f * K) && !(kap > D + 1e-5f * K);
             c1r = c0r;
             // both roots stay where the estimate is poor or their order (the sign of kappa Pz) is open
-            const bool good = fabsf(H) > 1e-4f * K * K && D > 1e-3f * K && kap > 1e-4f * K && fabsf(gPz) > 1e-5f * Lf;
+            const bool good = fabsf(H) > 1e-4f * KK && D > 1e-3f * K && kap > 1e-4f * K && fabsf(gPz) > 1e-5f * Lf;
             if (good) {
                 const float sqH = sqrt32(H), kp = kap * gPz, sq = E * sqH, iD = rcp32(D);
                 const float zs = (kp >= 0.0f ? kp + sq : kp - sq) * iD, zo = (kp >= 0.0f ? kp - sq : kp + sq) * iD;
-                const float dQ = 1e-5f * (fabsf(kp) + sq + K * fabsf(gPz) + E * K * K * rcp32(sqH));
+                const float dQ = 1e-5f * (fabsf(kp) + sq + K * fabsf(gPz) + E * KK * rcp32(sqH));
                 const float base = 1e-5f * (Lf + fabsf(gPz));
                 const float m0 = (dQ + 1e-5f * K * fabsf(zs)) * iD + base, m1 = (dQ + 1e-5f * K * fabsf(zo)) * iD + base;
                 c0r = c0r && !(fabsf(zs) > Lf + m0) && !(fabsf(gPz - zs) > Lf + m0);

@@ -40,3 +40,35 @@ def test_bits(nx, np_, L, mask, mode, N, sampler, bits, stride, offset):
     got = A.cpu().numpy()
     assert np.array_equal(got, ref["A"].reshape(-1)) and np.count_nonzero(got) > 0
     assert np.array_equal(h.flags()[:2], ref["flags"])
+
+
+SCALES = [
+    # L, m^2 / L^2 of (g, u, d, s), mask
+    (1e-12, (0.3, 0.1, 0.1, 0.2), 0x13),
+    (1e-18, (0.0, 0.0, 0.0, 0.0), 0x13),
+    (1e-19, (0.3, 0.1, 0.1, 0.2), 0x13),    # p^2 leaves FP32's range
+    (1e-25, (0.3, 0.1, 0.1, 0.2), 0x01),
+    (4e9, (0.3, 0.1, 0.1, 0.2), 0x13),      # the square of p^2 does
+    (1e20, (1e-3, 1e-6, 0.0, 1e-2), 0x13),  # p^2 itself
+    (2.0, (1e3, 1e-30, 1e12, 1e20), 0x0F),  # masses far from L
+]
+
+
+@pytest.mark.parametrize("L,m2,mask", SCALES)
+def test_bits_at_any_scale(L, m2, mask):
+    """Momenta and masses far from 1 (other units than GeV): the FP32 classification
+    works in units of L and keeps what leaves FP32's range."""
+    import torch
+    from paper_1912_04457_gb300 import bz
+    np_, N, dt = (6, 5, 4), 2000, 0.05 / L
+    m2 = np.array([m2]) * L * L
+    h = bz.Handle(np_=np_, L=L, seed=8, species_mask=mask, mass_mode=bz.MASS_FIXED)
+    h.set_masses(m2)
+    cfg = O.make_config(np_=np_, L=L, seed=8, species_mask=mask, mass_mode=2)
+    st = I.encode(I.random_f(np_, bin(mask).count("1"), 1, 15, 0.0, 0.6), mask)
+    A = torch.empty(st.size, dtype=torch.int64, device="cuda")
+    h.collision_term(torch.from_numpy(st.reshape(-1)).cuda(), A, N, 2, dt, bz.PREC_F64)
+    ref = O.collision(cfg, st, m2, N, step=2, dt=dt)
+    got = A.cpu().numpy()
+    assert np.array_equal(got, ref["A"].reshape(-1)) and np.count_nonzero(got) > 0
+    assert np.array_equal(h.flags()[:2], ref["flags"])
