@@ -52,10 +52,11 @@ template <int SB64> struct Smem64 {
 
 __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
 constexpr unsigned long long SIGN64 = 0x8000000000000000ull;
-// v < 0, v >= 0, v <= 0 on the bit pattern (a NaN counts as neither; -0 is zero)
-__device__ __forceinline__ bool lt0(double v) { return dbits(v) > SIGN64; }
-__device__ __forceinline__ bool ge0(double v) { return dbits(v) <= SIGN64; }
-__device__ __forceinline__ bool le0(double v) { return dbits(v) >= SIGN64 || dbits(v) == 0ull; }
+constexpr unsigned long long INF64 = 0x7FF0000000000000ull;
+// v < 0, v >= 0, v <= 0 on the bit pattern (a NaN is neither; -0 is zero)
+__device__ __forceinline__ bool lt0(double v) { return dbits(v) - (SIGN64 + 1ull) < INF64; }
+__device__ __forceinline__ bool ge0(double v) { return dbits(v) <= INF64 || dbits(v) == SIGN64; }
+__device__ __forceinline__ bool le0(double v) { return dbits(v) - SIGN64 <= INF64 || dbits(v) == 0ull; }
 // -L <= v < L (L > 0)
 __device__ __forceinline__ bool in_box64(double v, double L)
 {
@@ -139,7 +140,10 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
         S.tmb[lane] = massless ? 0.0 : m2x[T.mslot[1]];
         S.tmc[lane] = massless ? 0.0 : m2x[T.mslot[2]];
         S.tsym[lane] = T.sym;
-        S.tmf[lane] = make_float4(trunc32(S.tma[lane], reb2), trunc32(S.tmb[lane], reb2), trunc32(S.tmc[lane], reb2), 0.0f);
+        // .w: 0, or infinite where a leg's m^2 is negative: no bound of the classification holds then
+        const bool neg = lt0(S.tma[lane]) || lt0(S.tmb[lane]) || lt0(S.tmc[lane]) || (!massless && lt0(m2x[T.mslot[3]]));
+        S.tmf[lane] = make_float4(trunc32(S.tma[lane], reb2), trunc32(S.tmb[lane], reb2), trunc32(S.tmc[lane], reb2),
+                                  neg ? __int_as_float(0x7F800000) : 0.0f);
         S.tinfo[lane] = T.slot[0] | (T.slot[1] << 3) | (T.slot[2] << 6) | (T.quark[0] << 9) | (T.quark[1] << 10)
                         | (T.quark[2] << 11) | (T.quark[3] << 12) | (T.cls << 13);
     }
@@ -403,13 +407,13 @@ __device__ __forceinline__ void collide64_row(const CollideArgs<double>& P, uint
             // K = E^2 + a^2 + b^2 every operation's error is below 1e-6 K (kappa, D),
             // 5e-6 K^2 (H); the margins are at least four times what follows from
             // that.  Roots that may be valid stay: NaNs and overflows count as "may" (K^2 is taken first:
-            // it overflows before the terms of H do).
+            // it overflows before the terms of H do), and so do all roots of a term whose K is made infinite.
             const float4 tmf = S.tmf[ti];
             const float ma2 = tmf.x, mb2 = tmf.y, mc2 = tmf.z;
             const float E3 = sqrt32(gkk3 + mc2);
             const float E = gEp + E3, EE = E * E;
             const float a2 = ga2 + ma2, b2 = gb2 + mb2;
-            const float K = EE + a2 + b2, KK = K * K, Pz2 = gPz * gPz;
+            const float K = (EE + a2) + (b2 + tmf.w), KK = K * K, Pz2 = gPz * gPz;
             const float D = EE - Pz2;
             const float kap = (EE + a2 - b2 - Pz2) * 0.5f;
             const float H = kap * kap - a2 * D;

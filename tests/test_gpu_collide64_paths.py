@@ -72,3 +72,26 @@ def test_bits_at_any_scale(L, m2, mask):
     got = A.cpu().numpy()
     assert np.array_equal(got, ref["A"].reshape(-1)) and np.count_nonzero(got) > 0
     assert np.array_equal(h.flags()[:2], ref["flags"])
+
+
+@pytest.mark.parametrize("mask,alpha,lo,hi", [(0x01, 0.3, -0.6, 0.1), (0x13, 0.3, -0.6, 0.1), (0x7F, 1.0, -0.6, 0.1),
+                                              (0x7F, 5.0, -0.2, 0.15)])
+def test_negative_mass_squared(mask, alpha, lo, hi):
+    """A state with negative cells can have m^2 < 0: E^2 and a^2 may be negative, energies NaN, and
+    kappa no longer tells which roots are valid.  Bit for bit the formula, its flags included."""
+    import torch
+    from paper_1912_04457_gb300 import bz
+    np_, N = (6, 5, 4), 400
+    h = bz.Handle(np_=np_, L=2.0, seed=8, species_mask=mask, alpha_s=alpha)
+    cfg = O.make_config(np_=np_, L=2.0, seed=8, species_mask=mask, alpha_s=alpha)
+    st = I.encode(I.random_f(np_, bin(mask).count("1"), 1, 15, lo, hi), mask)
+    m2 = O.masses(cfg, st)
+    assert m2[0, 0] < 0
+    dev = torch.from_numpy(st.reshape(-1)).cuda()
+    A = torch.empty(st.size, dtype=torch.int64, device="cuda")
+    h.collision_term(dev, A, N, 2, 0.01, bz.PREC_F64)
+    assert np.array_equal(h.get_masses(), m2)
+    ref = O.collision(cfg, st, m2, N, step=2, dt=0.01)
+    got = A.cpu().numpy()
+    assert np.array_equal(got, ref["A"].reshape(-1)) and np.count_nonzero(got) > 0
+    assert np.array_equal(h.flags()[:2], ref["flags"])
