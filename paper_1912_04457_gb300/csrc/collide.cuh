@@ -167,15 +167,17 @@ __device__ __forceinline__ R upow(R x, int n)
     return r;
 }
 
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // a / b: FP64 as written (the same bits by integer instructions); FP32 by the hardware reciprocal (the arguments are
 // far from its range limits), without the scaling of the approximate division.
 __device__ __forceinline__ double div_approx(double a, double b) { return div64(a, b); }
-__device__ __forceinline__ float div_approx(float a, float b)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
-    return a * r;
-}
+__device__ __forceinline__ float div_approx(float a, float b) { return a * rcp_approx(b); }
 
 template <typename R>
 __device__ __forceinline__ R msq_user(const UserRow* row, R s, R t, R u, R mg2)

@@ -54,3 +54,31 @@ def test_units(nx, np_, mask, N, stride, offset):
             assert torch.equal(A, B), sched
     finally:
         del os.environ["BZ_F32_SCHEDULE"]
+
+
+@pytest.mark.parametrize("mask,alpha,lo,hi", [(0x01, 0.3, -0.6, 0.1), (0x13, 0.3, -0.6, 0.1), (0x7F, 1.0, -0.6, 0.1),
+                                              (0x7F, 5.0, -0.2, 0.15)])
+@pytest.mark.parametrize("sampler", [0, 2])
+def test_negative_mass_squared(mask, alpha, lo, hi, sampler):
+    """A state with negative cells can have m^2 < 0, where kappa alone no longer tells which roots
+    are valid.  Most valid roots then have t or u above the regulator, and flag 0 counts
+    those: the oracle's number but for roots within FP32 rounding (some 1e-6 of t's terms) of
+    it, fewer than 1e-4 of them."""
+    import torch
+    from paper_1912_04457_gb300 import bz
+    np_, N, seed = (6, 5, 4), 400, 8
+    h = bz.Handle(np_=np_, L=2.0, seed=seed, species_mask=mask, alpha_s=alpha)
+    cfg = O.make_config(np_=np_, L=2.0, seed=seed, species_mask=mask, alpha_s=alpha)
+    st = I.encode(I.random_f(np_, bin(mask).count("1"), 1, 15, lo, hi), mask)
+    m2 = O.masses(cfg, st)
+    assert m2[0, 0] < 0
+    prop = None
+    if sampler == 2:
+        h.proposal_init(3)
+        h.proposal_infer()
+        prop = h.anchor_params().astype(np.float64)
+    A = torch.empty(st.size, dtype=torch.int64, device="cuda")
+    h.collision_term(torch.from_numpy(st.reshape(-1)).cuda(), A, N, 2, 0.01, bz.PREC_F32, sampler)
+    want = int(O.collision(cfg, st, m2, N, step=2, dt=0.01, ubits=23, sampler=sampler, prop=prop)["flags"][0])
+    assert want > 1000 and abs(int(h.flags()[0]) - want) <= 1e-4 * want
+    assert int(A.sum().item()) == 0
