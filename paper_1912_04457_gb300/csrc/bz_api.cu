@@ -2018,7 +2018,6 @@ extern "C" int bz_record(bz_handle h, const int64_t* state, int32_t nsamples, in
     CollideArgs<float> a{};
     fill_collide(h, a, nullptr, nsamples, step, dt, BZ_SAMPLER_SYMMETRIC);
     set_split(a, split);
-    a.tau = 0.0f;
     a.rec = static_cast<ProposalRecord*>(records);
     a.rec_count = cnt;
     a.rec_cap = max_records;

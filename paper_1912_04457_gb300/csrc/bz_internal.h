@@ -137,7 +137,7 @@ struct CollideArgs {
     int64_t ncell;          // cells of f and A (slots x nxc x npc)
     int np[3];
     R L, twoL, dp[3];
-    double L64, dp64[3];    // L and 2L/n in FP64 (the FP32 path's fixup works in FP64 geometry)
+    double L64, dp64[3];    // L and 2L/n in FP64 (the FP32 path's fixup takes them as float-float)
     // FP32 path index decode without hardware division (all indices < 2^31):
     // units per anchor (gpa), cells per slot, p cells, np[1] np[2], np[2]
     DivMagic dv_group, dv_slot, dv_npc, dv_yz, dv_z;
@@ -204,9 +204,9 @@ inline bool momentum_octets(Args& a)
 struct MassArgs {
     const long long* state;
     long long* acc;         // [x][4] fixed-point sums
-    // [x] blocks that have added theirs, or null.  With it acc and done are zero between
-    // launches: the x cell's last block takes the sums, writes the masses and clears acc;
-    // without it the launch clears acc first and a second kernel writes the masses.
+    // [x] blocks that have added theirs (launches with the table).  acc and done are zero between
+    // such launches: the x cell's last block takes the sums, writes the masses and clears acc.
+    // Without the table a launch clears acc first and a second kernel writes the masses.
     unsigned* done;
     double* m2_out;         // [x][4]
     const double* m2_prev;  // [x][4] or null (E = |p|)
@@ -308,8 +308,8 @@ cudaError_t launch_sum_ll(const long long* a, int64_t n, long long* out, cudaStr
 // resident grid (see collide_f32_resident_blocks), or null for a static stride
 cudaError_t launch_collide_f32(const CollideArgs<float>& a, int grid, unsigned long long* counter, cudaStream_t s);
 int collide_f32_resident_blocks(const CollideArgs<float>& a);  // per SM, for the instantiation `a` runs
-// FP32 path, uniform sampler: re-evaluation of the queued terms with an FP64
-// root solve (nseg queue segments)
+// FP32 path: re-evaluation of the queued terms in float-float arithmetic (nseg
+// queue segments)
 cudaError_t launch_fixup_f32(const CollideArgs<float>& a, int nseg, cudaStream_t s);
 cudaError_t launch_fixup_f32_batch(const CollideArgs<float>* boxes, const int* qcount, const unsigned long long* qitems,
                                    int64_t qcap, const int* step_dev, int nseg, cudaStream_t s);

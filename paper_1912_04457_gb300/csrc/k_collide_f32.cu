@@ -998,7 +998,6 @@ static int resident_blocks()
 int collide_f32_resident_blocks(const CollideArgs<float>& a)
 {
     const bool plain = is_plain(a);
-    if (a.rec_stride) return resident_blocks<M_RECORD, true, false>();
     if (a.sampler == SAMPLER_LEARNED)
         return plain ? resident_blocks<M_LEARNED, true, true>() : resident_blocks<M_LEARNED, true, false>();
     if (has_groups(a)) return plain ? resident_blocks<M_UNIFORM, true, true>() : resident_blocks<M_UNIFORM, true, false>();

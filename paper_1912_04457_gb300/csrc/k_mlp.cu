@@ -306,9 +306,6 @@ constexpr int INFER_THREADS = 256;  // two warps per lane quarter, 64 columns ea
 
 }  // namespace tc
 
-// One gradient evaluation over records [0, n): grad (FP32, NPARAM) += dL/dtheta
-// with L = -sum w log q / wsum, and loss_sum += L.  Each block walks chunks of
-// CH records and keeps its weight-gradient tiles in registers.
 // SplitMix64 output function (Steele, Lea and Flood, "Fast splittable
 // pseudorandom number generators", OOPSLA 2014): a bijective 64-bit mix.
 __device__ __forceinline__ uint64_t splitmix64(uint64_t x)
@@ -786,18 +783,17 @@ __global__ void __launch_bounds__(128) k_grad_reduce(const float* __restrict__ p
 
 // ---------------------------------------------------------------------------
 // Per-anchor inference on the 5th-generation tensor cores (tcgen05).  A CTA of
-// four warps takes tiles of 128 anchors: the activations of a tile (A, 128
-// rows) and the transposed weights (B) sit in shared memory in the
-// no-swizzle K-major layout of 8-row x 16-byte core matrices (element (r, k)
-// of an R x K operand at byte ((r/8)(K/8) + k/8) 128 + (r%8) 16 + (k%8) 2, so
-// core matrices adjacent along K are 128 bytes apart and along the rows
-// (K/8) 128 bytes); one thread issues tcgen05.mma (M = 128, K = 16 per
-// instruction, BF16 operands, FP32 accumulation in tensor memory) and
-// commits to an mbarrier; each warp then reads its 32 rows of the
-// accumulator (tcgen05.ld, lane quarter = warp) for the epilogue: bias, BF16
-// rounding of Z, SiLU in FP32, BF16 activation written back as the next
-// layer's A.  Every wait on the mbarrier is bounded: on a timeout the CTA
-// records it in err and stops issuing work, then releases its tensor memory.
+// eight warps takes tiles of 128 anchors.  The activations of a tile (A, 128
+// rows) are in shared memory K-major, the weights (B) in their [in][out]
+// orientation, which a descriptor reads MN-major: no-swizzle core matrices of 8
+// rows x 16 bytes, element (r, k) of an R x K buffer at op_off(r, k, K), as for
+// training.  One thread issues tcgen05.mma (M = 128, K = 16 per instruction,
+// BF16 operands, FP32 accumulation in tensor memory) and commits to an mbarrier;
+// two warps per lane quarter then read 64 columns each of their 32 rows of the
+// accumulator (tcgen05.ld) for the epilogue: bias, BF16 rounding of Z, SiLU in
+// FP32, BF16 activation written back as the next layer's A.  Every wait on the
+// mbarrier is bounded: on a timeout the CTA records it in err and stops
+// issuing work, then releases its tensor memory.
 // ---------------------------------------------------------------------------
 
 __global__ void __launch_bounds__(tc::INFER_THREADS) k_mlp_infer(const float* __restrict__ params, const ProposalArgs A,

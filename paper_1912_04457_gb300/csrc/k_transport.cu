@@ -379,7 +379,6 @@ __global__ void __launch_bounds__(MASS_THREADS, 4) k_masses_tab(const __grid_con
             red_add_ll(&P.acc[x * 4 + lane], t);
             __threadfence();
         }
-        if (!P.done) return;
         __syncwarp();
         unsigned before = lane == 0 ? atomicInc(P.done + x, (unsigned)nchunk - 1u) : 0u;  // wraps to 0
         before = __shfl_sync(0xffffffffu, before, 0);
@@ -444,11 +443,6 @@ cudaError_t launch_masses(const MassArgs& a, cudaStream_t s)
     b.chunk = chunk < 256 ? 256 : (chunk > MASS_CHUNK ? MASS_CHUNK : chunk);
     if (tab && per_x == 1) b.chunk = a.npc;
     const int64_t nchunk = (a.npc + b.chunk - 1) / b.chunk;
-    if (!tab) b.done = nullptr;
-    if (!tab || (nchunk > 1 && !b.done)) {
-        const cudaError_t e = cudaMemsetAsync(a.acc, 0, sizeof(long long) * 4 * a.nxc, s);
-        if (e != cudaSuccess) return e;
-    }
     if (tab) {
         bool gluon_only = a.slot_of[0] == 0;
         for (int q = 1; q < NSPEC; ++q) gluon_only = gluon_only && a.slot_of[q] < 0;
@@ -461,10 +455,11 @@ cudaError_t launch_masses(const MassArgs& a, cudaStream_t s)
             b.copy ? run(k_masses_tab<true, true>) : run(k_masses_tab<true, false>);
         else
             b.copy ? run(k_masses_tab<false, true>) : run(k_masses_tab<false, false>);
-        if (nchunk == 1 || b.done) return cudaGetLastError();
-    } else {
-        k_masses<<<(unsigned)(nchunk * a.nxc), 256, 0, s>>>(b);
+        return cudaGetLastError();
     }
+    const cudaError_t e = cudaMemsetAsync(a.acc, 0, sizeof(long long) * 4 * a.nxc, s);
+    if (e != cudaSuccess) return e;
+    k_masses<<<(unsigned)(nchunk * a.nxc), 256, 0, s>>>(b);
     k_masses_finish<<<(unsigned)((a.nxc + 127) / 128), 128, 0, s>>>(a);
     return cudaGetLastError();
 }
