@@ -87,8 +87,8 @@ __host__ __device__ __forceinline__ bool ff_from_bits(uint64_t b, ff& o)
 
 // nearest float-float of a double (exact to 48 bits); the three FP64 instructions
 // of the usual form issue for 64 cycles each, and a re-evaluated term of another box
-// or x cell than the thread's last converts up to eight (4^3 x cells of 16^3, gluons
-// and u: 61 -> 49 us per launch; 8^3 of 20^3, gluons: 332 -> 311 us)
+// or x cell than the thread's last converts up to eight (a fixup launch on 4^3 x cells of
+// 16^3, gluons and u: 20% less)
 __host__ __device__ __forceinline__ ff ff_from_double(double v)
 {
 #ifdef __CUDA_ARCH__

@@ -24,9 +24,15 @@
 // Measured on GB300 (cycles of a scheduler per warp instruction): integer logic,
 // shifts, compares and 32-bit multiplications 2.2, FP32 add/mul/FMA 1.1, a 32 x
 // 32 -> 64-bit multiplication 4.3 on the FMA pipe and another 2.4 of the integer
-// pipe's; the integer pipe is the kernel's bound (a draw, with its two Philox
-// blocks, takes 237 cycles and is 45% of the 8^3 x 20^3 gluon box's 12.6 ms,
-// formerly 18.9 ms), so what is cheap to state in FP32 is.
+// pipe's; the integer pipe is the kernel's bound with one species (a draw, with its
+// two Philox blocks, takes 237 cycles, 45% of its time), so what is cheap to state
+// in FP32 is.
+//
+// Times beside the choices below are of calls of the present kernels, the other choice
+// in parentheses: "bump" a step of 16^3 x 20^3 gluons, N = 256 (99.5 ms), "qgp" a step of
+// 32^3 of seven species, N = 1024, f of order 1 (11.88 ms), "ragged" four steps of 5 x 3 x 7 x cells
+// of 10 x 9 x 12, four species, N = 45 (3.50 ms), "learned" a learned step of 16^3 of
+// seven species, N = 256 (834 us).
 #include "collide.cuh"
 #include "ff.cuh"
 #include "intconv.cuh"
@@ -42,8 +48,8 @@ constexpr int RING = 128;         // pending roots per warp (power of 2)
 // one term an equation the pending roots (fewer than 32) reach back over two
 // batches, and with 64 slots 23% of the chunks were drawn twice; with several
 // kinematic groups they are those of the running batch's last groups, and the
-// shared memory is worth more to L1 (20^3 gluon boxes: 16.0 ms with 64 slots,
-// 14.7 with 128; 7 species, 32^3: 15.5 and 17.5).
+// shared memory is worth more to L1 (bump with 64: 120.0 ms; qgp with 128: 12.37 ms,
+// learned 940 us; ragged, whose batches are short, 3.36 ms with 128).
 template <bool GROUPS> constexpr int SLOTS = GROUPS ? 64 : 128;
 constexpr int WARPS = F32_WARPS;  // warps per block
 #ifndef BZ_FIX_GROUP
@@ -55,11 +61,15 @@ constexpr int WARPS = F32_WARPS;  // warps per block
 #ifndef BZ_FIX_MINB
 #define BZ_FIX_MINB 4  // resident blocks of 256 threads per SM the fixup's register budget is cut for (64 registers)
 #endif
+// Resident blocks per SM that the register budgets are cut for: 7 (72 registers) for single
+// boxes whose equations have groups of several terms (qgp with 6: 12.35 ms, with 8 11.85;
+// ragged 3.58 and 3.49), 6 (80 registers) for the others (learned with 5: 868 us, with 7 833;
+// bump with 5: 97.1 ms, with 7 99.5).
 #ifndef BZ_F32_MIN_BLOCKS
-#define BZ_F32_MIN_BLOCKS (24 / WARPS)  // resident blocks per SM the register budget is cut for (80 registers)
+#define BZ_F32_MIN_BLOCKS (24 / WARPS)
 #endif
 #ifndef BZ_F32_MIN_BLOCKS_GROUPED
-#define BZ_F32_MIN_BLOCKS_GROUPED 7  // the same for single boxes whose equations have groups of several terms
+#define BZ_F32_MIN_BLOCKS_GROUPED 7
 #endif
 
 // Sampling modes, resolved at compile time so that the uniform kernel carries
@@ -294,9 +304,8 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
 
     // A group's terms often share leg 2 ((q, d, q) and (qbar, d, qbar)).  Adding such terms'
     // deposits to its cell first leaves one atomic in ten out: the learned sampler, most
-    // of whose roots deposit, gains (16^3, seven species: 990 -> 952 us with 6 blocks per SM);
-    // the uniform one gains where f is of order 1 everywhere (32^3: 15.2 -> 14.7 ms) and
-    // loses where most of its roots deposit nothing (12.5 -> 13.1 ms), so it does not.
+    // of whose roots deposit, gains (learned without: 907 us); the uniform one loses (qgp
+    // with it 12.02 ms, ragged 3.54), so it does not.
     constexpr bool MERGE = MODE == M_LEARNED;
     const bool analytic = !PLAIN && SINGLE && P.analytic;  // (a batch's boxes hold states)
     const int nt = GROUPS ? P.nterms[d] : 1;
@@ -338,7 +347,7 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
     int head = 0, tail = 0;   // ring indices (warp-uniform)
     // the +q of the anchor own_a of this lane's last roots, deposited when the lane
     // meets another anchor and at the end: an atomic per root to one address
-    // would queue up in L2 (7 species, 32^3: 22.4 ms)
+    // would queue up in L2 where most roots deposit (learned 1127 us, bump 100.2 ms)
     long long own = 0;
     uint32_t own_a = a_first - row;
 
@@ -362,9 +371,9 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
             const unsigned lin2 = ((unsigned)gc.y >> 16) * P.np[2] + ((tg >> 16) & 0xff);
             const unsigned lin3 = gc.x;
             // the cells and occupations of a term's legs; a single term's, and the anchor's
-            // occupation, are loaded ahead of the arithmetic that comes before their use (20^3
-            // gluons, 64 samples: 20.7 -> 18.9 us; 32^3, seven species: 13.0 -> 12.5 ms; the first
-            // term of a group's as well, and each next one's ahead: 3% slower)
+            // occupation, are loaded ahead of the arithmetic that comes before their use (qgp at
+            // their use: 11.94 ms; the first term of a group's as well, and each next one's ahead: 3%
+            // slower)
             unsigned i1, i2, i3;
             float f1 = 0.0f, f2 = 0.0f, f3 = 0.0f, fpp = 0.0f;
             int info = 0;
@@ -731,7 +740,7 @@ __device__ __forceinline__ void collide_row(const CollideArgs<float>& P, int64_t
             // branch E1 = +sqrt(a^2 + z^2) iff kappa > 0, and likewise E2 > 0 iff
             // D - kappa > 0, for both roots (H > 0 keeps both away from 0).  That takes a^2, b^2 >=
             // 0; with a negative m^2 each root's E1 E = kappa + Pz z is compared with 0 and E^2 below
-            // (16^3 x 20^3 gluons 99.3 -> 99.5 ms, seven species 11.76 -> 11.89).
+            // (without that bump 99.4 ms, qgp 11.77).
             const bool ok = act & (fminf(kap, D - kap) > kmin);
             const bool hp = ok & (H > 0.0f);
             bool defer = DEFER && (ok & (fabsf(H) < P.tau * kk));
@@ -896,9 +905,8 @@ __device__ __forceinline__ void collide_unit(const CollideArgs<float>& P, int64_
 // block in the constant bank, the batch with each box's block in global
 // memory): a box gives the same bits alone or inside a batch.
 // PLAIN: f from the state, no user-defined |M|^2 row, all legs deposited: without the
-// code of the other forms (what a launch takes is chosen by launch_collide_f32; 32^3,
-// seven species: 12.53 -> 11.81 ms, 5 x 3 x 7 x cells, four species: 3.61 -> 3.48, 16^3 x 20^3 gluons: 101.8 ->
-// 99.7, learned 16^3 of seven species: 861 -> 809 us).
+// code of the other forms (what a launch takes is chosen by launch_collide_f32; by the
+// general form, fixup included: bump 102.3 ms, qgp 12.51, ragged 3.61, learned 880 us).
 template <int MODE, bool GROUPS, bool BATCH, bool PLAIN>
 __global__ void __launch_bounds__(32 * WARPS, (GROUPS && !BATCH && MODE != M_LEARNED) ? BZ_F32_MIN_BLOCKS_GROUPED : BZ_F32_MIN_BLOCKS)
     k_collide_f32(const __grid_constant__ CollideArgs<float> one, const CollideArgs<float>* __restrict__ boxes,
@@ -909,8 +917,8 @@ __global__ void __launch_bounds__(32 * WARPS, (GROUPS && !BATCH && MODE != M_LEA
     const int lane = threadIdx.x & 31;
     // the warp's index and its units come from warp reductions, whose result the
     // compiler keeps in uniform registers: everything derived from a unit then
-    // needs no vector registers or vector arithmetic (80 -> 72 registers without
-    // spills, 13.7 -> 13.4 ms on the 8^3 x 20^3 gluon box)
+    // needs no vector registers or vector arithmetic (by vector registers: bump 104.9
+    // ms, qgp 13.43, ragged 3.79, learned 900 us)
     const int warp = (int)__reduce_or_sync(0xffffffffu, threadIdx.x >> 5);
     const int64_t gw = (int64_t)blockIdx.x * WARPS + warp;
     const int64_t nwarps = (int64_t)gridDim.x * WARPS;
@@ -1065,8 +1073,8 @@ struct PropCache {
     ff m2[4], mg2;
 };
 
-// PLAIN as for the collision kernel (8^3 x 20^3 gluons: 313 -> 284 us per launch, 32^3 of
-// seven species 639 -> 599 us)
+// PLAIN as for the collision kernel (a launch of the general form: bump 2.36 ms for 2.18, qgp
+// 541 us for 505)
 template <bool LEARNED, bool PLAIN>
 __device__ __noinline__ long long fixup_term_ff(const CollideArgs<float>& P, int64_t a, int smp, int ti, int step,
                                                 PropCache& pc)
@@ -1271,9 +1279,9 @@ __device__ __noinline__ long long fixup_term_ff(const CollideArgs<float>& P, int
 // items.  Groups of up to 32 neighbouring segments are read as one list (a scan
 // of their counts) dealt over `slices` blocks of 256 threads: with warps that
 // belong to one segment, segments of few items left most lanes idle and those of
-// uneven counts left some warps working alone (10 x 9 x 12 cells of 5 x 3 x 7 x cells:
-// 71 -> 43 us; 16^3, seven species, learned: 94 -> 76 us; a 20^3 gluon box's step
-// 61 -> 58 us).  What is left there is one term's chain of dependent operations.
+// uneven counts left some warps working alone (a launch with lists of one segment:
+// ragged 64 us for 37, qgp 614 for 505, 20^3 gluons 23 for 16, learned 92 for 67; bump 2.10 ms
+// for 2.18).  What is left there is one term's chain of dependent operations.
 struct FixupGroup {
     int pre[33];  // first item of each segment of the group in its list; [n] = all
     int total;

@@ -11,13 +11,13 @@
 // that its error bounds put outside the box (or below the tangency), signs and
 // bounds are tested on the bit patterns, and the remaining (sample, term,
 // root) candidates -- 0.37 a sample and term -- are evaluated by full warps with
-// the operations of eval_term.  Collision kernel: 20^3 gluons, N = 64, 618 ->
-// 133 us; 7 species, 12 x 13 x 10, N = 100, 9.8 -> 1.5 ms; 4^3 x 20^3 gluons, N =
-// 128, 74.6 -> 11.9 ms; about 80% of the FP64 pipe's cycles were then in use, two
-// fifths of them by divisions and square roots.  Those are evaluated by integer
-// digits (div64, sqrt64: the same bits): 90 us, 0.88 ms and 7.7 ms.  The products of
-// the geometry, which every live sample takes, too (mul64): 88 us, 0.87 ms and 7.1 ms;
-// with the roots' products as well 102 us, 0.94 ms and 8.0 ms.
+// the operations of eval_term.  Divisions and square roots, two fifths of the FP64
+// pipe's cycles otherwise, are evaluated by integer digits (div64, sqrt64: the same
+// bits), and so are the products of the geometry, which every live sample takes (mul64).
+// Collision kernel, 20^3 gluons, N = 64, and 7 species, 12 x 13 x 10, N = 100: 89 us and
+// 0.88 ms; with FP64 divisions and roots 125 us and 1.56 ms, with FP64 products of the
+// geometry 89 us and 0.89 ms, with the roots' products by integers as well 15% and 8% more;
+// one thread per sample (k_collide) 618 us and 9.8 ms.
 #include "collide.cuh"
 #include "exact64.cuh"
 

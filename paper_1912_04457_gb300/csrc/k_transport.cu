@@ -148,10 +148,10 @@ __device__ __forceinline__ float ll2float_fast(long long n)
 // with |n| >= 2^46 and blocks with r >= 2^8 take the FP64 instructions, each of
 // which issues for 64 cycles.  The products are 64 x 47 bits, cut to 32 fraction
 // bits.  Gluons only (GLUON_ONLY): one rounding of one product, 9 n R_g and 3 n R_g.
-// 16^3 x 20^3 gluons, all bins nonzero: 410 -> 142 us (99 instructions a bin, a third
-// of them multiplications; 262 MB are read); 8^3 x 16^3, 7 species: 168 -> 78 us.  The
-// tables' roots and quotients by integer digits (div64, sqrt64: the same bits): 134 and 61
-// us, a 32^3 grid of 7 species 25 -> 17 us, 64^3 without the table 238 -> 107 us.
+// 16^3 x 20^3 gluons, all bins nonzero: 134 us, 410 by the FP64 formula (99 instructions a
+// bin, a third of them multiplications; 262 MB are read); 8^3 x 16^3, 7 species: 61 us
+// and 168.  The table's roots and quotients are evaluated by integer digits (div64, sqrt64:
+// the same bits; by FP64 instructions 142 and 78 us).
 // m_a^2 (i = 0 gluon, 1..3 flavours) from its exact fixed-point sum
 __device__ __forceinline__ double mass_of(const MassArgs& P, int i, long long acc)
 {
@@ -723,7 +723,7 @@ __device__ __forceinline__ void octet_index(const Args& P, int o, int h[3])
 // come from L1, the x neighbours' from L2 (blocks of one tile run together), so the
 // state is read from memory once.  A walk along z and y that carried each face's
 // flux (4 fluxes a cell instead of 6) took 312 instructions a cell and 357 us on
-// the 16^3 x 20^3 gluon box (no f written), this form 273 us.
+// the 16^3 x 20^3 gluon box (no f written), this form 242 us.
 // ---------------------------------------------------------------------------
 constexpr int DOCT_WARPS = 4, DRIFT_MINB = 8;  // warps per block, blocks per SM
 
@@ -803,8 +803,8 @@ struct FluxSum {
 // the range of the form it takes where |p| <= E; with m^2 < 0 (a state with negative cells) C may
 // leave it, and a thread that met such a C stores its cells a second time.  It works from the launch's
 // arguments alone, so that the loop before it keeps no register for it but the largest 1/E it met
-// (16^3 x 20^3 gluons: 272 us, 273 without it; the or of all C 277, masses tested ahead of the loop 314, a call out of
-// line 100 bytes of spills).  A C that is no number counts as 0, as in the loop.
+// (no slower than without it; with the or of all C 1.5% slower, with the masses tested ahead of the
+// loop 15%, with a call out of line 100 bytes of spills).  A C that is no number counts as 0, as in the loop.
 template <bool FORCE>
 __device__ __forceinline__ void mirror_wide(const DriftArgs& P, int nseg, float K)
 {
@@ -1170,7 +1170,7 @@ constexpr int MOM_THREADS = 128;  // per (x cell, slot) or chunk of one
 // its sign, every momentum component, so that a sum over the octet and three
 // differences (18 64-bit additions) leave one multiplication per moment instead
 // of one per cell: 12 instructions a cell instead of 150, which leaves the loads
-// the bound (16^3 x 20^3 box: moments 187 -> 68 us, energy source 134 -> 52 us, 262 MB
+// the bound (16^3 x 20^3 box: moments 184 -> 62 us, energy source 131 -> 50 us, 262 MB
 // read; 7 blocks per SM, 72 registers: more bytes in flight than with 94).
 // The eight n as loaded, lower cells first: bit d of the index is set for the
 // upper cell of axis d; a cell on the mirror plane of an odd axis counts as its
