@@ -30,9 +30,9 @@
 //
 // Times beside the choices below are of calls of the present kernels, the other choice
 // in parentheses: "bump" a step of 16^3 x 20^3 gluons, N = 256 (99.5 ms), "qgp" a step of
-// 32^3 of seven species, N = 1024, f of order 1 (11.88 ms), "ragged" four steps of 5 x 3 x 7 x cells
-// of 10 x 9 x 12, four species, N = 45 (3.50 ms), "learned" a learned step of 16^3 of
-// seven species, N = 256 (834 us).
+// 32^3 of seven species, N = 1024 (11.88 ms), "ragged" four steps of 5 x 3 x 7 x cells of
+// 10 x 9 x 12, four species, N = 45 (3.50 ms), "learned" a learned step of 16^3 of seven
+// species, N = 256 (834 us), on the states of perf/cases.py.
 #include "collide.cuh"
 #include "ff.cuh"
 #include "intconv.cuh"
