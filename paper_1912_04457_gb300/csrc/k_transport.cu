@@ -148,7 +148,7 @@ __device__ __forceinline__ float ll2float_fast(long long n)
 // with |n| >= 2^46 and blocks with r >= 2^8 take the FP64 instructions, each of
 // which issues for 64 cycles.  The products are 64 x 47 bits, cut to 32 fraction
 // bits.  Gluons only (GLUON_ONLY): one rounding of one product, 9 n R_g and 3 n R_g.
-// 16^3 x 20^3 gluons, all bins nonzero: 134 us, 410 by the FP64 formula (99 instructions a
+// 16^3 x 20^3 gluons, all bins nonzero: 134 us, 410 by the FP64 formula (103 instructions a
 // bin, a third of them multiplications; 262 MB are read); 8^3 x 16^3, 7 species: 61 us
 // and 168.  The table's roots and quotients are evaluated by integer digits (div64, sqrt64:
 // the same bits; by FP64 instructions 142 and 78 us).
@@ -1037,7 +1037,7 @@ cudaError_t launch_drift(const DriftArgs& a, cudaStream_t s)
     const int64_t nslots = rows / a.nxc;
     // |C| <= 2^30 dt/dx < 2^31 (m^2 >= 0; else checked by the kernels), mirrored cells: by octets; else (long time steps, cell
     // centres that are no exact mirror images in FP32) by rows.  16^3 x 20^3 gluons, without f: 242 us, by rows 440
-    // (some 205 instructions a cell, multiplications and addresses the largest parts)
+    // (some 218 instructions a cell, multiplications and addresses the largest parts)
     if (moving && a.dtdxf < 1.99f && a.noct > 0) {
         const int64_t tiles_m = ((int64_t)a.half[0] * a.half[1] * a.np[2] + 31) / 32, base = nslots * a.nx[0] * tiles_m;
         // y segments of equal length: 40 blocks per SM (five waves, so that the last one matters little: 16^3 x
@@ -1169,7 +1169,7 @@ constexpr int MOM_THREADS = 128;  // per (x cell, slot) or chunk of one
 // Octets of mirrored cells.  The 8 cells (+-p_x, +-p_y, +-p_z) share E and, up to
 // its sign, every momentum component, so that a sum over the octet and three
 // differences (18 64-bit additions) leave one multiplication per moment instead
-// of one per cell: 12 instructions a cell instead of 150, which leaves the loads
+// of one per cell: 45 instructions a cell instead of 150, which leaves the loads
 // the bound (16^3 x 20^3 box: moments 184 -> 62 us, energy source 131 -> 50 us, 262 MB
 // read; 7 blocks per SM, 72 registers: more bytes in flight than with 94).
 // The eight n as loaded, lower cells first: bit d of the index is set for the
