@@ -59,7 +59,7 @@ h.collision_term(torch.from_numpy(st.reshape(-1)).cuda(), A2, 32, 3, 0.01, bz.PR
 del os.environ["BZ_F32_SCHEDULE"]
 out["f32_counter_equal"] = bool(torch.equal(A, A2))
 
-# streaming drift with the force term on an inhomogeneous grid, several species
+# drift by mirrored cells with the force term on an inhomogeneous grid, several species
 nx, np_, mask = (3, 2, 4), (4, 6, 4), 0x03
 nxc = 24
 h = bz.Handle(nx=nx, dx=0.2, np_=np_, L=2.0, seed=1, species_mask=mask, alpha_s=0.3, mass_mode=2)
@@ -74,9 +74,9 @@ h.drift(torch.from_numpy(st.reshape(-1)).cuda(), dst, 0.05)
 ref = O.drift(cfg, st, m2, 0.05).reshape(-1)
 out["drift_equal"] = bool(np.array_equal(dst.cpu().numpy(), ref))
 
-# the row kernel (n_z above the streaming kernel's buffer), with the force term
-nx, np_, mask = (2, 2, 41), (4, 4, 4), 0x01
-nxc = 164
+# the row kernel (z cells that the mirrored form's warps would share unevenly), with the force term
+nx, np_, mask = (2, 3, 5), (4, 4, 4), 0x01
+nxc = 30
 h = bz.Handle(nx=nx, dx=0.2, np_=np_, L=2.0, seed=1, species_mask=mask, alpha_s=0.3, mass_mode=2)
 cfg = O.make_config(nx=nx, dx=0.2, np_=np_, L=2.0, seed=1, species_mask=mask, alpha_s=0.3, mass_mode=2)
 cfg.force = 1
